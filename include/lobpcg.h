@@ -465,6 +465,11 @@ LOBPCG_API lobpcg_status lobpcg_row_norms(int64_t n, const int64_t* row_ptr, con
 LOBPCG_API lobpcg_status lobpcg_gram_f64_noalloc(int64_t n, int p, const double* X, int ldx, int q,
                                                  const double* Y, int ldy, double* C, lobpcg_stream stream);
 
+/* Give back the workspace that the building-block entry points keep between calls: at most
+ * 256 MB of device memory per device (a stream-ordered pool) and 8 small pinned host areas.
+ * Calls in flight on other threads keep theirs. */
+LOBPCG_API lobpcg_status lobpcg_trim_workspace(void);
+
 /* ------------------------------------------------------------------------------
  * Measurement.  The paper has no counterpart: this measures the part the solver runs on.
  * ------------------------------------------------------------------------------ */

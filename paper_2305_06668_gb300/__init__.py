@@ -79,7 +79,7 @@ def lib():
                      "lobpcg_spmm_csr_f32", "lobpcg_syev2_f64", "lobpcg_gram_f32", "lobpcg_update_f32",
                      "lobpcg_probe_fma_rate", "lobpcg_gram_f64_df", "lobpcg_update_f64_df",
                      "lobpcg_spmm_csr_f64_df", "lobpcg_gram_f32_tcgen05", "lobpcg_precond_tridiag",
-                     "lobpcg_mixed_switch_replay"):
+                     "lobpcg_mixed_switch_replay", "lobpcg_trim_workspace"):
             getattr(L, name).restype = C.c_int
         L.lobpcg_last_error.restype = C.c_char_p
         L.lobpcg_last_error.argtypes = [C.c_void_p]
@@ -486,6 +486,11 @@ def ortho_against(X, Y, tau=1e-14, cap=6, cap2=4, stream=None):
                                           _ptr(Y), C.c_int(Y.stride(0) if q else 1), C.c_double(tau), C.c_int(cap),
                                           C.c_int(cap2), st, _stream(stream)))
     return X, dict(passes=st[0], cholqr_passes_max=st[1], shifts=st[2], svqb=st[3], cap_hits=st[4])
+
+
+def trim_workspace():
+    """Give back the workspace the building blocks keep between calls (lobpcg_trim_workspace)."""
+    _check(lib().lobpcg_trim_workspace())
 
 
 def upload_csr(a, device="cuda"):
