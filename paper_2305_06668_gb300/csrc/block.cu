@@ -50,8 +50,10 @@ __device__ __forceinline__ void stage_rows(const Cols<T>& c, int64_t r0, int64_t
 template <class T, int TI, int TJ, int R>
 __global__ void __launch_bounds__(512) gram_kernel(int64_t n, Cols<T> A, Cols<T> B, int upper,
                                                    int ntiles, int groups,
-                                                   double* __restrict__ part, int64_t rows_per_cta) {
+                                                   double* __restrict__ part, int64_t rows_per_cta,
+                                                   const int* __restrict__ run_flag) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (run_flag && *run_flag == 0) return;
   __shared__ short tile_i[kMaxS * kMaxS / 16], tile_j[kMaxS * kMaxS / 16];
   const int pa = A.width(), pb = B.width();
   const int nti = (pa + TI - 1) / TI, ntj = (pb + TJ - 1) / TJ;
@@ -602,7 +604,7 @@ int count_tiles(int pa, int pb, int TI, int TJ, bool upper) {
 
 template <class T, int TI, int TJ, int R>
 int gram_launch(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, double* part,
-                int max_ctas, cudaStream_t st) {
+                int max_ctas, cudaStream_t st, const int* run_flag) {
   const int pa = a.width(), pb = b.width();
   const int pa_pad = round_up(pa, TI), pb_pad = round_up(pb, TJ);
   const int ntiles = count_tiles(pa, pb, TI, TJ, upper);
@@ -622,8 +624,9 @@ int gram_launch(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, doubl
   int64_t ctas = std::min<int64_t>(max_ctas, ceil_div(n, R));
   if (ctas < 1) ctas = 1;
   const int64_t rpc = (ceil_div(n, ctas) + R - 1) / R * R;
-  ctas = std::max<int64_t>(1, ceil_div(n, rpc));
-  gram_kernel<T, TI, TJ, R><<<(unsigned)ctas, threads, smem, st>>>(n, a, b, upper ? 1 : 0, ntiles, groups, part, rpc);
+  ctas = run_flag ? max_ctas : std::max<int64_t>(1, ceil_div(n, rpc));
+  gram_kernel<T, TI, TJ, R><<<(unsigned)ctas, threads, smem, st>>>(n, a, b, upper ? 1 : 0, ntiles, groups, part, rpc,
+                                                                   run_flag);
   LB_LAUNCH_CHECK();
   return (int)ctas;
 }
@@ -632,13 +635,13 @@ int gram_launch(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, doubl
 
 template <class T>
 int gram_partials(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, double* part,
-                  int max_ctas, cudaStream_t st) {
+                  int max_ctas, cudaStream_t st, const int* run_flag) {
   const int pa = a.width(), pb = b.width();
   if (pa > kMaxS || pb > kMaxS) throw std::invalid_argument("gram: width > 96");
-  if (const int parts = gram_partials_pipe<T>(n, a, b, upper, part, max_ctas, st)) return parts;
+  if (const int parts = gram_partials_pipe<T>(n, a, b, upper, part, max_ctas, st, run_flag)) return parts;
   if (count_tiles(pa, pb, 4, 4, upper) <= 512)
-    return gram_launch<T, 4, 4, 32>(n, a, b, upper, part, max_ctas, st);
-  return gram_launch<T, 8, 8, 32>(n, a, b, upper, part, max_ctas, st);
+    return gram_launch<T, 4, 4, 32>(n, a, b, upper, part, max_ctas, st, run_flag);
+  return gram_launch<T, 8, 8, 32>(n, a, b, upper, part, max_ctas, st, run_flag);
 }
 
 void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st) {
@@ -787,8 +790,10 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
   LB_LAUNCH_CHECK();
 }
 
-template int gram_partials<double>(int64_t, const Cols<double>&, const Cols<double>&, bool, double*, int, cudaStream_t);
-template int gram_partials<float>(int64_t, const Cols<float>&, const Cols<float>&, bool, double*, int, cudaStream_t);
+template int gram_partials<double>(int64_t, const Cols<double>&, const Cols<double>&, bool, double*, int, cudaStream_t,
+                                   const int*);
+template int gram_partials<float>(int64_t, const Cols<float>&, const Cols<float>&, bool, double*, int, cudaStream_t,
+                                   const int*);
 template int launch_update<double>(int64_t, const UpdateJob<double>&, const double*, int, int, double, const double*, double*, int, cudaStream_t);
 template int launch_update<float>(int64_t, const UpdateJob<float>&, const double*, int, int, double, const double*, double*, int, cudaStream_t);
 template void launch_precond<double>(int64_t, const double*, const double*, int, const double*, int, int, const double*, int, double*, int, cudaStream_t, const double*, double);

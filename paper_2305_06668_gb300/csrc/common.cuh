@@ -133,14 +133,16 @@ void launch_spmm_dense(int64_t n, const T* A, int64_t lda, int p, const T* X, in
 
 // Gram partials: part[g][i + j*pa] = sum over CTA g's rows of a_ri * b_rj.
 // upper: only i <= j entries are produced.  Returns the number of CTAs used.
+// run_flag (device, may be null): the kernel returns without writing unless *run_flag is not zero;
+// the launch then has exactly max_ctas CTAs (those past the rows write zeros).
 template <class T>
 int gram_partials(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, double* part,
-                  int max_ctas, cudaStream_t st);
+                  int max_ctas, cudaStream_t st, const int* run_flag = nullptr);
 // Pipelined variants (tiles.cu) for operands sharing one 16-byte aligned row stride;
 // return 0 without launching when they do not apply.
 template <class T>
 int gram_partials_pipe(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, double* part, int max_ctas,
-                       cudaStream_t st);
+                       cudaStream_t st, const int* run_flag = nullptr);
 template <class T>
 struct UpdateJob;
 template <class T>
@@ -153,6 +155,14 @@ int launch_update_pipe(int64_t n, const UpdateJob<T>& job, const double* U, int 
 int gram_partials_umma(int64_t n, const Cols<float>& a, const Cols<float>& b, bool upper, double* part,
                        int max_ctas, cudaStream_t st);
 void umma_check(cudaStream_t st);
+// FP64 Gram partials through exact digit products on the tensor cores (gram64.cu).  Returns the
+// number of CTAs, or 0 without launching where the blocks do not fit.  scratch:
+// gram64_scratch_ints(n) ints.  *scratch is the flag left at 1 when some column is outside the
+// digits' range: the partials are then to be formed by gram_partials with run_flag = scratch.
+size_t gram64_scratch_ints(int64_t n);
+int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
+                         int max_ctas, int* scratch, cudaStream_t st);
+void gram64_check(cudaStream_t st);
 // out[e] = sum_g part[g][e] for e < count (FP64, fixed order).
 void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st);
 

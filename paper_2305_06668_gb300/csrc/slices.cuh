@@ -1,0 +1,105 @@
+// FP64 numbers as sums of 8-bit digits for exact products on the tensor cores (the scheme of
+// Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast
+// routines of matrix multiplication", 2012).
+//
+// The numbers of one group (a column over 256 rows, or a row) share a power of two 2^e above
+// their largest magnitude.  x becomes the whole number X = x 2^(55-e), |X| < 2^55, rounded to
+// nearest (exact for every x within a factor of 4 of the group's binade), and X seven balanced
+// digits, X = sum_k d_k 256^(6-k), -128 <= d_k <= 128.  A digit is exact in FP16, a product of two
+// digits is a whole number of at most 2^14, and a sum of up to 2^10 such products is exact in the
+// tensor core's FP32 accumulator, whatever the order.  Products with i + j <= 7 are kept: what is
+// left out is below 2^-58 of the groups' largest product per term.
+#pragma once
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace lobpcg {
+namespace slices {
+
+constexpr int kSlices = 7;
+constexpr int kDiags = 8;  // accumulators: i + j = 0 .. 7
+// Groups whose biased exponent lies outside [kExpMin, kExpMax] (infinities and NaN among them)
+// take the general kernels; all-zero groups use kExpOne.
+constexpr int kExpMin = 1023 - 400, kExpMax = 1023 + 400, kExpOne = 1023;
+
+// |x|'s high word for a maximum over a group; a subnormal with an empty high word counts as 1.
+__device__ __forceinline__ uint32_t exp_key(double x) {
+  const uint32_t hw = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  return max(hw, (uint32_t)__double2loint(x) != 0u ? 1u : 0u);
+}
+// Biased exponent E of a group from the maximum of its keys (2^(E-1023) <= max < 2^(E-1022)), or
+// -1 when the group is outside the range of the digits.
+__device__ __forceinline__ int group_exp(uint32_t key) {
+  if (key == 0u) return kExpOne;
+  const int e = (int)(key >> 20);
+  return e < kExpMin || e > kExpMax ? -1 : e;
+}
+
+// X + 0x0080808080808080 with 0x64 in the top byte: byte 6-k of the result is d_k + 128
+// (a leading digit of 128 carries into the top byte).
+__device__ __forceinline__ uint64_t digits(double x, int E) {
+  const uint32_t hw = (uint32_t)__double2hiint(x), lw = (uint32_t)__double2loint(x);
+  const int e = (int)((hw >> 20) & 0x7ffu);
+  const int k = min(E - e, 63);  // >= 0; zeros and subnormals shift out (E >= kExpMin)
+  const uint64_t m = (uint64_t)((hw & 0xfffffu) | 0x100000u) << 32 | lw;
+  const uint64_t t = (((m << 3) >> k) + 1u) >> 1;
+  const uint64_t neg = (uint64_t)(int64_t)((int32_t)hw >> 31);
+  return (t ^ neg) + (0x6480808080808080ull - neg);
+}
+
+// The digits k of two numbers (a in the low half) as FP16.
+template <int K>
+__device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
+  constexpr uint32_t kByte = (uint32_t)(6 - K);
+  uint32_t r;
+  if constexpr (K == 0) {
+    // bytes 7 and 6 are 0x64 (0x65 where the leading digit is 128) and the digit: 1024 + d_0 + 128
+    r = __byte_perm((uint32_t)(a >> 32), (uint32_t)(b >> 32), 0x7632u);
+  } else {
+    constexpr uint32_t i = kByte & 3u;
+    constexpr int kShift = kByte >= 4 ? 32 : 0;
+    r = __byte_perm((uint32_t)(a >> kShift), (uint32_t)(b >> kShift), i | i << 4 | (4u + i) << 8 | (4u + i) << 12);
+    r = (r & 0x00ff00ffu) | 0x64006400u;
+  }
+  // (1024 + byte) - 1152 = byte - 128, exact
+  __half2 h = *reinterpret_cast<__half2*>(&r);
+  h = __hsub2(h, __half2half2(__ushort_as_half(0x6480)));
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// sum_t v_t 256^(7-t) of eight whole FP32 numbers |v_t| <= 2^24, times 2^s, rounded to FP64 with
+// integer operations only (an FP64 instruction takes 64 times the issue slots of an integer one).
+__device__ __forceinline__ double join(const float (&v)[kDiags], int s) {
+  int64_t hi = (int64_t)__float2int_rn(v[0]) * (1 << 24) + (int64_t)__float2int_rn(v[1]) * (1 << 16) +
+               (int64_t)__float2int_rn(v[2]) * (1 << 8) + (int64_t)__float2int_rn(v[3]);
+  const int64_t lo = (int64_t)__float2int_rn(v[4]) * (1 << 24) + (int64_t)__float2int_rn(v[5]) * (1 << 16) +
+                     (int64_t)__float2int_rn(v[6]) * (1 << 8) + (int64_t)__float2int_rn(v[7]);
+  hi += lo >> 32;
+  uint32_t l = (uint32_t)lo;  // value = hi 2^32 + l
+  const uint32_t sign = (uint32_t)(hi >> 63);
+  if (sign) {
+    hi = ~hi + (l == 0u ? 1 : 0);
+    l = 0u - l;
+  }
+  uint64_t h = (uint64_t)hi;
+  int top = 95;  // exponent of bit 63 of h
+  if ((h >> 32) == 0u) {
+    h = h << 32 | l;
+    l = 0u;
+    top = 63;
+    if (h == 0u) return 0.0;
+  }
+  const int n = __clzll((long long)h);
+  // the high word of h is not zero unless the value is below 2^32, where l is empty
+  uint64_t m = h << n;
+  if (n < 32) m |= n ? l >> (32 - n) : 0u;
+  else m |= (uint64_t)l << (n - 32);
+  m = (m >> 11) + ((m >> 10) & 1u);
+  return __longlong_as_double((long long)(((uint64_t)(sign & 1u) << 63) +
+                                          ((uint64_t)(1022 + top - n + s) << 52) + m));
+}
+
+}  // namespace slices
+}  // namespace lobpcg

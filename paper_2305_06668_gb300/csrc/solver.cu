@@ -391,6 +391,16 @@ struct lobpcg_ctx {
   DevBuf xbest;        // the FP32 phase's X with the smallest largest-sought residual (reading R22)
   DevBuf tri_offd;     // tridiagonal preconditioner: dl then du of A (n - 1 doubles each)
   DevBuf tri_scratch;  // its FP32 scratch (tridiag_scratch_floats(n, a))
+  DevBuf gram_buf;         // exponents of the digit Grams (allocated when first used)
+  int* gram_ints = nullptr;
+  bool used_digits = false;  // a digit Gram was launched: its give-up flag is checked at the end
+  int* gram_scratch() {
+    if (!gram_ints) {
+      gram_buf.ensure(gram64_scratch_ints(A.n) * sizeof(int));
+      gram_ints = gram_buf.as<int>();
+    }
+    return gram_ints;
+  }
   double* host = nullptr;  // pinned readback area
   Stats stats;
   Profiler prof;
@@ -417,6 +427,12 @@ struct lobpcg_ctx {
   bool trace_orth = false;  // LOBPCG_TRACE_ORTH=1: also trace max |V^T V - I|
 
   void sync() { LB_CUDA(cudaStreamSynchronize(st)); }
+  // the end of a call: waits for its work and reports a tensor-core kernel that gave up waiting
+  void finish() {
+    if (used_digits) gram64_check(st);
+    else sync();
+    used_digits = false;
+  }
 
   size_t small_bytes() const {
     const size_t gpart = (size_t)max_ctas * kMaxS * kMaxS;
@@ -565,12 +581,27 @@ void apply_A(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
   c.prof.mark(PH_OTHER);
 }
 
+// Multiply-adds of a Gram from which the digit products win over FP64 FMAs and over double-float.
+constexpr double kDigitGram = 2e7, kDigitGramDf = 6e7;
+
 template <class T>
 void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double* out) {
   const int pa = a.width(), pb = b.width();
   int parts = 0;
   if constexpr (std::is_same<T, double>::value) {
-    if (c.df_on) parts = gram_partials_df(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
+    // digit products on the tensor cores from the size where they are the faster form; a column
+    // outside the digits' range raises their flag, and the FMA kernel behind them (else an empty
+    // launch) forms the partials
+    const double mults = (double)c.A.n * pa * pb * (upper ? 0.5 : 1.0);
+    if (mults >= (c.df_on ? kDigitGramDf : kDigitGram)) {
+      int* flag = c.gram_scratch();
+      parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.st);
+      if (parts) {
+        c.used_digits = true;
+        gram_partials<T>(c.A.n, a, b, upper, c.Gpart, parts, c.st, flag);
+      }
+    }
+    if (!parts && c.df_on) parts = gram_partials_df(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
   } else {
     // FP32: the tcgen05 kernel when the blocks fit it (every block the solver allocates);
     // its give-up flag is checked once per solve (umma_check)
@@ -1433,7 +1464,7 @@ extern "C" lobpcg_status lobpcg_solve(lobpcg_ctx* c, int k, double tol, const do
     LB_CUDA(cudaMemcpyAsync(evals, c->lam, k * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     LB_CUDA(cudaMemcpyAsync(resnorms, c->resnorm, k * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     LB_CUDA(cudaEventRecord(e1, c->st));
-    c->sync();
+    c->finish();
     if (c->opt.precision == LOBPCG_MIXED) umma_check(c->st);
     float ms = 0.f;
     LB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
@@ -1498,6 +1529,7 @@ extern "C" void lobpcg_destroy(lobpcg_ctx* c) {
   c->xbest.release();
   c->tri_offd.release();
   c->tri_scratch.release();
+  c->gram_buf.release();
   c->mlp_params.release();
   c->rho.release();
   if (c->host) cudaFreeHost(c->host);
@@ -1524,8 +1556,10 @@ struct ScratchCtx {
     LB_CUDA(cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev));
     c.max_ctas = 2 * c.sms;
     lobpcg_options_default(&c.opt);
-    mem.alloc(c.small_bytes());
+    const size_t small = (c.small_bytes() + 255) / 256 * 256;
+    mem.alloc(small + gram64_scratch_ints(n) * sizeof(int));
     c.lay_out_small(mem.as<double>());
+    c.gram_ints = reinterpret_cast<int*>(mem.as<char>() + small);
     c.host = pinned_take();
   }
   ~ScratchCtx() {
@@ -1659,7 +1693,7 @@ extern "C" lobpcg_status lobpcg_gram_f64(int64_t n, int p, const double* X, int 
             "lobpcg_gram_f64: need 1 <= p, q <= 96, ld >= width");
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
     gram<double>(s.c, cols1<double>(X, ldx, p), cols1<double>(Y, ldy, q), false, C);
-    s.c.sync();
+    s.c.finish();
     return LOBPCG_OK;
   });
 }
@@ -1676,7 +1710,7 @@ extern "C" lobpcg_status lobpcg_gram_f64_df(int64_t n, int p, const double* X, i
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
     s.c.df_on = true;
     gram<double>(s.c, cols1<double>(X, ldx, p), cols1<double>(Y, ldy, q), false, C);
-    s.c.sync();
+    s.c.finish();
     return LOBPCG_OK;
   });
 }
@@ -1826,7 +1860,7 @@ extern "C" lobpcg_status lobpcg_ortho_f64(int64_t n, int p, double* X, int ldx, 
     require(tau > 0 && cap >= 1, "lobpcg_ortho_f64: tau > 0 and cap >= 1 required");
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
     const int passes = ortho<double>(s.c, X, ldx, p, tau, cap);
-    s.c.sync();
+    s.c.finish();
     if (stats) {
       stats[0] = passes;
       stats[1] = s.c.stats.shifts;
@@ -1847,7 +1881,7 @@ extern "C" lobpcg_status lobpcg_ortho_against_f64(int64_t n, int p, double* X, i
     require(tau > 0 && cap >= 1 && cap2 >= 1, "lobpcg_ortho_against_f64: tau > 0 and caps >= 1 required");
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
     const int passes = ortho_against<double>(s.c, X, ldx, p, cols1<double>(Y, ldy, q), tau, cap, cap2);
-    s.c.sync();
+    s.c.finish();
     if (stats) {
       stats[0] = passes;
       stats[1] = s.c.stats.cholqr_passes_max;
@@ -1916,6 +1950,8 @@ extern "C" lobpcg_status lobpcg_solve_batched(lobpcg_ctx* const* ctxs, int nprob
       ctxs[i]->b32.buf.release();
       ctxs[i]->x0buf.release();
       ctxs[i]->xbest.release();
+      ctxs[i]->gram_buf.release();
+      ctxs[i]->gram_ints = nullptr;
     }
   };
   std::vector<std::thread> pool;

@@ -71,8 +71,9 @@ __device__ __forceinline__ int col_offset(const Cols<T>& c, int col, int R, int 
 template <class T, int TI, int TJ, int R, int S>
 __global__ void __launch_bounds__(256) gram_pipe_kernel(int64_t n, Cols<T> A, Cols<T> B, int ld, int upper,
                                                         int ntiles, int groups, double* __restrict__ part,
-                                                        int64_t rows_per_cta) {
+                                                        int64_t rows_per_cta, const int* __restrict__ run_flag) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (run_flag && *run_flag == 0) return;
   const int lds = padded_ld<T>(ld);
   const int stageA = A.nseg * R * lds, stageB = B.nseg * R * lds;
   const int stage = stageA + stageB;
@@ -1003,7 +1004,7 @@ bool aligned(const Cols<T>& c, int ld) {
 
 template <class T, int TI, int TJ, int R, int S>
 int gram_pipe_launch(int64_t n, const Cols<T>& a, const Cols<T>& b, int ld, bool upper, double* part,
-                     int max_ctas, cudaStream_t st) {
+                     int max_ctas, cudaStream_t st, const int* run_flag) {
   const int pa = a.width(), pb = b.width();
   const int ntiles = count_tiles(pa, pb, TI, TJ, upper);
   const int threads = 256;
@@ -1022,9 +1023,9 @@ int gram_pipe_launch(int64_t n, const Cols<T>& a, const Cols<T>& b, int ld, bool
   int64_t ctas = std::min<int64_t>(max_ctas, ceil_div(n, R));
   if (ctas < 1) ctas = 1;
   const int64_t rpc = (ceil_div(n, ctas) + R - 1) / R * R;
-  ctas = std::max<int64_t>(1, ceil_div(n, rpc));
+  ctas = run_flag ? max_ctas : std::max<int64_t>(1, ceil_div(n, rpc));
   gram_pipe_kernel<T, TI, TJ, R, S><<<(unsigned)ctas, threads, smem, st>>>(n, a, b, ld, upper ? 1 : 0, ntiles,
-                                                                          groups, part, rpc);
+                                                                          groups, part, rpc, run_flag);
   LB_LAUNCH_CHECK();
   return (int)ctas;
 }
@@ -1079,7 +1080,7 @@ int gram_partials_df(int64_t n, const Cols<double>& a, const Cols<double>& b, bo
 // one aligned row stride, so the caller can use the general kernel instead.
 template <class T>
 int gram_partials_pipe(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, double* part, int max_ctas,
-                       cudaStream_t st) {
+                       cudaStream_t st, const int* run_flag) {
   if (a.nseg == 0 || b.nseg == 0) return 0;
   const int ld = a.ld[0];
   if (!aligned(a, ld) || !aligned(b, ld)) return 0;
@@ -1099,15 +1100,15 @@ int gram_partials_pipe(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper
   if (sizeof(T) == 4 && pa >= 16 && pb >= 16 && count_tiles(pa, pb, 8, 8, upper) <= 256) {
     // long stages: enough rows per thread group between barriers
     const size_t stage128 = (size_t)(a.nseg + b.nseg) * 128 * padded_ld<T>(ld) * sizeof(T);
-    if (stage128 * 2 <= 190 * 1024) return gram_pipe_launch<T, 8, 8, 128, 2>(n, a, b, ld, upper, part, max_ctas, st);
-    return gram_pipe_launch<T, 8, 8, 32, 3>(n, a, b, ld, upper, part, max_ctas, st);
+    if (stage128 * 2 <= 190 * 1024) return gram_pipe_launch<T, 8, 8, 128, 2>(n, a, b, ld, upper, part, max_ctas, st, run_flag);
+    return gram_pipe_launch<T, 8, 8, 32, 3>(n, a, b, ld, upper, part, max_ctas, st, run_flag);
   }
   // FP64: 2 x 4 tiles (more threads on the FP64 units) when they fit the CTA, e.g. the
   // Grams of Algorithms 2 and 3; measured ~4% faster there than 4 x 4
   if (sizeof(T) == 8 && count_tiles(pa, pb, 2, 4, upper) <= 256)
-    return gram_pipe_launch<T, 2, 4, 32, 2>(n, a, b, ld, upper, part, max_ctas, st);
+    return gram_pipe_launch<T, 2, 4, 32, 2>(n, a, b, ld, upper, part, max_ctas, st, run_flag);
   if (count_tiles(pa, pb, 4, 4, upper) <= 256)
-    return gram_pipe_launch<T, 4, 4, 32, 2>(n, a, b, ld, upper, part, max_ctas, st);
+    return gram_pipe_launch<T, 4, 4, 32, 2>(n, a, b, ld, upper, part, max_ctas, st, run_flag);
   return 0;
 }
 
@@ -1164,9 +1165,9 @@ int launch_update_pipe(int64_t n, const UpdateJob<T>& job, const double* U, int 
 }
 
 template int gram_partials_pipe<double>(int64_t, const Cols<double>&, const Cols<double>&, bool, double*, int,
-                                        cudaStream_t);
+                                        cudaStream_t, const int*);
 template int gram_partials_pipe<float>(int64_t, const Cols<float>&, const Cols<float>&, bool, double*, int,
-                                       cudaStream_t);
+                                       cudaStream_t, const int*);
 template int launch_update_pipe<double>(int64_t, const UpdateJob<double>&, const double*, int, int, double,
                                         const double*, double*, int, cudaStream_t);
 template int launch_update_pipe<float>(int64_t, const UpdateJob<float>&, const double*, int, int, double,
