@@ -195,6 +195,11 @@ int gram_partials_df(int64_t n, const Cols<double>& a, const Cols<double>& b, bo
                      int max_ctas, cudaStream_t st);
 int launch_update_df(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
                      const double* lam, double* norm_part, int max_ctas, cudaStream_t st);
+// The FP64 update through exact digit products on the tensor cores (update64.cu); unit_base is
+// not needed there and ignored.  Returns 0 without launching where the blocks do not fit.
+int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
+                         const double* lam, double* norm_part, int max_ctas, cudaStream_t st);
+void update64_check(cudaStream_t st);
 // dst[i] = (hi, lo) split of src[i] (the double-float operands: matrix values, blocks).
 void launch_split_df(int64_t count, const double* src, float2* dst, cudaStream_t st);
 // Y = A X (FP64 result) from the split values vs (nnz) and the split block Xs (n x ldx

@@ -70,35 +70,28 @@ __device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
 }
 
 // sum_t v_t 256^(7-t) of eight whole FP32 numbers |v_t| <= 2^24, times 2^s, rounded to FP64 with
-// integer operations only (an FP64 instruction takes 64 times the issue slots of an integer one).
+// integer operations only (an FP64 instruction takes 64 times the issue slots of an integer one) and
+// without branches, so that the joins of several elements overlap.
 __device__ __forceinline__ double join(const float (&v)[kDiags], int s) {
-  int64_t hi = (int64_t)__float2int_rn(v[0]) * (1 << 24) + (int64_t)__float2int_rn(v[1]) * (1 << 16) +
-               (int64_t)__float2int_rn(v[2]) * (1 << 8) + (int64_t)__float2int_rn(v[3]);
-  const int64_t lo = (int64_t)__float2int_rn(v[4]) * (1 << 24) + (int64_t)__float2int_rn(v[5]) * (1 << 16) +
-                     (int64_t)__float2int_rn(v[6]) * (1 << 8) + (int64_t)__float2int_rn(v[7]);
-  hi += lo >> 32;
-  uint32_t l = (uint32_t)lo;  // value = hi 2^32 + l
-  const uint32_t sign = (uint32_t)(hi >> 63);
-  if (sign) {
-    hi = ~hi + (l == 0u ? 1 : 0);
-    l = 0u - l;
-  }
-  uint64_t h = (uint64_t)hi;
-  int top = 95;  // exponent of bit 63 of h
-  if ((h >> 32) == 0u) {
-    h = h << 32 | l;
-    l = 0u;
-    top = 63;
-    if (h == 0u) return 0.0;
-  }
-  const int n = __clzll((long long)h);
-  // the high word of h is not zero unless the value is below 2^32, where l is empty
-  uint64_t m = h << n;
-  if (n < 32) m |= n ? l >> (32 - n) : 0u;
-  else m |= (uint64_t)l << (n - 32);
-  m = (m >> 11) + ((m >> 10) & 1u);
-  return __longlong_as_double((long long)(((uint64_t)(sign & 1u) << 63) +
-                                          ((uint64_t)(1022 + top - n + s) << 52) + m));
+  auto i = [&](int t) { return __float2int_rn(v[t]); };
+  int64_t hi = (int64_t)i(0) * (1 << 24) + ((int64_t)i(1) * (1 << 16) + ((int64_t)i(2) * (1 << 8) + i(3)));
+  const int64_t lo = (int64_t)i(4) * (1 << 24) + ((int64_t)i(5) * (1 << 16) + ((int64_t)i(6) * (1 << 8) + i(7)));
+  hi += lo >> 32;  // the sum is hi 2^32 + (low word of lo)
+  const uint32_t neg = (uint32_t)(hi >> 63);
+  // magnitude in three words: complement, plus one where negative
+  uint32_t w0 = (uint32_t)lo ^ neg;
+  uint64_t h = (uint64_t)hi ^ ((uint64_t)neg << 32 | neg);
+  w0 -= neg;
+  h += (neg & 1u) & (w0 == 0u ? 1u : 0u);
+  uint32_t w2 = (uint32_t)(h >> 32), w1 = (uint32_t)h;
+  int e = 1022 + 95 + s;  // biased exponent of the top bit of w2, less one for the implicit bit
+  if (w2 == 0u) w2 = w1, w1 = w0, w0 = 0u, e -= 32;
+  if (w2 == 0u) w2 = w1, w1 = w0, w0 = 0u, e -= 32;
+  const int n = __clz((int)w2);
+  const uint32_t m1 = __funnelshift_l(w1, w2, n), m0 = __funnelshift_l(w0, w1, n);
+  const uint64_t m = (uint64_t)m1 << 32 | m0;
+  const uint64_t bits = ((uint64_t)((uint32_t)(e - n) + (neg << 11)) << 52) + (m >> 11) + ((m0 >> 10) & 1u);
+  return __longlong_as_double(w2 ? (long long)bits : 0ll);
 }
 
 }  // namespace slices

@@ -393,7 +393,7 @@ struct lobpcg_ctx {
   DevBuf tri_scratch;  // its FP32 scratch (tridiag_scratch_floats(n, a))
   DevBuf gram_buf;         // exponents of the digit Grams (allocated when first used)
   int* gram_ints = nullptr;
-  bool used_digits = false;  // a digit Gram was launched: its give-up flag is checked at the end
+  bool used_digits = false, used_update64 = false;  // launched: the give-up flags are checked at the end
   int* gram_scratch() {
     if (!gram_ints) {
       gram_buf.ensure(gram64_scratch_ints(A.n) * sizeof(int));
@@ -430,8 +430,9 @@ struct lobpcg_ctx {
   // the end of a call: waits for its work and reports a tensor-core kernel that gave up waiting
   void finish() {
     if (used_digits) gram64_check(st);
-    else sync();
-    used_digits = false;
+    if (used_update64) update64_check(st);
+    if (!used_digits && !used_update64) sync();
+    used_digits = used_update64 = false;
   }
 
   size_t small_bytes() const {
@@ -488,6 +489,10 @@ struct Prec<float> {
   static int64_t lda(lobpcg_ctx& c) { return c.A.n; }
 };
 
+// Multiply-adds from which the digit products win over FP64 FMAs and over double-float.
+constexpr double kDigitGram = 2e7, kDigitGramDf = 6e7;
+constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7;
+
 // launch_update with, in profile mode, the FP64 launches timed and their flops counted.
 template <class T>
 int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q, double alpha, const double* lam,
@@ -496,6 +501,13 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   if (timed) c.prof.kmark();
   int parts;
   if constexpr (std::is_same<T, double>::value) {
+    // digit products on the tensor cores from the size where they are the faster form
+    parts = 0;
+    if ((double)c.A.n * s * q * job.nprod >= (c.df_on ? kDigitUpdateDf : kDigitUpdate)) {
+      parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
+      c.used_update64 |= parts > 0;
+    }
+    if (!parts)
     parts = c.df_on ? launch_update_df(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st)
                     : launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
   } else {
@@ -580,9 +592,6 @@ void apply_A(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
   if (sizeof(T) == 8) c.stats.spmm_launches64 += 1, c.stats.spmm_columns64 += p;
   c.prof.mark(PH_OTHER);
 }
-
-// Multiply-adds of a Gram from which the digit products win over FP64 FMAs and over double-float.
-constexpr double kDigitGram = 2e7, kDigitGramDf = 6e7;
 
 template <class T>
 void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double* out) {
@@ -1749,7 +1758,7 @@ extern "C" lobpcg_status lobpcg_update_f64_df(int64_t n, int nseg, const double*
       reduce_partials(sc.c.npart, parts, 2 * q, sc.c.G, sc.c.st);
       LB_CUDA(cudaMemcpyAsync(sc.c.host, sc.c.G, (size_t)q * sizeof(double), cudaMemcpyDeviceToHost, sc.c.st));
     }
-    sc.c.sync();
+    sc.c.finish();
     if (resnorm)
       for (int j = 0; j < q; ++j) resnorm[j] = std::sqrt(sc.c.host[j]);
     return LOBPCG_OK;

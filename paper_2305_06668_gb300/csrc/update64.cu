@@ -1,0 +1,501 @@
+// FP64 block updates out_t = base_t + alpha in_t U (X = V u_x with AX = AV u_x and the residual
+// norms, P = V u_p, W - Y C, W L^{-T}) on the 5th-generation tensor cores: the rows of in_t and the
+// columns of U are cut into FP16 digits (slices.cuh) whose products the tensor core sums exactly.
+//
+// What bounds it.  As FP64 FMAs (2 per clock and SM) the pair X, AX of 10^6 rows, 63 columns to 21,
+// takes 5 ms, in double-float on the FP32 pipes 2.4 ms; its bytes take 0.2 ms and its digit products
+// 0.12 ms of tensor time.  What is left to pay is the cutting into digits and the joining of the sums.
+//
+// Scaling.  Column l of V and row l of U are scaled against each other by the power of two above
+// max_j |alpha U_lj|, so an entry of a row counts by the most it contributes to any output; then every
+// row of V has one exponent and every column of U one.  A row's entries are held to 2^-56 of its
+// largest contribution, digit sums are exact, each product is rounded to FP64 once and the base is
+// added in FP64.
+//
+// One persistent CTA per SM takes a contiguous range of 128-row tiles:
+//   * warps 0..15, splitters: warp w owns rows 8 w .. 8 w + 7 of the tile.  Its lane 0 copies them
+//     (1-D TMA bulk copies, one per segment) into the warp's own raw slot, the next tile's as soon
+//     as this tile's are in registers.  A lane holds 8 columns of one row per 32-column chunk; the
+//     row's exponent comes from two shuffles; a chunk's digits go to a tile buffer as K-major core
+//     matrices, 128 bytes per quarter warp without bank conflicts.
+//   * warp 24, one thread: the MMA issuer.  Digit i of V against digits j, j + 1, .. of U writes TMEM
+//     columns 32 (i + j), ..: region t of an accumulator sums the products with i + j = t, at most
+//     7 * 96 * 2^14 < 2^24, exact.
+//   * warps 16..23, epilogue: two threads per row, which take the groups of four columns in turn.  The
+//     eight regions of an element are joined into FP64 with integer operations, the base is added, and
+//     the residuals of the four columns are handed through shared memory to one warp per column, which
+//     keeps their squares' sum and maximum.
+// Rows with an infinity, a NaN or an exponent outside 2^+-400 (and all rows when U has one) are
+// formed by their epilogue thread with FP64 FMAs.
+#include <algorithm>
+#include <climits>
+#include <type_traits>
+
+#include "common.cuh"
+#include "slices.cuh"
+#include "umma.cuh"
+
+namespace lobpcg {
+namespace {
+
+using namespace umma;
+using namespace slices;
+
+constexpr int kTile = 128;      // rows per tile
+constexpr int kQ = 32;          // output columns, padded
+constexpr int kKC = 32;         // columns of V per chunk
+constexpr int kMaxTS = 2;       // chunk buffers: two where shared memory holds them, else one
+constexpr int kRing = 8;        // row-exponent ring (a splitter is at most 4 products ahead)
+constexpr int kSplitWarps = 16, kEpi0 = 16, kEpiWarps = 8, kMma = 24;
+constexpr int kThreads = 32 * 25;
+constexpr uint32_t kLBO = 128, kSBO = kKC / 8 * 128;
+constexpr uint32_t kSlice = kTile / 8 * kSBO;  // bytes of one digit of a chunk of V
+constexpr uint32_t kBuf = kSlices * kSlice;
+constexpr int kAcc = kDiags * kQ;              // TMEM columns of one accumulator
+constexpr int kBad = INT_MIN;
+constexpr long long kWaitCycles = 1ll << 31;
+constexpr size_t kStatic = 14 * 1024;  // static shared memory, at most
+constexpr size_t kSmemBudget = 227 * 1024;
+
+__device__ int g_update64_err = 0;
+
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int code) {
+  const long long t0 = clock64();
+  for (uint32_t i = 0;; ++i) {
+    if (mbar_try(bar, parity)) return true;
+    if ((i & 15u) == 15u) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > kWaitCycles) break;
+    }
+  }
+  *abort_flag = 1;
+  atomicExch(&g_update64_err, code);
+  return false;
+}
+
+// bytes of U's digits: kSlices slices of kQ columns x KP rows
+__host__ __device__ constexpr uint32_t u_slice(int kp) { return (uint32_t)(kQ * kp * 2); }
+
+// NC: 32-column chunks of V (ceil(s / 32)).
+template <int NC, bool NORM>
+__global__ void __launch_bounds__(kThreads, 1)
+    update64_kernel(int64_t n, UpdateJob<double> job, const double* __restrict__ U, int s, int q, double alpha,
+                    const double* __restrict__ lam, double* __restrict__ norm_part, int64_t tiles_per_cta,
+                    int ts) {
+  constexpr int KP = NC * kKC;
+  constexpr uint32_t kSliceU = u_slice(KP), kSBOU = KP / 8 * 128;
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ uint64_t raw_full[kSplitWarps], tile_full[kMaxTS], tile_empty[kMaxTS], acc_full[2], acc_empty[2], exp_full[kRing];
+  __shared__ int row_exp[kRing][kTile];
+  __shared__ int col_exp[kQ];
+  __shared__ __align__(16) int16_t up[KP];  // exponent of row l of U: V's column l is scaled by 2^up
+  __shared__ double res[2][NORM ? 4 : 1][NORM ? kTile : 1];
+  __shared__ double lam_s[kQ];
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
+  __shared__ int u_bad;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nseg = job.in[0].nseg, nprod = job.nprod;
+  int raw_row = 0;  // doubles of one row of all segments
+  for (int g = 0; g < nseg; ++g) raw_row += job.in[0].ld[g];
+  unsigned char* tiles = smem;                                            // [ts][kBuf]
+  unsigned char* udig = smem + (uint32_t)ts * kBuf;                       // [kSlices][kSliceU]
+  double* raw = reinterpret_cast<double*>(udig + kSlices * kSliceU);      // [kSplitWarps][segment][8][ld]
+
+  if (tid == 0) {
+    abort_flag = 0, u_bad = 0;
+    for (int i = 0; i < kSplitWarps; ++i) mbar_init(&raw_full[i], 1);
+    for (int i = 0; i < kMaxTS; ++i) mbar_init(&tile_full[i], kSplitWarps), mbar_init(&tile_empty[i], 1);
+    for (int i = 0; i < 2; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], kEpiWarps);
+    for (int i = 0; i < kRing; ++i) mbar_init(&exp_full[i], kSplitWarps);
+    fence_barrier_init();
+  }
+  for (uint32_t e = tid; e < kSlices * kSliceU / 16; e += kThreads) reinterpret_cast<uint4*>(udig)[e] = make_uint4(0, 0, 0, 0);
+  // alpha U, staged in the first tile buffer (s x q column-major, at most 24 KB of its 56)
+  double* us = reinterpret_cast<double*>(tiles);
+  for (int e = tid; e < s * q; e += kThreads) us[e] = alpha * U[e];
+  __syncthreads();
+  for (int l = tid; l < KP; l += kThreads) {
+    uint32_t key = 0u;
+    if (l < s)
+      for (int j = 0; j < q; ++j) key = max(key, exp_key(us[l + j * s]));
+    const int e = group_exp(key);
+    if (e < 0) u_bad = 1;
+    up[l] = key ? (int16_t)(e - 1022) : (int16_t)-4000;  // a zero row of U: no contribution
+  }
+  __syncthreads();
+  // U's entry (l, j) scaled by 2^-up: below 1 in magnitude; exponent of a column over its scaled entries
+  for (int j = tid; j < kQ; j += kThreads) {
+    if (NORM) lam_s[j] = j < q ? lam[j] : 0.0;
+    int E = 0;
+    bool any = false;
+    if (j < q)
+      for (int l = 0; l < s; ++l) {
+        const uint32_t key = exp_key(us[l + j * s]);
+        any |= key != 0u;
+        if (key >> 20) E = max(E, (int)(key >> 20) - up[l]);
+      }
+    if (any && E < kExpMin) u_bad = 1;  // a column of numbers far below their rows'
+    col_exp[j] = any ? E : kExpOne;
+  }
+  __syncthreads();
+  for (int e = tid; e < s * q; e += kThreads) {
+    const int l = e % s, j = e / s;
+    // digits() takes the exponent in the entry's own scale; entries far below their column shift out
+    const uint64_t w = up[l] > -4000 ? digits(us[e], col_exp[j] + up[l]) : digits(0.0, kExpOne);
+    unsigned char* o = udig + (uint32_t)(j >> 3) * kSBOU + (uint32_t)(l >> 3) * kLBO + 16u * (j & 7) + 2u * (l & 7);
+    auto put = [&](auto k) {
+      constexpr int K = decltype(k)::value;
+      *reinterpret_cast<uint16_t*>(o + K * kSliceU) = (uint16_t)digit_pair<K>(w, w);
+    };
+    put(std::integral_constant<int, 0>{}), put(std::integral_constant<int, 1>{});
+    put(std::integral_constant<int, 2>{}), put(std::integral_constant<int, 3>{});
+    put(std::integral_constant<int, 4>{}), put(std::integral_constant<int, 5>{});
+    put(std::integral_constant<int, 6>{});
+  }
+  __syncwarp();
+  if (warp == kMma) tmem_alloc(&tmem_slot, 2 * kAcc);
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const bool all_bad = u_bad != 0;
+
+  const int64_t t_begin = (int64_t)blockIdx.x * tiles_per_cta;
+  const int64_t r_begin = t_begin * kTile, r_end = min(n, r_begin + tiles_per_cta * kTile);
+  const int ntiles = r_end > r_begin ? (int)((r_end - r_begin + kTile - 1) / kTile) : 0;
+  const int nT = ntiles * nprod;  // tile-products, in the order tile, product
+  int copied = 0, committed = 0;  // splitter lane 0 / MMA thread
+
+  if (warp < kSplitWarps) {
+    const int r = lane & 7, k8 = lane >> 3;  // row within the warp's eight; group of 8 columns within a chunk
+    double* slot = raw + (size_t)warp * 8 * raw_row;
+    auto copy = [&](int T) {
+      const Cols<double>& c = job.in[T % nprod];
+      const int64_t r0 = r_begin + (int64_t)(T / nprod) * kTile + 8 * warp;
+      const int rows = (int)min((int64_t)8, r_end - r0);
+      if (rows <= 0) {  // no row of this warp in the last tile
+        mbar_arrive(&raw_full[warp]);
+        return;
+      }
+      uint32_t total = 0;  // a segment's last row is copied up to its used columns
+      for (int g = 0; g < nseg; ++g) total += (uint32_t)((rows - 1) * c.ld[g] + (c.w[g] + 1) / 2 * 2) * 8u;
+      mbar_expect_tx(&raw_full[warp], total);
+      double* d = slot;
+      for (int g = 0; g < nseg; ++g) {
+        bulk_g2s(d, c.p[g] + r0 * c.ld[g], (uint32_t)((rows - 1) * c.ld[g] + (c.w[g] + 1) / 2 * 2) * 8u, &raw_full[warp]);
+        d += 8 * c.ld[g];
+      }
+    };
+    // column l of row r in the slot: base_g + l with the segment's base
+    const int w0 = job.in[0].w[0], w1 = nseg > 1 ? w0 + job.in[0].w[1] : INT_MAX;
+    const int b0 = r * job.in[0].ld[0];
+    const int b1 = nseg > 1 ? 8 * job.in[0].ld[0] + r * job.in[0].ld[1] - w0 : 0;
+    const int b2 = nseg > 2 ? 8 * (job.in[0].ld[0] + job.in[0].ld[1]) + r * job.in[0].ld[2] - w1 : 0;
+    if (lane == 0 && nT > 0) copy(0), copied = 1;
+    int buf = 0;
+    uint32_t tph = 1;  // parity of the tile_empty phase to wait for (the first ts chunks do not wait)
+    int chunk = 0;
+    for (int T = 0; T < nT; ++T) {
+      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[warp], (uint32_t)T & 1u, &abort_flag, 1))) break;
+      const bool live = r_begin + (int64_t)(T / nprod) * kTile + 8 * warp + r < r_end;
+      double x[NC][8];
+      int E = 0;
+      bool bad = false;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const int4 u4 = *reinterpret_cast<const int4*>(&up[c * kKC + 8 * k8]);
+        const int us4[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int l = c * kKC + 8 * k8 + i;
+          x[c][i] = live && l < s ? slot[(l < w0 ? b0 : l < w1 ? b1 : b2) + l] : 0.0;
+          const int e = (__double2hiint(x[c][i]) >> 20) & 0x7ff;
+          const int v = i & 1 ? us4[i >> 1] >> 16 : (int)(int16_t)us4[i >> 1];
+          bad |= e == 0x7ff;
+          if (e > 0) E = max(E, e + v);
+        }
+      }
+      __syncwarp();  // the warp's slot is in registers: refill it
+      if (lane == 0 && T + 1 < nT) copy(T + 1), copied = T + 2;
+      E = max(E, __shfl_xor_sync(0xffffffffu, E, 8));
+      E = max(E, __shfl_xor_sync(0xffffffffu, E, 16));
+      const uint32_t badm = __ballot_sync(0xffffffffu, bad);
+      bad = (badm & (0x01010101u << r)) != 0u || (E > 0 && (E < kExpMin || E > kExpMax));
+      if (__any_sync(0xffffffffu, E <= 0)) {  // no contribution of normal size: a row of zeros, or too small
+        bool some = false;
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) some |= up[c * kKC + 8 * k8 + i] > -4000 && x[c][i] != 0.0;
+        const uint32_t somem = __ballot_sync(0xffffffffu, some);
+        bad |= E <= 0 && (somem & (0x01010101u << r)) != 0u;
+      }
+      if (E <= 0 || bad) E = kExpOne;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (chunk >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph, &abort_flag, 2))) break;
+        if (c == 0) {
+          if (lane < 8) row_exp[T & (kRing - 1)][8 * warp + lane] = bad ? kBad : E;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&exp_full[T & (kRing - 1)]);
+        }
+        const int4 u4 = *reinterpret_cast<const int4*>(&up[c * kKC + 8 * k8]);
+        const int us4[4] = {u4.x, u4.y, u4.z, u4.w};
+        uint64_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int v = i & 1 ? us4[i >> 1] >> 16 : (int)(int16_t)us4[i >> 1];
+          // the row's exponent in the entry's own scale; a bad row's digits are not used
+          w[i] = digits(bad ? 0.0 : x[c][i], v > -4000 ? E - v : 4 * kExpOne);
+        }
+        unsigned char* o = tiles + (uint32_t)buf * kBuf + (uint32_t)warp * kSBO + (uint32_t)k8 * kLBO + 16u * r;
+        auto put = [&](auto k) {
+          constexpr int K = decltype(k)::value;
+          *reinterpret_cast<uint4*>(o + K * kSlice) =
+              make_uint4(digit_pair<K>(w[0], w[1]), digit_pair<K>(w[2], w[3]), digit_pair<K>(w[4], w[5]),
+                         digit_pair<K>(w[6], w[7]));
+        };
+        put(std::integral_constant<int, 0>{}), put(std::integral_constant<int, 1>{});
+        put(std::integral_constant<int, 2>{}), put(std::integral_constant<int, 3>{});
+        put(std::integral_constant<int, 4>{}), put(std::integral_constant<int, 5>{});
+        put(std::integral_constant<int, 6>{});
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tile_full[buf]);
+        ++chunk;
+        if (++buf == ts) buf = 0, tph ^= 1u;
+      }
+    }
+  } else if (warp == kMma) {
+    if (lane == 0) {
+      const uint64_t dA = desc_kmajor(smem_addr(tiles), kLBO, kSBO);
+      const uint64_t dB = desc_kmajor(smem_addr(udig), kLBO, kSBOU);
+      const int ksteps = (s + 15) / 16;
+      int buf = 0;
+      uint32_t tph = 0, aph = 0;
+      bool ok = true;
+      for (int T = 0; T < nT && ok; ++T) {
+        const int a = T & 1;
+        if (T >= 2 && !wait_bar(&acc_empty[a], aph ^ 1u, &abort_flag, 3)) break;
+        const uint32_t d = tmem + (uint32_t)(a * kAcc);
+        for (int c = 0; c < NC; ++c) {
+          if (!wait_bar(&tile_full[buf], tph, &abort_flag, 3)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t bo = dA + (uint64_t)((uint32_t)buf * kBuf >> 4);
+          for (int kk = 0; kk < kKC / 16 && 2 * c + kk < ksteps; ++kk) {
+            const uint32_t acc = c > 0 || kk > 0 ? 1u : 0u;
+            const uint64_t ka = bo + (uint64_t)(kk * 16), kb = dB + (uint64_t)((2 * c + kk) * 16);
+            auto mma = [&](int i, int j, int cnt, uint32_t ac) {
+              mma_f16(d + (uint32_t)(kQ * (i + j)), ka + (uint64_t)(i * (kSlice >> 4)),
+                      kb + (uint64_t)(j * (kSliceU >> 4)), idesc_f16(kTile, (uint32_t)(kQ * cnt)), ac);
+            };
+            mma(0, 0, 7, acc);  // regions 0..6
+            mma(1, 0, 6, 1u);
+            mma(1, 6, 1, acc);  // region 7, overwriting what an earlier product left
+#pragma unroll
+            for (int i = 2; i < kSlices; ++i) mma(i, 0, kDiags - i, 1u);
+          }
+          mma_commit(&tile_empty[buf]);
+          if (++buf == ts) buf = 0, tph ^= 1u;
+        }
+        if (ok) {
+          mma_commit(&acc_full[a]);
+          committed = T + 1;
+          if (a == 1) aph ^= 1u;
+        }
+      }
+    }
+  } else {
+    const int quad = warp & 3, half = (warp - kEpi0) >> 2, row = 32 * quad + lane;
+    double nsum[kQ / 8], nmax[kQ / 8];
+#pragma unroll
+    for (int g = 0; g < kQ / 8; ++g) nsum[g] = 0.0, nmax[g] = 0.0;
+    bool ok = true;
+    for (int it = 0; it < ntiles && ok; ++it) {
+      const int64_t grow = r_begin + (int64_t)it * kTile + row;
+      const bool live = grow < r_end;
+      int er[2] = {kExpOne, kExpOne};
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (t >= nprod) break;
+        const int T = it * nprod + t;
+        ok = ok && __all_sync(0xffffffffu, wait_bar(&exp_full[T & (kRing - 1)], (uint32_t)(T / kRing) & 1u, &abort_flag, 2));
+        ok = ok && __all_sync(0xffffffffu, wait_bar(&acc_full[T & 1], (uint32_t)(T / 2) & 1u, &abort_flag, 2));
+        if (ok) er[t] = all_bad ? kBad : row_exp[T & (kRing - 1)][row];
+      }
+      if (!ok) break;
+      tc_fence_after();
+      // rows outside the digits' range: FP64 FMAs from global memory, all of the row before any store
+      double slow[2][kQ];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (t >= nprod || !live || er[t] != kBad) continue;
+        for (int j = 0; j < q; ++j) slow[t][j] = 0.0;
+        int l = 0;
+        for (int g = 0; g < nseg; ++g)
+          for (int i = 0; i < job.in[t].w[g]; ++i, ++l) {
+            const double v = job.in[t].p[g][grow * job.in[t].ld[g] + i];
+            for (int j = 0; j < q; ++j) slow[t][j] = fma(v, alpha * U[l + j * s], slow[t][j]);
+          }
+      }
+      // both threads of a row have read it before either stores
+      if (__any_sync(0xffffffffu, er[0] == kBad || er[1] == kBad)) asm volatile("bar.sync %0, 64;\n" ::"r"(5 + quad) : "memory");
+#pragma unroll
+      for (int gh = 0; gh < kQ / 8; ++gh) {
+        const int g = 2 * gh + half;
+        if (4 * g >= q) break;
+        double o[2][4];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          if (t >= nprod) break;
+          const int a = (it * nprod + t) & 1;
+          float v[kDiags][4];
+#pragma unroll
+          for (int d = 0; d < kDiags; ++d)
+            tmem_ld4(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(a * kAcc + kQ * d + 4 * g), v[d]);
+          tmem_wait_ld(v);
+          const double* b = job.base[t] && live ? job.base[t] + grow * job.ld_base[t] : nullptr;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int j = 4 * g + i;
+            float w[kDiags];
+#pragma unroll
+            for (int d = 0; d < kDiags; ++d) w[d] = v[d][i];
+            o[t][i] = er[t] == kBad ? (j < q ? slow[t][j] : 0.0) : join(w, er[t] - 1022 + col_exp[j] - 1022 - 70);
+            if (b && j < q) o[t][i] = b[j] + o[t][i];
+          }
+          if (live) {
+            double* p = job.out[t] + grow * job.ld_out[t] + 4 * g;
+            if (4 * g + 4 <= q && !(job.ld_out[t] & 1) && !(reinterpret_cast<uintptr_t>(job.out[t]) & 15)) {
+              reinterpret_cast<double2*>(p)[0] = make_double2(o[t][0], o[t][1]);
+              reinterpret_cast<double2*>(p)[1] = make_double2(o[t][2], o[t][3]);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                if (4 * g + i < q) p[i] = o[t][i];
+            }
+          }
+        }
+        if constexpr (NORM) {
+          // residuals AX - lam X of the four columns; warp `quad` of this half then takes column 4 g + quad
+          asm volatile("bar.sync %0, 128;\n" ::"r"(3 + half) : "memory");  // the previous group is read
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            res[half][i][row] = live && 4 * g + i < q ? fma(-lam_s[4 * g + i], o[0][i], o[1][i]) : 0.0;
+          asm volatile("bar.sync %0, 128;\n" ::"r"(3 + half) : "memory");
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const double x = res[half][quad][32 * u + lane];
+            nsum[gh] = fma(x, x, nsum[gh]);
+            // max of magnitudes by their bits (a NaN does not count, as in fmax)
+            const long long ax = __double_as_longlong(x) & 0x7fffffffffffffffll;
+            if (ax > __double_as_longlong(nmax[gh]) && ax <= 0x7ff0000000000000ll) nmax[gh] = __longlong_as_double(ax);
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+        if (t < nprod && lane == 0) mbar_arrive(&acc_empty[(it * nprod + t) & 1]);
+    }
+    if constexpr (NORM) {
+#pragma unroll
+      for (int gh = 0; gh < kQ / 8; ++gh) {
+        const double s2 = warp_sum(nsum[gh]), mx = warp_max(nmax[gh]);
+        const int j = 4 * (2 * gh + half) + quad;
+        if (lane == 0 && j < q) {
+          norm_part[(int64_t)blockIdx.x * 2 * q + j] = s2;
+          norm_part[(int64_t)blockIdx.x * 2 * q + q + j] = mx;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (abort_flag) {
+    if (warp < kSplitWarps && lane == 0 && copied > 0) mbar_wait(&raw_full[warp], (uint32_t)(copied - 1) & 1u, kWaitCycles);
+    if (warp == kMma && lane == 0 && committed > 0)
+      mbar_wait(&acc_full[(committed - 1) & 1], (uint32_t)((committed - 1) / 2) & 1u, kWaitCycles);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMma) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem, 2 * kAcc);
+  }
+}
+
+__global__ void update64_err_reset_kernel() { g_update64_err = 0; }
+
+template <int NC, bool NORM>
+int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
+                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, cudaStream_t st) {
+  static const bool attr = [&] {
+    LB_CUDA(cudaFuncSetAttribute(update64_kernel<NC, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBudget - kStatic)));
+    return true;
+  }();
+  (void)attr;
+  int dev = 0, sms = 152;
+  LB_CUDA(cudaGetDevice(&dev));
+  LB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int64_t tiles = ceil_div(n, kTile);
+  const int64_t per = ceil_div(tiles, std::min<int64_t>(std::min<int64_t>(max_ctas, sms), tiles));
+  const int64_t ctas = ceil_div(tiles, per);
+  update64_kernel<NC, NORM><<<(unsigned)ctas, kThreads, smem, st>>>(n, job, U, s, q, alpha, lam, norm_part, per,
+                                                                     ts);
+  LB_LAUNCH_CHECK();
+  return (int)ctas;
+}
+
+}  // namespace
+
+// The block update through digit products; returns 0 without launching where the blocks do not fit
+// (unaligned or odd row strides, products of different layout, more shared memory than a CTA has).
+int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
+                         const double* lam, double* norm_part, int max_ctas, cudaStream_t st) {
+  if (n <= 0 || q < 1 || q > kQ || s < 1 || s > kMaxS || job.in[0].nseg < 1) return 0;
+  if (norm_part && (job.nprod != 2 || job.base[0] || job.base[1])) return 0;
+  size_t raw = 0;
+  for (int t = 0; t < job.nprod; ++t) {
+    const Cols<double>& c = job.in[t];
+    if (c.nseg != job.in[0].nseg) return 0;
+    for (int g = 0; g < c.nseg; ++g) {
+      if ((c.ld[g] & 1) || c.w[g] > c.ld[g] || (reinterpret_cast<uintptr_t>(c.p[g]) & 15)) return 0;
+      if (c.w[g] != job.in[0].w[g] || c.ld[g] != job.in[0].ld[g]) return 0;
+      if (t == 0) raw += (size_t)kTile * c.ld[g] * 8;
+    }
+  }
+  const int nc = (s + kKC - 1) / kKC;
+  const size_t fixed = kSlices * (size_t)u_slice(nc * kKC) + raw;
+  const int ts = fixed + 2 * (size_t)kBuf <= kSmemBudget - kStatic ? 2 : 1;
+  const size_t smem = fixed + (size_t)ts * kBuf;
+  if (smem > kSmemBudget - kStatic) return 0;
+#define LB_UPDATE64(NC)                                                                                          \
+  return norm_part ? update64_launch<NC, true>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, st)        \
+                   : update64_launch<NC, false>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, st)
+  if (nc == 1) LB_UPDATE64(1);
+  if (nc == 2) LB_UPDATE64(2);
+  LB_UPDATE64(3);
+#undef LB_UPDATE64
+}
+
+void update64_check(cudaStream_t st) {
+  int err = 0;
+  LB_CUDA(cudaMemcpyFromSymbolAsync(&err, g_update64_err, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
+  LB_CUDA(cudaStreamSynchronize(st));
+  if (err) {
+    update64_err_reset_kernel<<<1, 1, 0, st>>>();
+    LB_LAUNCH_CHECK();
+    LB_CUDA(cudaStreamSynchronize(st));
+    throw CudaError("tensor-core FP64 update: a pipeline stage did not complete in time");
+  }
+}
+
+}  // namespace lobpcg
