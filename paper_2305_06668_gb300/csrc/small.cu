@@ -755,15 +755,23 @@ __device__ void small_ortho(int s, int a, double* X, int ldx, double tau, int ca
     } else {
       svqb_cta(a, M, ld, L, Z, ld, Tm, ld, rot, red, theta);
     }
-    // X <- X Tm, row by row (each thread owns rows of X)
-    for (int r = threadIdx.x; r < s; r += blockDim.x) {
-      double row[kMaxM];
-      for (int j = 0; j < a; ++j) row[j] = X[r + j * ldx];
-      for (int j = 0; j < a; ++j) {
-        double acc = 0.0;
-        for (int l = 0; l < a; ++l) acc += row[l] * Tm[l + j * ld];
-        X[r + j * ldx] = acc;
-      }
+    // X <- X Tm: every thread forms its entries, then all are stored
+    constexpr int kPer = (kMaxS * kMaxM + kSmallThreads - 1) / kSmallThreads;
+    double v[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int e = threadIdx.x + k * kSmallThreads;
+      if (e >= s * a) break;
+      const int r = e % s, j = e / s;
+      double acc = 0.0;
+      for (int l = 0; l < a; ++l) acc += X[r + l * ldx] * Tm[l + j * ld];
+      v[k] = acc;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int e = threadIdx.x + k * kSmallThreads;
+      if (e < s * a) X[e % s + (e / s) * ldx] = v[k];
     }
     __syncthreads();
   }
@@ -782,12 +790,16 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
   __shared__ double theta[kMaxS];
   __shared__ int conv[kMaxM];
   __shared__ int flag, shifts, s_mconv, s_mact, s_done, s_pw;
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
+  // one warp per column, its lanes over the partial sums (fixed order)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  for (int j = warp; j < m; j += nwarps) {
     double s2 = 0.0, mx = 0.0;
-    for (int g = 0; g < nparts; ++g) {
+    for (int g = lane; g < nparts; g += 32) {
       s2 += norm_part[(int64_t)g * 2 * m + j];
       mx = fmax(mx, norm_part[(int64_t)g * 2 * m + m + j]);
     }
+    s2 = warp_sum(s2), mx = warp_max(mx);
+    if (lane) continue;
     const double nr = sqrt(s2);
     resnorm[j] = nr;
     colmax[j] = mx;
@@ -829,20 +841,23 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
   // vanishes exactly (a zero vector cannot be normalised and would give a spurious Ritz
   // value 0 in V); pack the kept columns to the front.
   __shared__ int keep[kMaxM];
-  for (int c = threadIdx.x; c < a; c += blockDim.x) {
-    double cf[kMaxM];
-    for (int i = 0; i < m; ++i) {
-      double d = 0.0;
-      for (int r = 0; r < s; ++r) d += Y[r + i * ld] * X[r + c * ld];
-      cf[i] = d;
-    }
+  // (C = u_x^T u~_p by all threads, then one warp per column)
+  for (int e = threadIdx.x; e < m * a; e += blockDim.x) {
+    const int i = e % m, j = e / m;
+    double acc = 0.0;
+    for (int r = 0; r < s; ++r) acc += Y[r + i * ld] * X[r + j * ld];
+    C[i + j * lds] = acc;
+  }
+  __syncthreads();
+  for (int c = warp; c < a; c += nwarps) {
     double nrm = 0.0;
-    for (int r = 0; r < s; ++r) {
+    for (int r = lane; r < s; r += 32) {
       double v = X[r + c * ld];
-      for (int i = 0; i < m; ++i) v -= Y[r + i * ld] * cf[i];
+      for (int i = 0; i < m; ++i) v -= Y[r + i * ld] * C[i + c * lds];
       nrm += v * v;
     }
-    keep[c] = sqrt(nrm) > 1e-200 ? 1 : 0;
+    nrm = warp_sum(nrm);
+    if (lane == 0) keep[c] = sqrt(nrm) > 1e-200 ? 1 : 0;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -893,15 +908,16 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
   }
   // drop columns that could not be made orthonormal against u_x (more P directions than
   // the complement of u_x holds, e.g. after a column was unlocked); pack the rest
-  for (int c = threadIdx.x; c < ap; c += blockDim.x) {
+  for (int c = warp; c < ap; c += nwarps) {
     double worst = 0.0, nrm = 0.0;
-    for (int i = 0; i < m; ++i) {
+    for (int i = lane; i < m; i += 32) {
       double d = 0.0;
       for (int r = 0; r < s; ++r) d += Y[r + i * ld] * X[r + c * ld];
       worst = fmax(worst, fabs(d));
     }
-    for (int r = 0; r < s; ++r) nrm += X[r + c * ld] * X[r + c * ld];
-    keep[c] = (worst <= sqrt(tau) && fabs(sqrt(nrm) - 1.0) <= sqrt(tau)) ? 1 : 0;
+    for (int r = lane; r < s; r += 32) nrm += X[r + c * ld] * X[r + c * ld];
+    worst = warp_max(worst), nrm = warp_sum(nrm);
+    if (lane == 0) keep[c] = (worst <= sqrt(tau) && fabs(sqrt(nrm) - 1.0) <= sqrt(tau)) ? 1 : 0;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
