@@ -250,6 +250,10 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,
                  cudaStream_t st, bool two_stage = false, double tol64 = 1e-15);
 
+// The cluster eigensolver behind launch_syev (syev.cu): lam[0] = NaN where it gave up.
+void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, double* U, int* steps_out, float stop,
+                         cudaStream_t st);
+
 // Cholesky-QR step on the reduced Gram matrix M (p x p, column-major):
 //  ctl[0] <- 1 if max|M - I| <= tau (already orthonormal), else 0 and Linv <- L^{-T}
 //  of chol(M + shift) (upper triangular, column-major p x p).  ctl[1] += shifted

@@ -395,8 +395,11 @@ template <bool TWO_STAGE>
 __global__ void __launch_bounds__(kSmallThreads) syev_kernel(int s, const double* __restrict__ a_in,
                                                              int upper_only, double* __restrict__ lam,
                                                              double* __restrict__ U, int* sweeps_out,
-                                                             double tol32, double tol64) {
+                                                             double tol32, double tol64, int behind) {
   extern __shared__ double sm[];
+  // behind syev_cluster_kernel: only where that one gave up
+  if (behind && !isnan(*static_cast<volatile double*>(lam))) return;
+  __syncthreads();
   __shared__ double red[32];
   __shared__ double rot[4 * (kMaxS / 2 + 1)];
   __shared__ int rank[kMaxS];
@@ -956,11 +959,17 @@ void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U
     return true;
   }();
   (void)attr;
+  // The cluster solver from 2 columns on (syev.cu; measured per call at s = 63, see there); this
+  // kernel then runs only where that one gave up.
+  const bool behind = s > 1;
+  if (behind) launch_syev_cluster(s, a, upper_only, lam, U, sweeps_out, tol64 >= 1e-12 ? 1e-5f : 1e-9f, st);
   const double tol32 = 1e-4;  // measured: the stopping point of this stage hardly changes the total
   if (two_stage)
-    syev_kernel<true><<<1, kSmallThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, sweeps_out, tol32, tol64);
+    syev_kernel<true><<<1, kSmallThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, sweeps_out, tol32, tol64,
+                                                     behind ? 1 : 0);
   else
-    syev_kernel<false><<<1, kSmallThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, sweeps_out, tol32, tol64);
+    syev_kernel<false><<<1, kSmallThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, sweeps_out, tol32, tol64,
+                                                     behind ? 1 : 0);
   LB_LAUNCH_CHECK();
 }
 
