@@ -559,9 +559,42 @@ __device__ int chol_cta(int p, double* L, int ld, int* flag) {
   return f;
 }
 
-// Shifted Cholesky of M (p x p, ld): tries M, then M + sigma I with sigma = 100 eps
-// trace(M) * 10^t, t = 0..7.  L receives the factor.  Returns 0 on success.
-__device__ int shifted_chol_cta(int p, const double* M, int ldm, double* L, int ld, int* flag,
+// T = L^{-T} (upper triangular, column-major, ldt) of the Cholesky factor L of the p x p matrix in the
+// lower part of W (ld, destroyed), by one elimination of [W | I] in square-root-free form; Y (p x p, ld)
+// is scratch.  A step is one pass between two barriers and one reciprocal that every thread forms for
+// itself.  (Factor, then one substitution per column: three barriers and a chain of a square root and a
+// division per column, then p^2 / 2 dependent FMAs in a thread, 50 us at p = 21.)  Returns 0, or j + 1 for
+// the first non-positive pivot (same value in every thread).
+__device__ int chol_inverse_cta(int p, double* W, double* Y, int ld, double* T, int ldt) {
+  for (int e = threadIdx.x; e < p * p; e += blockDim.x) Y[e % p + (e / p) * ld] = e % p == e / p ? 1.0 : 0.0;
+  __syncthreads();
+  for (int j = 0; j < p; ++j) {
+    const double d = W[j + j * ld];
+    if (!(d > 0.0)) {
+      __syncthreads();  // every thread has read the pivot before a caller overwrites W
+      return j + 1;
+    }
+    const double inv = 1.0 / d;
+    // rows i > j: columns up to j of Y, columns j + 1 .. i of W
+    for (int e = threadIdx.x; e < (p - j - 1) * p; e += blockDim.x) {
+      const int i = j + 1 + e % (p - j - 1), c = e / (p - j - 1);
+      const double f = W[i + j * ld] * inv;
+      if (c <= j) Y[i + c * ld] -= f * Y[j + c * ld];
+      else if (c <= i) W[i + c * ld] -= f * W[c + j * ld];
+    }
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
+    const int i = e % p, j = e / p;  // L^{-1}(i, j), transposed into T
+    T[j + i * ldt] = i >= j ? Y[i + j * ld] / sqrt(W[i + i * ld]) : 0.0;
+  }
+  __syncthreads();
+  return 0;
+}
+
+// T = L^{-T} of the shifted Cholesky factor of M (p x p, ldm): tries M, then M + sigma I with
+// sigma = 100 eps trace(M) * 10^t, t = 0..7.  W and Y (p x p, ld) are scratch.  Returns 0 on success.
+__device__ int shifted_chol_cta(int p, const double* M, int ldm, double* W, double* Y, int ld, double* T, int ldt,
                                 int* shifts, double* red) {
   double tr = 0.0;
   for (int i = threadIdx.x; i < p; i += blockDim.x) tr += M[i + i * ldm];
@@ -571,27 +604,12 @@ __device__ int shifted_chol_cta(int p, const double* M, int ldm, double* L, int 
     const double sigma = t < 0 ? 0.0 : 100.0 * DBL_EPSILON * tr * pow(10.0, (double)t);
     for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
       const int i = e % p, j = e / p;
-      L[i + j * ld] = M[i + j * ldm] + (i == j ? sigma : 0.0);
+      W[i + j * ld] = M[i + j * ldm] + (i == j ? sigma : 0.0);
     }
-    __syncthreads();
     if (t >= 0 && threadIdx.x == 0) ++*shifts;
-    fail = chol_cta(p, L, ld, flag);
+    fail = chol_inverse_cta(p, W, Y, ld, T, ldt);  // its first barrier completes W
   }
   return fail;
-}
-
-// T = L^{-T} (upper triangular p x p, column-major, ldt) from the lower factor L.
-__device__ void inv_lower_transpose_cta(int p, const double* L, int ld, double* T, int ldt) {
-  // column j of L^{-1} by forward substitution; written transposed into row j of T
-  for (int j = threadIdx.x; j < p; j += blockDim.x) {
-    for (int i = 0; i < p; ++i) T[j + i * ldt] = 0.0;
-    for (int i = j; i < p; ++i) {
-      double s = i == j ? 1.0 : 0.0;
-      for (int l = j; l < i; ++l) s -= L[i + l * ld] * T[j + l * ldt];
-      T[j + i * ldt] = s / L[i + i * ld];
-    }
-  }
-  __syncthreads();
 }
 
 // SVQB transform T = D Z Theta^{-1/2} for Gram M (Stathopoulos & Wu).  Uses B (p x p,
@@ -633,12 +651,13 @@ __global__ void __launch_bounds__(kSmallThreads) cholqr_small_kernel(int p, cons
   __shared__ double red[32];
   __shared__ double rot[4 * (kMaxS / 2 + 1)];
   __shared__ double theta[kMaxS];
-  __shared__ int flag, shifts;
+  __shared__ int shifts;
   const int ld = p | 1;  // odd stride: row accesses hit distinct banks
   double* M = sm;
   double* L = M + p * ld;
   double* T = L + p * ld;
   double* Z = T + p * ld;
+  double* Y = Z + p * ld;
   double dev = 0.0;
   for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
     const int i = e % p, j = e / p;
@@ -684,9 +703,8 @@ __global__ void __launch_bounds__(kSmallThreads) cholqr_small_kernel(int p, cons
   }
   fro = sqrt(block_sum(fro, red));
   __syncthreads();
-  const int fail = shifted_chol_cta(p, Z, ld, L, ld, &flag, &shifts, red);
+  const int fail = shifted_chol_cta(p, Z, ld, L, Y, ld, T, ld, &shifts, red);
   if (!fail) {
-    inv_lower_transpose_cta(p, L, ld, T, ld);
     for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
       const int i = e % p, j = e / p;
       T[i + j * ld] *= theta[i];
@@ -724,8 +742,8 @@ __global__ void maxabs_kernel(int count, const double* __restrict__ C, double* o
 // ---- Algorithm 2 / 3 in the small s-dimensional space (for u_p) -----------------------
 // X: s x a (column-major, ldx), Y: s x q (ldy); everything in shared memory.
 __device__ void small_ortho(int s, int a, double* X, int ldx, double tau, int cap, double* M,
-                            double* L, double* Tm, double* Z, int ld, double* rot, double* red,
-                            double* theta, int* flag, int* shifts) {
+                            double* L, double* Tm, double* Z, double* Yb, int ld, double* rot, double* red,
+                            double* theta, int* shifts) {
   for (int pass = 0;; ++pass) {
     for (int e = threadIdx.x; e < a * a; e += blockDim.x) {
       const int i = e % a, j = e / a;
@@ -750,9 +768,8 @@ __device__ void small_ortho(int s, int a, double* X, int ldx, double tau, int ca
       Z[i + j * ld] = theta[i] * M[i + j * ld] * theta[j];
     }
     __syncthreads();
-    const int fail = shifted_chol_cta(a, Z, ld, L, ld, flag, shifts, red);
+    const int fail = shifted_chol_cta(a, Z, ld, L, Yb, ld, Tm, ld, shifts, red);
     if (!fail) {
-      inv_lower_transpose_cta(a, L, ld, Tm, ld);
       for (int e = threadIdx.x; e < a * a; e += blockDim.x) Tm[(e % a) + (e / a) * ld] *= theta[e % a];
       __syncthreads();
     } else {
@@ -792,7 +809,7 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
   __shared__ double rot[4 * (kMaxS / 2 + 1)];
   __shared__ double theta[kMaxS];
   __shared__ int conv[kMaxM];
-  __shared__ int flag, shifts, s_mconv, s_mact, s_done, s_pw;
+  __shared__ int shifts, s_mconv, s_mact, s_done, s_pw;
   // one warp per column, its lanes over the partial sums (fixed order)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   for (int j = warp; j < m; j += nwarps) {
@@ -834,6 +851,7 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
   double* L = M + kMaxM * lds;
   double* Tm = L + kMaxM * lds;
   double* Z = Tm + kMaxM * lds;
+  double* Yb = Z + kMaxM * lds;
   for (int e = threadIdx.x; e < s * a; e += blockDim.x) {
     const int r = e % s, c = e / s;
     X[r + c * ld] = U[r + (mc + c) * s] - (r == mc + c ? 1.0 : 0.0);  // u~_p = u_x[:,act] - E_act
@@ -895,7 +913,7 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
       X[r + j * ld] -= acc;
     }
     __syncthreads();
-    small_ortho(s, ap, X, ld, tau, cap, M, L, Tm, Z, lds, rot, red, theta, &flag, &shifts);
+    small_ortho(s, ap, X, ld, tau, cap, M, L, Tm, Z, Yb, lds, rot, red, theta, &shifts);
     ++passes;
     double mx = 0.0;
     for (int e = threadIdx.x; e < m * ap; e += blockDim.x) {
@@ -977,10 +995,10 @@ void launch_cholqr_small(int p, const double* M, double tau, double* Linv, int* 
                          const double* C, int q, double growth2) {
   if (p <= 0) return;
   if (p > kMaxCholP) throw std::invalid_argument("cholqr: p > 64");
-  const size_t smem = (size_t)4 * p * (p + 1) * sizeof(double);
+  const size_t smem = (size_t)5 * p * (p + 1) * sizeof(double);
   // set once per process; function-local statics initialise thread-safely
   static const bool attr = [&] {
-    LB_CUDA(cudaFuncSetAttribute(cholqr_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kMaxCholP * (kMaxCholP + 1) * 8));
+    LB_CUDA(cudaFuncSetAttribute(cholqr_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 5 * kMaxCholP * (kMaxCholP + 1) * 8));
     return true;
   }();
   (void)attr;
@@ -1015,7 +1033,7 @@ void launch_maxabs(int count, const double* C, double* out, cudaStream_t st) {
 void launch_lock_and_p(int s, int m, int k, int64_t n, const double* norm_part, int nparts,
                        const double* U, double tol, int tol_kind, double tau, LockState* state,
                        double* resnorm, double* colmax, double* up, bool build_p, cudaStream_t st) {
-  const size_t smem = ((size_t)2 * kMaxM * (kMaxS + 1) + (size_t)5 * kMaxM * (kMaxM + 1)) * sizeof(double);
+  const size_t smem = ((size_t)2 * kMaxM * (kMaxS + 1) + (size_t)6 * kMaxM * (kMaxM + 1)) * sizeof(double);
   // set once per process; function-local statics initialise thread-safely
   static const bool attr = [&] {
     LB_CUDA(cudaFuncSetAttribute(lock_p_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
