@@ -126,10 +126,17 @@ bool launch_spmm_band_packed(int64_t n, const int64_t* rp_packed, const int2* pa
 // Smallest half-width b in {16, ..., 2048} with 80% of the non-zeros at |col - row| <= b,
 // or -1 (synchronises the stream).
 int profile_band(int64_t n, const int64_t* row_ptr, const int32_t* col_idx, int64_t nnz, cudaStream_t st);
-// Y = A X, dense column-major symmetric A.
+// Y = A X, dense column-major symmetric A.  run_flag (device, may be null): the kernels return
+// without writing unless *run_flag is not zero.
 template <class T>
 void launch_spmm_dense(int64_t n, const T* A, int64_t lda, int p, const T* X, int ldx, T* Y,
-                       int ldy, cudaStream_t st);
+                       int ldy, cudaStream_t st, const int* run_flag = nullptr);
+// The FP64 product through exact digit products on the tensor cores (gram64.cu); false without
+// launching where the operands do not fit.  *scratch (dense64_scratch_bytes) is the flag left at 1
+// when a number is outside the digits' range: Y is then to be formed by launch_spmm_dense on it.
+size_t dense64_scratch_bytes(int64_t n, int p);
+bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
+                              int ldy, void* scratch, cudaStream_t st);
 
 // Gram partials: part[g][i + j*pa] = sum over CTA g's rows of a_ri * b_rj.
 // upper: only i <= j entries are produced.  Returns the number of CTAs used.

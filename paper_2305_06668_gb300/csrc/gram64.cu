@@ -19,14 +19,22 @@
 //     so consecutive slices are one operand of N = NB, 2 NB, ... columns.  The MMA of A pair i and
 //     B slices j, j + 1, .. writes TMEM columns NB (i + j), ..: TMEM lanes 0..63 of region t sum the
 //     products with i + j = t (i even) and lanes 64..127 those with i + j = t + 1 (i odd).
+//     A of at most 32 columns has slices of 32 (CA), four to an operand: five products of 608 TMEM columns
+//     a K step become three of 352, and A and B of one block share their tiles.
 //   * At most four digit products per row meet in one accumulator: 4 * 256 * 2^14 = 2^24, exact.
 //   * After 256 rows the epilogue joins the eight regions of every element into one FP64 number
 //     with integer operations and adds it to its running sum (one FP64 add).
+// The dense symmetric product Y = A X (PANEL) is the same contraction with A's columns in memory order:
+// a CTA owns 64 columns of A and a range of its rows and writes its 64 x p sums; ranges of rows split a
+// matrix of few panels over the SMs.  The splitters load A from global memory straight into registers, a
+// chunk ahead (a lane's 8 rows of a column are 64 contiguous bytes): 256-byte bulk copies of the columns
+// took 70 clocks each, 4.5k per chunk, and made a product of n = 8192 wait on them for 0.45 of 0.6 ms.
+//
 // A flag set by exp_kernel (a column's block with an infinity, a NaN or an exponent outside
 // 2^+-400) makes gram64_kernel return at once; the caller's general kernel, launched behind it on
 // the same flag, then forms the partials.
 #include <algorithm>
-#include <type_traits>
+#include <climits>
 
 #include "common.cuh"
 #include "slices.cuh"
@@ -49,7 +57,6 @@ constexpr int kEpi0 = 2, kEpiWarps = 8;
 constexpr int kSplit0 = kEpi0 + kEpiWarps, kSplitWarps = 8, kSplitGroups = 2;
 constexpr int kThreads = 32 * (kSplit0 + kSplitWarps);
 constexpr uint32_t kLBO = 128, kSBO = kKC / 8 * 128;  // bytes between core matrices along K and M / N
-constexpr uint32_t kSliceA = kCB / 8 * kSBO;          // bytes of one A slice
 constexpr long long kWaitCycles = 1ll << 31;
 constexpr size_t kSmemBudget = 220 * 1024;
 
@@ -116,15 +123,63 @@ __global__ void __launch_bounds__(256) exp_kernel(int64_t n, Cols<double> A, Col
   }
 }
 
-// Columns [a0, a0 + pa) of A and [b0, b0 + pb) of B; NB: B columns per slice (>= pb).
-template <int NB>
+// Exponents of a dense column-major A (n x n, lda): one warp per column and group of kGroupRows rows.
+__global__ void __launch_bounds__(256) exp_dense_kernel(int64_t n, const double* __restrict__ A, int64_t lda,
+                                                        int* __restrict__ exps, int64_t stride,
+                                                        int* __restrict__ flag) {
+  const int64_t col = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (col >= n) return;
+  const int64_t r0 = (int64_t)blockIdx.y * kGroupRows;
+  const int rows = (int)min((int64_t)kGroupRows, n - r0);
+  const double2* p = reinterpret_cast<const double2*>(A + col * lda + r0);
+  double2 x[kGroupRows / 64];
+#pragma unroll
+  for (int u = 0; u < kGroupRows / 64; ++u)
+    x[u] = 2 * (lane + 32 * u) < rows ? __ldg(p + lane + 32 * u) : make_double2(0.0, 0.0);  // rows is even
+  uint32_t k = 0u;
+#pragma unroll
+  for (int u = 0; u < kGroupRows / 64; ++u) k = max(k, max(exp_key(x[u].x), exp_key(x[u].y)));
+  k = __reduce_max_sync(0xffffffffu, k);
+  if (lane) return;
+  const int e = group_exp(k);
+  if (e < 0) *flag = 1;
+  exps[blockIdx.y * stride + col] = e;
+}
+
+// Exponents of a row-major block of p <= 32 columns (any row stride), one CTA per group.
+__global__ void __launch_bounds__(256) exp_rows_kernel(int64_t n, int p, const double* __restrict__ X, int ldx,
+                                                       int* __restrict__ exps, int64_t stride,
+                                                       int* __restrict__ flag) {
+  __shared__ uint32_t key[32];
+  if (threadIdx.x < 32) key[threadIdx.x] = 0u;
+  __syncthreads();
+  const int64_t r0 = (int64_t)blockIdx.x * kGroupRows;
+  const int rows = (int)min((int64_t)kGroupRows, n - r0), j = threadIdx.x & 31;
+  uint32_t k = 0u;
+  if (j < p)
+    for (int r = threadIdx.x >> 5; r < rows; r += 8) k = max(k, exp_key(__ldg(X + (r0 + r) * ldx + j)));
+  atomicMax(&key[j], k);
+  __syncthreads();
+  if (threadIdx.x < p) {
+    const int e = group_exp(key[threadIdx.x]);
+    if (e < 0) *flag = 1;
+    exps[blockIdx.x * stride + threadIdx.x] = e;
+  }
+}
+
+// Columns [a0, a0 + pa) of A and [b0, b0 + pb) of B; NB: B columns per slice (>= pb).  PANEL: A and B
+// hold one dense column-major A (ld: its leading dimension) and one row-major block; the CTA's a0 and
+// rows follow from its index, and element (row, j) goes to part[split][row * pb + j].
+// CA: columns of an A slice (32 or 64; >= pa).
+template <int CA, int NB, bool PANEL>
 __global__ void __launch_bounds__(kThreads, 1)
     gram64_kernel(int64_t n, Cols<double> A, Cols<double> B, int ld, int a0, int pa, int b0, int pb, int upper,
                   int same, int rs, const int* __restrict__ exps, int estride, int eb0,
-                  const int* __restrict__ flag, double* __restrict__ part, int64_t groups_per_cta) {
+                  const int* __restrict__ flag, double* __restrict__ part, int64_t groups_per_cta, int npanels) {
   constexpr int kAS = NB <= 32 ? 2 : 1;  // accumulators (of kDiags * NB TMEM columns)
   constexpr int kAcc = kDiags * NB;
-  constexpr uint32_t kSliceB = NB / 8 * kSBO;
+  constexpr uint32_t kSliceA = CA / 8 * kSBO, kSliceB = NB / 8 * kSBO;  // bytes of a slice
   constexpr int kEW = NB / 2;  // columns per epilogue warp (two warps per lane quadrant)
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t raw_full[kMaxRS], raw_empty[kMaxRS], tile_full[kTS], tile_empty[kTS];
@@ -139,10 +194,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (*flag) return;  // written by an earlier kernel: the same for every thread
   const int ta = A.width(), tb = B.width();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if constexpr (PANEL) {
+    a0 = (int)(blockIdx.x % (unsigned)npanels) * kCB;
+    pa = (int)min((int64_t)kCB, n - a0);
+  }
   const int seg = kKC * ld;
   if (tid == 0) {
     int nu = 0;
-    for (int o = 0; o < (same ? 1 : 2); ++o) {
+    for (int o = 0; o < (PANEL ? 0 : same ? 1 : 2); ++o) {
       const Cols<double>& c = o == 0 ? A : B;
       const int lo = o == 0 ? a0 : b0, hi = lo + (o == 0 ? pa : pb);
       int base = 0;
@@ -167,7 +226,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int o = i / kCB, m = i % kCB;
     const Cols<double>& c = o == 0 ? A : B;
     int off = -1;
-    if (m < (o == 0 ? pa : pb) && !(o == 1 && same)) {
+    if (PANEL) {
+      if (m < (o == 0 ? pa : pb)) off = m;  // A: not staged
+    } else if (m < (o == 0 ? pa : pb) && !(o == 1 && same)) {
       const int col = m + (o == 0 ? a0 : b0);
       int base = 0, g = 0;
       while (col >= base + c.w[g]) base += c.w[g], ++g;
@@ -177,8 +238,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     colofs[o][m] = off;
   }
-  const size_t raw_bytes = ((size_t)rs * nu * seg * 8 + 127) / 128 * 128;
-  double* raw = reinterpret_cast<double*>(smem);  // [rs][nu][kKC][ld]
+  // doubles of a raw stage: [nu][kKC][ld], or kKC rows of X
+  const int stage = PANEL ? kKC * B.ld[0] : nu * seg;
+  const size_t raw_bytes = ((size_t)rs * stage * 8 + 127) / 128 * 128;
+  double* raw = reinterpret_cast<double*>(smem);  // [rs][stage]
   unsigned char* tiles = smem + raw_bytes;
   const uint32_t oB = same ? 0u : 8u * kSliceA;
   const uint32_t tbuf = 8u * kSliceA + (same ? 0u : (uint32_t)kSlices * kSliceB);
@@ -191,13 +254,28 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
 
-  const int64_t g_begin = (int64_t)blockIdx.x * groups_per_cta;
+  const int64_t g_begin = (int64_t)(PANEL ? blockIdx.x / (unsigned)npanels : blockIdx.x) * groups_per_cta;
   const int64_t r_begin = g_begin * kGroupRows;
   const int64_t r_end = min(n, r_begin + groups_per_cta * kGroupRows);
   const int nchunks = r_end > r_begin ? (int)((r_end - r_begin + kKC - 1) / kKC) : 0;
   const int ngroups = (nchunks + kChunks - 1) / kChunks;
   int issued = 0, committed = 0;  // producer thread; MMA thread (groups)
-  if (warp == 0) {
+  if (PANEL && warp == 0) {
+    if (lane == 0) {
+      int st = 0;
+      uint32_t ph = 0;
+      for (int c = 0; c < nchunks; ++c) {
+        if (c >= rs && !wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, 3)) break;
+        const int64_t r0 = r_begin + (int64_t)c * kKC;
+        const int rows = (int)min((int64_t)kKC, r_end - r0);  // even: n is
+        const uint32_t bytes = (uint32_t)((rows - 1) * B.ld[0] + pb + 1) / 2 * 16u;
+        mbar_expect_tx(&raw_full[st], bytes);
+        bulk_g2s(raw + (size_t)st * stage, B.p[0] + r0 * B.ld[0], bytes, &raw_full[st]);
+        issued = c + 1;
+        if (++st == rs) st = 0, ph ^= 1u;
+      }
+    }
+  } else if (warp == 0) {
     if (lane == 0) {
       int st = 0;
       uint32_t ph = 0;
@@ -209,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = 0; u < nu; ++u) total += (uint32_t)((rows - 1) * ld + ucopy[u]) * 8u;
         mbar_expect_tx(&raw_full[st], total);
         for (int u = 0; u < nu; ++u)
-          bulk_g2s(raw + ((size_t)st * nu + u) * seg, useg[u] + r0 * ld, (uint32_t)((rows - 1) * ld + ucopy[u]) * 8u,
+          bulk_g2s(raw + (size_t)st * stage + u * seg, useg[u] + r0 * ld, (uint32_t)((rows - 1) * ld + ucopy[u]) * 8u,
                    &raw_full[st]);
         issued = c + 1;
         if (++st == rs) st = 0, ph ^= 1u;
@@ -238,6 +316,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int kk = 0; kk < kKC / 16; ++kk) {
           const uint32_t acc = in_group > 0 || kk > 0 ? 1u : 0u;
+          if constexpr (CA == 32) {  // four A slices an operand: TMEM lanes 32 u .. hold i + j = t + u
+            mma(kk, 0, 0, kSlices, acc);  // regions 0..6
+            mma(kk, 4, 0, 3, 1u);
+            mma(kk, 4, 3, 1, acc);  // region 7
+          } else {
           // regions 0..6
 #pragma unroll
           for (int j = 0; j < kSlices; j += W) mma(kk, 0, j, min(W, kSlices - j), acc);
@@ -247,6 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           mma(kk, 2, 5, 1, acc);
           mma(kk, 4, 0, 4, 1u);
           mma(kk, 6, 0, 2, 1u);
+          }
         }
         mma_commit(&tile_empty[buf]);
         if (in_group == kChunks - 1 || c == nchunks - 1) {
@@ -260,21 +344,23 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp < kSplit0) {
     // epilogue: warp w reads TMEM lanes 32 (w mod 4) .. + 31, columns [kEW half, + kEW) of each region
     const int quad = warp & 3, half = (warp - kEpi0) >> 2;
-    const int row = (32 * quad + lane) & 63;  // column of A
-    const bool odd = quad >= 2;               // regions hold i + j = t + 1
+    const int row = (32 * quad + lane) & (CA - 1);  // column of A
+    const int part_ = 32 * quad / CA;               // regions hold i + j = t + part_
     double acc[kEW];
 #pragma unroll
     for (int j = 0; j < kEW; ++j) acc[j] = 0.0;
     int r = 0, g = 0;
     uint32_t aph = 0;
     for (; g < ngroups; ++g) {
-      const int* ge = exps + (g_begin + g) * estride;
+      const int* ge = exps + (g_begin + g) * (int64_t)estride;
+      // exponents of this lane's row and of column `lane` of this warp, before the wait
       const int ea = row < pa ? __ldg(ge + a0 + row) : kExpOne;
+      const int ebl = lane < kEW && kEW * half + lane < pb ? __ldg(ge + eb0 + b0 + kEW * half + lane) : kExpOne;
       if (!__all_sync(0xffffffffu, wait_bar(&acc_full[r], aph, &abort_flag, 2))) break;
       tc_fence_after();
       const uint32_t t0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(r * kAcc + kEW * half);
-      // element: (sum_t v_t 256^(7-t)) 2^(40 - 110) 2^(ea - 1022) 2^(eb - 1022), / 256 in lanes 64..127
-      const int sa = ea - 1022 - 70 - (odd ? 8 : 0);
+      // element: (sum_t v_t 256^(7-t)) 2^(40 - 110) 2^(ea - 1022) 2^(eb - 1022) / 256^part_
+      const int sa = ea - 1022 - 70 - 8 * part_;
 #pragma unroll
       for (int j0 = 0; j0 < kEW; j0 += 4) {
         if (kEW * half + j0 < pb) {  // warp-uniform
@@ -284,8 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_wait_ld(v);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int j = kEW * half + j0 + i;
-            const int eb = j < pb ? __ldg(ge + eb0 + b0 + j) : kExpOne;
+            const int eb = __shfl_sync(0xffffffffu, ebl, j0 + i);
             float w[kDiags];
 #pragma unroll
             for (int t = 0; t < kDiags; ++t) w[t] = v[t][i];
@@ -298,22 +383,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive(&acc_empty[r]);
       if (++r == kAS) r = 0, aph ^= 1u;
     }
-    // every group's MMAs done means every copy and tile is done with: lanes 64..127 hand their
-    // sums to lanes 0..63 through the raw ring's memory
+    // every group's MMAs done means every copy and tile is done with: the other parts hand their sums to
+    // part 0 through the raw ring's memory
     const bool done = g == ngroups;
     double* red = reinterpret_cast<double*>(smem);
-    if (odd && done)
+    if (part_ && done)
 #pragma unroll
-      for (int j = 0; j < kEW; ++j) red[(kEW * half + j) * 64 + row] = acc[j];
+      for (int j = 0; j < kEW; ++j) red[((part_ - 1) * NB + kEW * half + j) * CA + row] = acc[j];
     asm volatile("bar.sync 3, 256;\n" ::: "memory");  // the eight epilogue warps
-    if (!odd && row < pa) {
+    if (!part_ && row < pa) {
       const bool ok = done && !abort_flag;
-      double* out = part + (int64_t)blockIdx.x * ta * tb;
+#pragma unroll
+      for (int j = 0; j < kEW; ++j)
+#pragma unroll
+        for (int u = 0; u < 128 / CA - 1; ++u) acc[j] += red[(u * NB + kEW * half + j) * CA + row];
+      double* out = part + (PANEL ? (int64_t)(blockIdx.x / (unsigned)npanels) * n * pb : (int64_t)blockIdx.x * ta * tb);
 #pragma unroll
       for (int j = 0; j < kEW; ++j) {
         const int col = kEW * half + j;
-        if (col < pb && (!upper || a0 + row <= b0 + col))
-          out[(a0 + row) + (int64_t)(b0 + col) * ta] = ok ? acc[j] + red[col * 64 + row] : 0.0;
+        if constexpr (PANEL) {
+          if (col < pb) out[(int64_t)(a0 + row) * pb + col] = ok ? acc[j] : 0.0;
+        } else if (col < pb && (!upper || a0 + row <= b0 + col))
+          out[(a0 + row) + (int64_t)(b0 + col) * ta] = ok ? acc[j] : 0.0;
       }
     }
   } else {
@@ -323,19 +414,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int sw = warp - kSplit0, g = sw / wpg, sg = sw % wpg;
     const int gA = (pa + 31) / 32, gB = same ? 0 : (pb + 31) / 32;
     const int units = (gA + gB) * K8;
-    int src[kMaxUW], ecol[kMaxUW], exp_[kMaxUW];
+    bool fromA[kMaxUW];  // PANEL: a unit of A
+    int src[kMaxUW], ecol[kMaxUW], exp_[kMaxUW], rstep[kMaxUW];  // rstep: doubles between rows
     uint32_t dst[kMaxUW], step[kMaxUW], k0[kMaxUW];
 #pragma unroll
     for (int j = 0; j < kMaxUW; ++j) {
       const int u = sg + j * wpg;
-      src[j] = -1, dst[j] = 0, step[j] = 0, ecol[j] = 0, exp_[j] = kExpOne, k0[j] = 0;
+      fromA[j] = false;
+      src[j] = -1, dst[j] = 0, step[j] = 0, ecol[j] = 0, rstep[j] = ld, exp_[j] = kExpOne, k0[j] = 0;
       if (u < units) {
         const bool isA = u < gA * K8;
         const int v = isA ? u : u - gA * K8;
         const int k8 = v % K8, m = v / K8 * 32 + lane;
         const int off = colofs[isA ? 0 : 1][m];
         if (off >= 0) {
-          src[j] = off + 8 * k8 * ld;
+          if constexpr (PANEL) rstep[j] = B.ld[0], fromA[j] = isA;
+          src[j] = off + 8 * k8 * rstep[j];
           k0[j] = 8 * k8;
           ecol[j] = isA ? a0 + m : eb0 + b0 + m;
           dst[j] = (isA ? 0u : oB) + (uint32_t)(m >> 3) * kSBO + (uint32_t)k8 * kLBO + 16u * (m & 7);
@@ -343,6 +437,24 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
+    // PANEL: the first two units of a warp (the A units are among them) a chunk ahead in registers
+    constexpr int kAhead = PANEL ? 2 : 1;
+    double2 ahead[kAhead][4];
+    auto load_ahead = [&](int c) {
+      if constexpr (PANEL) {
+        const int64_t r0 = r_begin + (int64_t)c * kKC;
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+          if (!fromA[j]) continue;
+          const double* p = A.p[0] + (int64_t)ecol[j] * ld + r0 + k0[j];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            ahead[j][i] = c < nchunks && r0 + k0[j] + 2 * i < r_end ? __ldg(reinterpret_cast<const double2*>(p) + i)
+                                                                    : make_double2(0.0, 0.0);
+        }
+      }
+    };
+    load_ahead(g);
     int st = g % rs, buf = g % kTS, cur = -1;
     uint32_t ph = 0, tph = 0;
     for (int c = g; c < nchunks; c += kSplitGroups) {
@@ -350,42 +462,34 @@ __global__ void __launch_bounds__(kThreads, 1)
         cur = c / kChunks;
 #pragma unroll
         for (int j = 0; j < kMaxUW; ++j)
-          if (src[j] >= 0) exp_[j] = __ldg(exps + (g_begin + cur) * estride + ecol[j]);
+          if (src[j] >= 0) exp_[j] = __ldg(exps + (g_begin + cur) * (int64_t)estride + ecol[j]);
       }
       if (!__all_sync(0xffffffffu, wait_bar(&raw_full[st], ph, &abort_flag, 1))) break;
       if (c >= kTS && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph ^ 1u, &abort_flag, 2))) break;
       const int rows = (int)min((int64_t)kKC, r_end - (r_begin + (int64_t)c * kKC));
-      const double* rsb = raw + (size_t)st * nu * seg;
+      const double* rsb = raw + (size_t)st * stage;
       unsigned char* tb_ = tiles + (uint32_t)buf * tbuf;
 #pragma unroll
       for (int j = 0; j < kMaxUW; ++j) {
         if (src[j] < 0) continue;
         double x[8];
-        if (rows == kKC) {
+        if (PANEL && j < kAhead && fromA[j]) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) x[i] = rsb[src[j] + i * ld];
+          for (int i = 0; i < 4; ++i) x[2 * i] = ahead[j < kAhead ? j : 0][i].x, x[2 * i + 1] = ahead[j < kAhead ? j : 0][i].y;
+        } else if (rows == kKC) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[i] = rsb[src[j] + i * rstep[j]];
         } else {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) x[i] = (int)k0[j] + i < rows ? rsb[src[j] + i * ld] : 0.0;
+          for (int i = 0; i < 8; ++i) x[i] = (int)k0[j] + i < rows ? rsb[src[j] + i * rstep[j]] : 0.0;
         }
         uint64_t w[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = digits(x[i], exp_[j]);
         unsigned char* o = tb_ + dst[j];
-        auto put = [&](auto k) {
-          constexpr int K = decltype(k)::value;
-          *reinterpret_cast<uint4*>(o + K * step[j]) =
-              make_uint4(digit_pair<K>(w[0], w[1]), digit_pair<K>(w[2], w[3]), digit_pair<K>(w[4], w[5]),
-                         digit_pair<K>(w[6], w[7]));
-        };
-        put(std::integral_constant<int, 0>{});
-        put(std::integral_constant<int, 1>{});
-        put(std::integral_constant<int, 2>{});
-        put(std::integral_constant<int, 3>{});
-        put(std::integral_constant<int, 4>{});
-        put(std::integral_constant<int, 5>{});
-        put(std::integral_constant<int, 6>{});
+        put_digits(w, o, step[j]);
       }
+      load_ahead(c + kSplitGroups);
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) {
@@ -442,17 +546,17 @@ int sm_count() {
   return sms;
 }
 
-template <int NB>
+template <int CA, int NB>
 void gram64_launch(int64_t n, const Cols<double>& a, const Cols<double>& b, int ld, int a0, int pa, int b0, int pb,
                    bool upper, bool same, int rs, size_t smem, const int* exps, int estride, int eb0,
                    const int* flag, double* part, int ctas, int64_t gpc, cudaStream_t st) {
   static const bool attr = [&] {
-    LB_CUDA(cudaFuncSetAttribute(gram64_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget));
+    LB_CUDA(cudaFuncSetAttribute(gram64_kernel<CA, NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget));
     return true;
   }();
   (void)attr;
-  gram64_kernel<NB><<<(unsigned)ctas, kThreads, smem, st>>>(n, a, b, ld, a0, pa, b0, pb, upper ? 1 : 0, same ? 1 : 0,
-                                                           rs, exps, estride, eb0, flag, part, gpc);
+  gram64_kernel<CA, NB, false><<<(unsigned)ctas, kThreads, smem, st>>>(n, a, b, ld, a0, pa, b0, pb, upper ? 1 : 0, same ? 1 : 0,
+                                                           rs, exps, estride, eb0, flag, part, gpc, 0);
   LB_LAUNCH_CHECK();
 }
 
@@ -480,13 +584,13 @@ int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b
   const bool same = same_cols(a, b);
   const int na = (pa + kCB - 1) / kCB, nb = (pb + kCB - 1) / kCB;  // column blocks, of equal widths
   const int wa = (pa + na - 1) / na, wb = (pb + nb - 1) / nb;
-  const int nbw = wb <= 32 ? 32 : 64;
+  const int nbw = wb <= 32 ? 32 : 64, caw = wa <= 32 && wb <= 32 ? 32 : 64;  // columns of B and A slices
   const size_t stage = (size_t)kKC * count_blocks(a, b) * ld * 8;
-  const size_t tiles = (size_t)kTS * (8 * kSliceA + kSlices * (size_t)(nbw / 8) * kSBO);
+  const size_t tiles = (size_t)kTS * (8 * (size_t)(caw / 8) + kSlices * (size_t)(nbw / 8)) * kSBO;
   if (tiles + 2 * stage + 128 > kSmemBudget) return 0;
   const int rs = (int)std::min<size_t>(kMaxRS, (kSmemBudget - tiles - 128) / stage);
   // the raw ring also holds the epilogue's exchange
-  const size_t smem = std::max((rs * stage + 127) / 128 * 128, (size_t)64 * nbw * 8) + tiles;
+  const size_t smem = std::max((rs * stage + 127) / 128 * 128, (size_t)(128 - caw) * nbw * 8) + tiles;
   if (smem > kSmemBudget) return 0;
   const int64_t ngroups = ceil_div(n, kGroupRows);
   int64_t ctas = std::min<int64_t>(std::min<int64_t>(max_ctas, sm_count()), ngroups);
@@ -504,15 +608,93 @@ int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b
       const int ca = std::min(wa, pa - a0), cb = std::min(wb, pb - b0);
       if (upper && a0 > b0 + cb - 1) continue;
       // B can read A's tiles where its slices have A's width
-      const bool diag = same && ia == ib && nbw == kCB;
-      if (nbw == 32)
-        gram64_launch<32>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
+      const bool diag = same && ia == ib && nbw == caw;
+      if (caw == 32)
+        gram64_launch<32, 32>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
+                              (int)ctas, gpc, st);
+      else if (nbw == 32)
+        gram64_launch<64, 32>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
                           (int)ctas, gpc, st);
       else
-        gram64_launch<64>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
+        gram64_launch<64, 64>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
                           (int)ctas, gpc, st);
     }
   return (int)ctas;
+}
+
+namespace {
+// Y[i][j] = sum over the splits, in order
+__global__ void panel_reduce_kernel(int64_t n, int p, int splits, const double* __restrict__ part, double* __restrict__ Y,
+                                    int ldy, const int* __restrict__ flag) {
+  if (*flag) return;  // no sums were written
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * p; e += (int64_t)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int g = 0; g < splits; ++g) s += part[g * n * p + e];
+    Y[e / p * ldy + e % p] = s;
+  }
+}
+
+constexpr int kMaxSplits = 8;
+// Row ranges per panel: the count that fills whole waves of the SMs best (fewer where equal: every
+// range pays the kernel's start).
+int panel_splits(int64_t panels, int64_t groups, int sms) {
+  int best = 1;
+  double cost = 1e300;
+  for (int k = 1; k <= kMaxSplits && k <= groups; ++k) {
+    const int64_t per = ceil_div(groups, k), used = ceil_div(groups, per);
+    // waves x (groups of a range + the start, about the time of two groups)
+    const double c = (double)ceil_div(panels * used, sms) * ((double)per + 2.0);
+    if (c < cost * 0.98) cost = c, best = (int)used;
+  }
+  return best;
+}
+}  // namespace
+
+// Scratch of launch_spmm_dense_digits in bytes: flag, exponents, partial sums.
+size_t dense64_scratch_bytes(int64_t n, int p) {
+  const size_t exps = ((size_t)ceil_div(n, kGroupRows) * (n + p) * sizeof(int) + 255) / 256 * 256;
+  return 256 + exps + (size_t)kMaxSplits * n * p * sizeof(double);
+}
+
+// Y = A X (column i of the dense column-major A against X) through digit products; false without
+// launching where A or X do not fit (odd n or lda, unaligned).  *scratch is the flag left at 1 when a
+// number is outside the digits' range: Y is then to be formed by launch_spmm_dense on that flag.
+bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
+                              int ldy, void* scratch, cudaStream_t st) {
+  if (n < 2 || (n & 1) || (lda & 1) || lda > INT_MAX || p < 1 || p > 32 || (reinterpret_cast<uintptr_t>(A) & 15) ||
+      (reinterpret_cast<uintptr_t>(X) & 15))
+    return false;
+  constexpr int NB = 32;
+  const size_t stage = (size_t)kKC * ldx * 8;
+  const size_t tiles = (size_t)kTS * (8 * (size_t)(kCB / 8) + kSlices * (size_t)(NB / 8)) * kSBO;
+  if (tiles + 2 * stage + 128 > kSmemBudget) return false;
+  const int rs = (int)std::min<size_t>(kMaxRS, (kSmemBudget - tiles - 128) / stage);
+  const size_t smem = std::max((rs * stage + 127) / 128 * 128, (size_t)64 * NB * 8) + tiles;
+  static const bool attr = [&] {
+    LB_CUDA(cudaFuncSetAttribute(gram64_kernel<kCB, NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget));
+    return true;
+  }();
+  (void)attr;
+  const int64_t groups = ceil_div(n, kGroupRows), panels = ceil_div(n, kCB);
+  const int splits = panel_splits(panels, groups, sm_count());
+  int* flag = static_cast<int*>(scratch);
+  int* exps = flag + 64;
+  const int64_t estride = n + p;
+  double* part = reinterpret_cast<double*>(static_cast<char*>(scratch) + 256 +
+                                           ((size_t)groups * estride * sizeof(int) + 255) / 256 * 256);
+  LB_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
+  exp_dense_kernel<<<dim3((unsigned)ceil_div(n, 8), (unsigned)groups), 256, 0, st>>>(n, A, lda, exps, estride, flag);
+  LB_LAUNCH_CHECK();
+  exp_rows_kernel<<<(unsigned)groups, 256, 0, st>>>(n, p, X, ldx, exps + n, estride, flag);
+  LB_LAUNCH_CHECK();
+  gram64_kernel<kCB, NB, true><<<(unsigned)(panels * splits), kThreads, smem, st>>>(
+      n, cols1<double>(A, (int)lda, 1), cols1<double>(X, ldx, p), (int)lda, 0, 0, 0, p, 0, 0, rs, exps, (int)estride,
+      (int)n, flag, part, ceil_div(groups, splits), (int)panels);
+  LB_LAUNCH_CHECK();
+  panel_reduce_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n * p, 256), 4096), 256, 0, st>>>(n, p, splits, part, Y,
+                                                                                               ldy, flag);
+  LB_LAUNCH_CHECK();
+  return true;
 }
 
 // Reads and clears the give-up flag (synchronises the stream); throws when a CTA gave up waiting.

@@ -41,32 +41,49 @@ __device__ __forceinline__ int group_exp(uint32_t key) {
 // (a leading digit of 128 carries into the top byte).
 __device__ __forceinline__ uint64_t digits(double x, int E) {
   const uint32_t hw = (uint32_t)__double2hiint(x), lw = (uint32_t)__double2loint(x);
-  const int e = (int)((hw >> 20) & 0x7ffu);
-  const int k = min(E - e, 63);  // >= 0; zeros and subnormals shift out (E >= kExpMin)
+  const uint32_t k = (uint32_t)(E - (int)((hw >> 20) & 0x7ffu));  // >= 0
   const uint64_t m = (uint64_t)((hw & 0xfffffu) | 0x100000u) << 32 | lw;
-  const uint64_t t = (((m << 3) >> k) + 1u) >> 1;
+  uint64_t t;  // 2 |X|, cut; shr clamps, so zeros and subnormals shift out (E >= kExpMin)
+  asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(m << 3), "r"(k));
   const uint64_t neg = (uint64_t)(int64_t)((int32_t)hw >> 31);
-  return (t ^ neg) + (0x6480808080808080ull - neg);
+  // X + bias = (t + 1 + 2 bias) / 2, or (-t + 2 bias) / 2 with -t = ~t + 1: rounding, sign and bias in one
+  // addition
+  return ((t ^ neg) + 0xc901010101010101ull) >> 1;
 }
 
-// The digits k of two numbers (a in the low half) as FP16.
-template <int K>
-__device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
-  constexpr uint32_t kByte = (uint32_t)(6 - K);
-  uint32_t r;
-  if constexpr (K == 0) {
-    // bytes 7 and 6 are 0x64 (0x65 where the leading digit is 128) and the digit: 1024 + d_0 + 128
-    r = __byte_perm((uint32_t)(a >> 32), (uint32_t)(b >> 32), 0x7632u);
-  } else {
-    constexpr uint32_t i = kByte & 3u;
-    constexpr int kShift = kByte >= 4 ? 32 : 0;
-    r = __byte_perm((uint32_t)(a >> kShift), (uint32_t)(b >> kShift), i | i << 4 | (4u + i) << 8 | (4u + i) << 12);
-    r = (r & 0x00ff00ffu) | 0x64006400u;
-  }
-  // (1024 + byte) - 1152 = byte - 128, exact
+// (1024 + byte) - 1152 = byte - 128 in both halves, exact.
+__device__ __forceinline__ uint32_t unbias(uint32_t r) {
   __half2 h = *reinterpret_cast<__half2*>(&r);
   h = __hsub2(h, __half2half2(__ushort_as_half(0x6480)));
   return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// d[k]: the digits k of two numbers (a in the low half) as FP16.  A byte permute gathers two
+// neighbouring digits of both numbers, a second one per digit sets 0x64 above each (1024 + byte).
+__device__ __forceinline__ void digit_pairs(uint64_t a, uint64_t b, uint32_t (&d)[kSlices]) {
+  constexpr uint32_t c = 0x64646464u;
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+  // bytes 7 and 6 are 0x64 (0x65 where the leading digit is 128) and the digit already
+  d[0] = unbias(__byte_perm(ah, bh, 0x7632));
+  uint32_t q = __byte_perm(ah, bh, 0x5410);  // bytes 4, 5 of a, then of b
+  d[1] = unbias(__byte_perm(q, c, 0x4341));
+  d[2] = unbias(__byte_perm(q, c, 0x4240));
+  q = __byte_perm(al, bl, 0x7632);  // bytes 2, 3
+  d[3] = unbias(__byte_perm(q, c, 0x4341));
+  d[4] = unbias(__byte_perm(q, c, 0x4240));
+  q = __byte_perm(al, bl, 0x5410);  // bytes 0, 1
+  d[5] = unbias(__byte_perm(q, c, 0x4341));
+  d[6] = unbias(__byte_perm(q, c, 0x4240));
+}
+
+// The digits of eight numbers, 16 bytes per digit, `step` bytes apart at o.
+__device__ __forceinline__ void put_digits(const uint64_t (&w)[8], unsigned char* o, uint32_t step) {
+  uint32_t d[4][kSlices];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) digit_pairs(w[2 * i], w[2 * i + 1], d[i]);
+#pragma unroll
+  for (int k = 0; k < kSlices; ++k)
+    *reinterpret_cast<uint4*>(o + k * step) = make_uint4(d[0][k], d[1][k], d[2][k], d[3][k]);
 }
 
 // sum_t v_t 256^(7-t) of eight whole FP32 numbers |v_t| <= 2^24, times 2^s, rounded to FP64 with

@@ -401,6 +401,7 @@ struct lobpcg_ctx {
     }
     return gram_ints;
   }
+  DevBuf dense_buf;  // exponents and partial sums of the dense digit product
   double* host = nullptr;  // pinned readback area
   Stats stats;
   Profiler prof;
@@ -491,6 +492,7 @@ struct Prec<float> {
 
 // Multiply-adds from which the digit products win over FP64 FMAs and over double-float.
 constexpr double kDigitGram = 2e7, kDigitGramDf = 6e7;
+constexpr double kDigitDense = 3e7;
 constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7;
 
 // launch_update with, in profile mode, the FP64 launches timed and their flops counted.
@@ -520,6 +522,9 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   return parts;
 }
 
+// Whether the dense FP64 product is the faster form through digit products.
+bool dense_digits_pay(int64_t n, int p) { return (double)n * n * p >= kDigitDense; }
+
 // Y = A X with the product kernel chosen for this precision (no statistics).
 template <class T>
 void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
@@ -529,8 +534,19 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
   else if (c.A.fmt == LOBPCG_CSR)
     launch_spmm_csr<T, T>(c.A.n, c.A.row_ptr, c.A.col_idx, Prec<T>::val(c), p, X, ldx, Y, ldy, c.st, c.band,
                           false, var);
-  else
+  else {
+    if constexpr (std::is_same<T, double>::value) {
+      if (dense_digits_pay(c.A.n, p)) {
+        c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
+        if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, c.st)) {
+          c.used_digits = true;
+          launch_spmm_dense<T>(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.st, c.dense_buf.as<int>());
+          return;
+        }
+      }
+    }
     launch_spmm_dense<T>(c.A.n, Prec<T>::dense(c), Prec<T>::lda(c), p, X, ldx, Y, ldy, c.st);
+  }
 }
 
 // Autotuner of the CSR product: on the first solve with block width p, time every kernel
@@ -1539,6 +1555,7 @@ extern "C" void lobpcg_destroy(lobpcg_ctx* c) {
   c->tri_offd.release();
   c->tri_scratch.release();
   c->gram_buf.release();
+  c->dense_buf.release();
   c->mlp_params.release();
   c->rho.release();
   if (c->host) cudaFreeHost(c->host);
@@ -1688,6 +1705,15 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
     require(n >= 0 && A && X && Y && lda >= n, "lobpcg_spmm_dense_f64: NULL argument or lda < n");
     require(p >= 1 && p <= 32 && ldx >= p && ldy >= p, "lobpcg_spmm_dense_f64: need 1 <= p <= 32, ld >= p");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    PoolBuf work(st);
+    if (dense_digits_pay(n, p)) {
+      work.alloc(dense64_scratch_bytes(n, p));
+      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, st)) {
+        launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st, work.as<int>());
+        gram64_check(st);
+        return LOBPCG_OK;
+      }
+    }
     launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st);
     LB_CUDA(cudaStreamSynchronize(st));
     return LOBPCG_OK;
@@ -1961,6 +1987,7 @@ extern "C" lobpcg_status lobpcg_solve_batched(lobpcg_ctx* const* ctxs, int nprob
       ctxs[i]->xbest.release();
       ctxs[i]->gram_buf.release();
       ctxs[i]->gram_ints = nullptr;
+      ctxs[i]->dense_buf.release();
     }
   };
   std::vector<std::thread> pool;

@@ -1181,7 +1181,9 @@ constexpr int kDenseSlab = 128;
 template <class T, int RB, int PC>
 __global__ void __launch_bounds__(256) spmm_dense_kernel(int64_t n, const T* __restrict__ A, int64_t lda, int p,
                                                          int c0, const T* __restrict__ X, int ldx,
-                                                         T* __restrict__ Y, int ldy) {
+                                                         T* __restrict__ Y, int ldy,
+                                                         const int* __restrict__ run_flag) {
+  if (run_flag && *run_flag == 0) return;
   // 16-byte reads at a row stride of 4 (mod 8) words (PC >= 16 bytes; narrower rows are read
   // element by element)
   constexpr int XS = sizeof(T) == 8 ? PC + 2 : PC + 4;
@@ -1313,7 +1315,7 @@ void launch_spmm_csr(int64_t n, const int64_t* rp, const int32_t* ci, const V* v
 
 template <class T>
 void launch_spmm_dense(int64_t n, const T* A, int64_t lda, int p, const T* X, int ldx, T* Y,
-                       int ldy, cudaStream_t st) {
+                       int ldy, cudaStream_t st, const int* run_flag) {
   if (n <= 0 || p <= 0) return;
   // one pass over A for p <= 32 columns: RB x PC = 32 accumulators per thread
   const int threads = 256;
@@ -1321,16 +1323,16 @@ void launch_spmm_dense(int64_t n, const T* A, int64_t lda, int p, const T* X, in
   // narrowest width that holds p
   const unsigned g32 = (unsigned)ceil_div(n, 32);
   if (p <= 2) {
-    spmm_dense_kernel<T, 4, 2><<<g32, threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy);
+    spmm_dense_kernel<T, 4, 2><<<g32, threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy, run_flag);
   } else if (p <= 4) {
-    spmm_dense_kernel<T, 4, 4><<<g32, threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy);
+    spmm_dense_kernel<T, 4, 4><<<g32, threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy, run_flag);
   } else if (p <= 8) {
-    spmm_dense_kernel<T, 4, 8><<<g32, threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy);
+    spmm_dense_kernel<T, 4, 8><<<g32, threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy, run_flag);
   } else if (p <= 16) {
-    spmm_dense_kernel<T, 2, 16><<<(unsigned)ceil_div(n, 16), threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy);
+    spmm_dense_kernel<T, 2, 16><<<(unsigned)ceil_div(n, 16), threads, 0, st>>>(n, A, lda, p, 0, X, ldx, Y, ldy, run_flag);
   } else {
     for (int c0 = 0; c0 < p; c0 += 32)
-      spmm_dense_kernel<T, 1, 32><<<(unsigned)ceil_div(n, 8), threads, 0, st>>>(n, A, lda, p, c0, X, ldx, Y, ldy);
+      spmm_dense_kernel<T, 1, 32><<<(unsigned)ceil_div(n, 8), threads, 0, st>>>(n, A, lda, p, c0, X, ldx, Y, ldy, run_flag);
   }
   LB_LAUNCH_CHECK();
 }
@@ -1441,9 +1443,9 @@ int profile_band(int64_t n, const int64_t* rp, const int32_t* ci, int64_t nnz, c
   return -1;
 }
 template void launch_spmm_dense<double>(int64_t, const double*, int64_t, int, const double*, int,
-                                        double*, int, cudaStream_t);
+                                        double*, int, cudaStream_t, const int*);
 template void launch_spmm_dense<float>(int64_t, const float*, int64_t, int, const float*, int,
-                                       float*, int, cudaStream_t);
+                                       float*, int, cudaStream_t, const int*);
 
 void launch_split_df(int64_t count, const double* src, float2* dst, cudaStream_t st) {
   if (count <= 0) return;

@@ -22,14 +22,13 @@
 //     columns 32 (i + j), ..: region t of an accumulator sums the products with i + j = t, at most
 //     7 * 96 * 2^14 < 2^24, exact.
 //   * warps 16..23, epilogue: two threads per row, which take the groups of four columns in turn.  The
-//     eight regions of an element are joined into FP64 with integer operations, the base is added, and
-//     the residuals of the four columns are handed through shared memory to one warp per column, which
-//     keeps their squares' sum and maximum.
+//     eight regions of an element are joined into FP64 with integer operations and turned inside the warp
+//     to four lanes per row, which add the base, store 32-byte pieces of rows and, from the pair's two
+//     elements, keep the sum of squares and the maximum of the residuals of their column.
 // Rows with an infinity, a NaN or an exponent outside 2^+-400 (and all rows when U has one) are
 // formed by their epilogue thread with FP64 FMAs.
 #include <algorithm>
 #include <climits>
-#include <type_traits>
 
 #include "common.cuh"
 #include "slices.cuh"
@@ -52,7 +51,7 @@ constexpr uint32_t kLBO = 128, kSBO = kKC / 8 * 128;
 constexpr uint32_t kSlice = kTile / 8 * kSBO;  // bytes of one digit of a chunk of V
 constexpr uint32_t kBuf = kSlices * kSlice;
 constexpr int kAcc = kDiags * kQ;              // TMEM columns of one accumulator
-constexpr int kBad = INT_MIN;
+constexpr int kBad = -1;
 constexpr long long kWaitCycles = 1ll << 31;
 constexpr size_t kStatic = 14 * 1024;  // static shared memory, at most
 constexpr size_t kSmemBudget = 227 * 1024;
@@ -86,11 +85,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr uint32_t kSliceU = u_slice(KP), kSBOU = KP / 8 * 128;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t raw_full[kSplitWarps], tile_full[kMaxTS], tile_empty[kMaxTS], acc_full[2], acc_empty[2], exp_full[kRing];
-  __shared__ int row_exp[kRing][kTile];
+  __shared__ int16_t row_exp[kRing][kTile];
   __shared__ int col_exp[kQ];
   __shared__ __align__(16) int16_t up[KP];  // exponent of row l of U: V's column l is scaled by 2^up
-  __shared__ double res[2][NORM ? 4 : 1][NORM ? kTile : 1];
+  __shared__ double nred[2][kEpiWarps][NORM ? kQ / 2 : 1];  // a warp's sums and maxima of its columns
   __shared__ double lam_s[kQ];
+  __shared__ double stage[kEpiWarps][32][4];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   __shared__ int u_bad;
@@ -145,14 +145,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // digits() takes the exponent in the entry's own scale; entries far below their column shift out
     const uint64_t w = up[l] > -4000 ? digits(us[e], col_exp[j] + up[l]) : digits(0.0, kExpOne);
     unsigned char* o = udig + (uint32_t)(j >> 3) * kSBOU + (uint32_t)(l >> 3) * kLBO + 16u * (j & 7) + 2u * (l & 7);
-    auto put = [&](auto k) {
-      constexpr int K = decltype(k)::value;
-      *reinterpret_cast<uint16_t*>(o + K * kSliceU) = (uint16_t)digit_pair<K>(w, w);
-    };
-    put(std::integral_constant<int, 0>{}), put(std::integral_constant<int, 1>{});
-    put(std::integral_constant<int, 2>{}), put(std::integral_constant<int, 3>{});
-    put(std::integral_constant<int, 4>{}), put(std::integral_constant<int, 5>{});
-    put(std::integral_constant<int, 6>{});
+    uint32_t d[kSlices];
+    digit_pairs(w, w, d);
+#pragma unroll
+    for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint16_t*>(o + k * kSliceU) = (uint16_t)d[k];
   }
   __syncwarp();
   if (warp == kMma) tmem_alloc(&tmem_slot, 2 * kAcc);
@@ -238,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; c < NC; ++c) {
         if (chunk >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph, &abort_flag, 2))) break;
         if (c == 0) {
-          if (lane < 8) row_exp[T & (kRing - 1)][8 * warp + lane] = bad ? kBad : E;
+          if (lane < 8) row_exp[T & (kRing - 1)][8 * warp + lane] = (int16_t)(bad ? kBad : E);
           __syncwarp();
           if (lane == 0) mbar_arrive(&exp_full[T & (kRing - 1)]);
         }
@@ -252,16 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           w[i] = digits(bad ? 0.0 : x[c][i], v > -4000 ? E - v : 4 * kExpOne);
         }
         unsigned char* o = tiles + (uint32_t)buf * kBuf + (uint32_t)warp * kSBO + (uint32_t)k8 * kLBO + 16u * r;
-        auto put = [&](auto k) {
-          constexpr int K = decltype(k)::value;
-          *reinterpret_cast<uint4*>(o + K * kSlice) =
-              make_uint4(digit_pair<K>(w[0], w[1]), digit_pair<K>(w[2], w[3]), digit_pair<K>(w[4], w[5]),
-                         digit_pair<K>(w[6], w[7]));
-        };
-        put(std::integral_constant<int, 0>{}), put(std::integral_constant<int, 1>{});
-        put(std::integral_constant<int, 2>{}), put(std::integral_constant<int, 3>{});
-        put(std::integral_constant<int, 4>{}), put(std::integral_constant<int, 5>{});
-        put(std::integral_constant<int, 6>{});
+        put_digits(w, o, kSlice);
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tile_full[buf]);
@@ -336,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         if (t >= nprod || !live || er[t] != kBad) continue;
-        for (int j = 0; j < q; ++j) slow[t][j] = 0.0;
+        for (int j = 0; j < kQ; ++j) slow[t][j] = 0.0;
         int l = 0;
         for (int g = 0; g < nseg; ++g)
           for (int i = 0; i < job.in[t].w[g]; ++i, ++l) {
@@ -344,13 +331,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int j = 0; j < q; ++j) slow[t][j] = fma(v, alpha * U[l + j * s], slow[t][j]);
           }
       }
+      int se[2];  // element: (sum_t v_t 256^(7-t)) 2^(40 - 110) 2^(er - 1022) 2^(col_exp - 1022)
+#pragma unroll
+      for (int t = 0; t < 2; ++t) se[t] = (er[t] == kBad ? kExpOne : er[t]) - 2 * 1022 - 70;
+      // rows of this warp
+      const int64_t row0 = r_begin + (int64_t)it * kTile + 32 * quad;
+      const int nrows = (int)max((int64_t)0, min((int64_t)32, r_end - row0));
       // both threads of a row have read it before either stores
-      if (__any_sync(0xffffffffu, er[0] == kBad || er[1] == kBad)) asm volatile("bar.sync %0, 64;\n" ::"r"(5 + quad) : "memory");
+      const bool any_bad = __any_sync(0xffffffffu, er[0] == kBad || er[1] == kBad);
+      if (any_bad) asm volatile("bar.sync %0, 64;\n" ::"r"(5 + quad) : "memory");
 #pragma unroll
       for (int gh = 0; gh < kQ / 8; ++gh) {
         const int g = 2 * gh + half;
         if (4 * g >= q) break;
-        double o[2][4];
+        double xs[4];  // NORM: the pair's X elements of this lane's rows and column
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           if (t >= nprod) break;
@@ -360,43 +354,48 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int d = 0; d < kDiags; ++d)
             tmem_ld4(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(a * kAcc + kQ * d + 4 * g), v[d]);
           tmem_wait_ld(v);
-          const double* b = job.base[t] && live ? job.base[t] + grow * job.ld_base[t] : nullptr;
+          double o[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int j = 4 * g + i;
             float w[kDiags];
 #pragma unroll
             for (int d = 0; d < kDiags; ++d) w[d] = v[d][i];
-            o[t][i] = er[t] == kBad ? (j < q ? slow[t][j] : 0.0) : join(w, er[t] - 1022 + col_exp[j] - 1022 - 70);
-            if (b && j < q) o[t][i] = b[j] + o[t][i];
+            o[i] = join(w, se[t] + col_exp[j]);
           }
-          if (live) {
-            double* p = job.out[t] + grow * job.ld_out[t] + 4 * g;
-            if (4 * g + 4 <= q && !(job.ld_out[t] & 1) && !(reinterpret_cast<uintptr_t>(job.out[t]) & 15)) {
-              reinterpret_cast<double2*>(p)[0] = make_double2(o[t][0], o[t][1]);
-              reinterpret_cast<double2*>(p)[1] = make_double2(o[t][2], o[t][3]);
-            } else {
+          if (any_bad && er[t] == kBad)
 #pragma unroll
-              for (int i = 0; i < 4; ++i)
-                if (4 * g + i < q) p[i] = o[t][i];
+            for (int i = 0; i < 4; ++i) o[i] = slow[t][4 * g + i];
+          // to the warp's stage (columns turned by row / 4: no bank conflicts either way), then four lanes per
+          // row: whole 32-byte pieces of eight rows a store
+#pragma unroll
+          for (int i = 0; i < 4; ++i) stage[warp - kEpi0][lane][(i + (lane >> 2)) & 3] = o[i];
+          __syncwarp();
+          const int j = 4 * g + (lane & 3);
+          double* out = job.out[t] + (row0 + (lane >> 2)) * job.ld_out[t] + j;
+          const double* base = NORM || !job.base[t] ? nullptr : job.base[t] + (row0 + (lane >> 2)) * job.ld_base[t] + j;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int rr = 8 * k + (lane >> 2);
+            double x = stage[warp - kEpi0][rr][((lane & 3) + (rr >> 2)) & 3];
+            const bool mine = rr < nrows && j < q;
+            if (mine) {
+              if (!NORM && base) x = base[(int64_t)(8 * k) * job.ld_base[t]] + x;
+              out[(int64_t)(8 * k) * job.ld_out[t]] = x;
+            }
+            if constexpr (NORM) {
+              if (t == 0) {
+                xs[k] = x;
+              } else if (mine) {
+                const double res = fma(-lam_s[j], xs[k], x);  // AX - lam X, one rounding
+                nsum[gh] = fma(res, res, nsum[gh]);
+                // max of magnitudes by their bits (a NaN does not count, as in fmax)
+                const long long ax = __double_as_longlong(res) & 0x7fffffffffffffffll;
+                if (ax > __double_as_longlong(nmax[gh]) && ax <= 0x7ff0000000000000ll) nmax[gh] = __longlong_as_double(ax);
+              }
             }
           }
-        }
-        if constexpr (NORM) {
-          // residuals AX - lam X of the four columns; warp `quad` of this half then takes column 4 g + quad
-          asm volatile("bar.sync %0, 128;\n" ::"r"(3 + half) : "memory");  // the previous group is read
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            res[half][i][row] = live && 4 * g + i < q ? fma(-lam_s[4 * g + i], o[0][i], o[1][i]) : 0.0;
-          asm volatile("bar.sync %0, 128;\n" ::"r"(3 + half) : "memory");
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const double x = res[half][quad][32 * u + lane];
-            nsum[gh] = fma(x, x, nsum[gh]);
-            // max of magnitudes by their bits (a NaN does not count, as in fmax)
-            const long long ax = __double_as_longlong(x) & 0x7fffffffffffffffll;
-            if (ax > __double_as_longlong(nmax[gh]) && ax <= 0x7ff0000000000000ll) nmax[gh] = __longlong_as_double(ax);
-          }
+          __syncwarp();
         }
       }
       tc_fence_before();
@@ -406,14 +405,25 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (t < nprod && lane == 0) mbar_arrive(&acc_empty[(it * nprod + t) & 1]);
     }
     if constexpr (NORM) {
+      // lanes of one column, then the four warps of one half, in a fixed order
 #pragma unroll
       for (int gh = 0; gh < kQ / 8; ++gh) {
-        const double s2 = warp_sum(nsum[gh]), mx = warp_max(nmax[gh]);
-        const int j = 4 * (2 * gh + half) + quad;
-        if (lane == 0 && j < q) {
-          norm_part[(int64_t)blockIdx.x * 2 * q + j] = s2;
-          norm_part[(int64_t)blockIdx.x * 2 * q + q + j] = mx;
+        double s2 = nsum[gh], mx = nmax[gh];
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+          mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         }
+        if (lane < 4) nred[0][warp - kEpi0][4 * gh + lane] = s2, nred[1][warp - kEpi0][4 * gh + lane] = mx;
+      }
+      asm volatile("bar.sync 3, 256;\n" ::: "memory");  // the eight epilogue warps
+      const int j = tid - 32 * kEpi0;
+      if (j < q) {
+        const int h = (j >> 2) & 1, c = 4 * (j >> 3) + (j & 3);  // half and column within it
+        double s2 = 0.0, mx = 0.0;
+        for (int u = 0; u < 4; ++u) s2 += nred[0][4 * h + u][c], mx = fmax(mx, nred[1][4 * h + u][c]);
+        norm_part[(int64_t)blockIdx.x * 2 * q + j] = s2;
+        norm_part[(int64_t)blockIdx.x * 2 * q + q + j] = mx;
       }
     }
   }
