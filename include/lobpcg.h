@@ -301,6 +301,13 @@ LOBPCG_API lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
                                     const double* X, int ldx, double* Y, int ldy,
                                     lobpcg_stream stream);
 
+/* The same product (column i of A against X) of a row-major A, read in place.  *done (host) is 0, and Y not
+ * written, where this form does not apply: fewer than 1.5e7 multiply-adds, odd n or lda, A or X not 16-byte
+ * aligned, or a number that is infinite, NaN or outside about 2^+-400 (zeros apart); pass the
+ * column-major matrix to lobpcg_spmm_dense_f64 then. */
+LOBPCG_API lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, int64_t lda, int p, const double* X,
+                                                    int ldx, double* Y, int ldy, int* done, lobpcg_stream stream);
+
 /* C = X^T Y (the Gram / projected matrices of Algorithm 1 and Eq. (CDOrtho)).
  * X: n x p (ldx), Y: n x q (ldy), p, q <= 96.  C: device, column-major p x q. */
 LOBPCG_API lobpcg_status lobpcg_gram_f64(int64_t n, int p, const double* X, int ldx, int q, const double* Y,

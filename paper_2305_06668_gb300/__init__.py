@@ -79,7 +79,8 @@ def lib():
                      "lobpcg_spmm_csr_f32", "lobpcg_syev2_f64", "lobpcg_gram_f32", "lobpcg_update_f32",
                      "lobpcg_probe_fma_rate", "lobpcg_gram_f64_df", "lobpcg_update_f64_df",
                      "lobpcg_spmm_csr_f64_df", "lobpcg_gram_f32_tcgen05", "lobpcg_precond_tridiag",
-                     "lobpcg_mixed_switch_replay", "lobpcg_trim_workspace"):
+                     "lobpcg_mixed_switch_replay", "lobpcg_trim_workspace",
+                     "lobpcg_spmm_dense_rows_f64"):
             getattr(L, name).restype = C.c_int
         L.lobpcg_last_error.restype = C.c_char_p
         L.lobpcg_last_error.argtypes = [C.c_void_p]
@@ -299,6 +300,13 @@ def spmm_dense(A, X, stream=None):
     torch = _torch()
     n, p = X.shape
     Y = torch.empty_like(X)
+    if A.is_contiguous() and not A.t().is_contiguous():  # row-major storage, read in place where that applies
+        done = C.c_int(0)
+        _check(lib().lobpcg_spmm_dense_rows_f64(C.c_int64(n), _ptr(A), C.c_int64(n), C.c_int(p), _ptr(X),
+                                                C.c_int(X.stride(0)), _ptr(Y), C.c_int(Y.stride(0)), C.byref(done),
+                                                _stream(stream)))
+        if done.value:
+            return Y
     At = A if A.t().is_contiguous() else A.t().contiguous().t()  # column-major storage
     _check(lib().lobpcg_spmm_dense_f64(C.c_int64(n), _ptr(At), C.c_int64(n), C.c_int(p), _ptr(X),
                                        C.c_int(X.stride(0)), _ptr(Y), C.c_int(Y.stride(0)), _stream(stream)))

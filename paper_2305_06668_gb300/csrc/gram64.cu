@@ -26,9 +26,11 @@
 //     with integer operations and adds it to its running sum (one FP64 add).
 // The dense symmetric product Y = A X (PANEL) is the same contraction with A's columns in memory order:
 // a CTA owns 64 columns of A and a range of its rows and writes its 64 x p sums; ranges of rows split a
-// matrix of few panels over the SMs.  The splitters load A from global memory straight into registers, a
-// chunk ahead (a lane's 8 rows of a column are 64 contiguous bytes): 256-byte bulk copies of the columns
-// took 70 clocks each, 4.5k per chunk, and made a product of n = 8192 wait on them for 0.45 of 0.6 ms.
+// matrix of few panels over the SMs.  The producer warp copies 32 rows of each column with cp.async, half a
+// warp per column (256 bytes, at a 272-byte stride in shared memory, which keeps the splitters' reads of 8
+// columns in different banks), as far ahead as the raw ring holds.  256-byte bulk copies took 70 clocks
+// each, 4.5k per chunk (1078 us a product of n = 8192), loads by the splitters a chunk ahead left 16 KB in
+// flight (899 us).  A row-major A (row_a) is copied by rows of 64 columns; it needs no transposed copy.
 //
 // A flag set by exp_kernel (a column's block with an infinity, a NaN or an exponent outside
 // 2^+-400) makes gram64_kernel return at once; the caller's general kernel, launched behind it on
@@ -74,6 +76,14 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
   *abort_flag = 1;
   atomicExch(&g_gram64_err, code);
   return false;
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+// Arrive on the barrier when this thread's cp.async copies so far have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
 }
 
 // exps[g * stride + j]: biased exponent of column j (A's columns, then B's) over the rows of group
@@ -147,6 +157,36 @@ __global__ void __launch_bounds__(256) exp_dense_kernel(int64_t n, const double*
   exps[blockIdx.y * stride + col] = e;
 }
 
+// The same of a row-major A: one CTA per group and 64 columns, a lane per 16-byte pair of columns.
+__global__ void __launch_bounds__(256) exp_dense_rows_kernel(int64_t n, const double* __restrict__ A, int64_t lda,
+                                                             int* __restrict__ exps, int64_t stride,
+                                                             int* __restrict__ flag) {
+  __shared__ uint32_t key[64];
+  if (threadIdx.x < 64) key[threadIdx.x] = 0u;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t c = (int64_t)blockIdx.x * 64 + 2 * lane, r0 = (int64_t)blockIdx.y * kGroupRows;
+  const int rows = (int)min((int64_t)kGroupRows, n - r0);
+  uint32_t k0 = 0u, k1 = 0u;
+  if (c < n) {  // n is even
+    const double* p = A + r0 * lda + c;
+#pragma unroll 8
+    for (int r = w; r < rows; r += 8) {
+      const double2 x = __ldg(reinterpret_cast<const double2*>(p + r * lda));
+      k0 = max(k0, exp_key(x.x)), k1 = max(k1, exp_key(x.y));
+    }
+  }
+  atomicMax(&key[2 * lane], k0);
+  atomicMax(&key[2 * lane + 1], k1);
+  __syncthreads();
+  const int64_t col = (int64_t)blockIdx.x * 64 + threadIdx.x;
+  if (threadIdx.x < 64 && col < n) {
+    const int e = group_exp(key[threadIdx.x]);
+    if (e < 0) *flag = 1;
+    exps[blockIdx.y * stride + col] = e;
+  }
+}
+
 // Exponents of a row-major block of p <= 32 columns (any row stride), one CTA per group.
 __global__ void __launch_bounds__(256) exp_rows_kernel(int64_t n, int p, const double* __restrict__ X, int ldx,
                                                        int* __restrict__ exps, int64_t stride,
@@ -176,10 +216,12 @@ template <int CA, int NB, bool PANEL>
 __global__ void __launch_bounds__(kThreads, 1)
     gram64_kernel(int64_t n, Cols<double> A, Cols<double> B, int ld, int a0, int pa, int b0, int pb, int upper,
                   int same, int rs, const int* __restrict__ exps, int estride, int eb0,
-                  const int* __restrict__ flag, double* __restrict__ part, int64_t groups_per_cta, int npanels) {
+                  const int* __restrict__ flag, double* __restrict__ part, int64_t groups_per_cta, int npanels,
+                  int row_a) {
   constexpr int kAS = NB <= 32 ? 2 : 1;  // accumulators (of kDiags * NB TMEM columns)
   constexpr int kAcc = kDiags * NB;
   constexpr uint32_t kSliceA = CA / 8 * kSBO, kSliceB = NB / 8 * kSBO;  // bytes of a slice
+  constexpr int kColStride = kKC + 2;  // PANEL: doubles between the columns of a raw stage
   constexpr int kEW = NB / 2;  // columns per epilogue warp (two warps per lane quadrant)
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t raw_full[kMaxRS], raw_empty[kMaxRS], tile_full[kTS], tile_empty[kTS];
@@ -215,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     nu_s = nu;
     abort_flag = 0;
-    for (int s = 0; s < kMaxRS; ++s) mbar_init(&raw_full[s], 1), mbar_init(&raw_empty[s], kSplitWarps / kSplitGroups);
+    for (int s = 0; s < kMaxRS; ++s) mbar_init(&raw_full[s], PANEL ? 33 : 1), mbar_init(&raw_empty[s], kSplitWarps / kSplitGroups);
     for (int s = 0; s < kTS; ++s) mbar_init(&tile_full[s], kSplitWarps / kSplitGroups), mbar_init(&tile_empty[s], 1);
     for (int s = 0; s < 2; ++s) mbar_init(&acc_full[s], 1), mbar_init(&acc_empty[s], kEpiWarps);
     fence_barrier_init();
@@ -227,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const Cols<double>& c = o == 0 ? A : B;
     int off = -1;
     if (PANEL) {
-      if (m < (o == 0 ? pa : pb)) off = m;  // A: not staged
+      if (m < (o == 0 ? pa : pb)) off = o == 0 ? m * (row_a ? 1 : kColStride) : kCB * kColStride + m;
     } else if (m < (o == 0 ? pa : pb) && !(o == 1 && same)) {
       const int col = m + (o == 0 ? a0 : b0);
       int base = 0, g = 0;
@@ -238,8 +280,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     colofs[o][m] = off;
   }
-  // doubles of a raw stage: [nu][kKC][ld], or kKC rows of X
-  const int stage = PANEL ? kKC * B.ld[0] : nu * seg;
+  // doubles of a raw stage: [nu][kKC][ld], or kCB columns of A and kKC rows of X
+  const int stage = PANEL ? kCB * kColStride + kKC * B.ld[0] : nu * seg;
   const size_t raw_bytes = ((size_t)rs * stage * 8 + 127) / 128 * 128;
   double* raw = reinterpret_cast<double*>(smem);  // [rs][stage]
   unsigned char* tiles = smem + raw_bytes;
@@ -261,19 +303,31 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int ngroups = (nchunks + kChunks - 1) / kChunks;
   int issued = 0, committed = 0;  // producer thread; MMA thread (groups)
   if (PANEL && warp == 0) {
-    if (lane == 0) {
-      int st = 0;
-      uint32_t ph = 0;
-      for (int c = 0; c < nchunks; ++c) {
-        if (c >= rs && !wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, 3)) break;
-        const int64_t r0 = r_begin + (int64_t)c * kKC;
-        const int rows = (int)min((int64_t)kKC, r_end - r0);  // even: n is
+    int st = 0;
+    uint32_t ph = 0;
+    for (int c = 0; c < nchunks; ++c) {
+      if (c >= rs && !__all_sync(0xffffffffu, wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, 3))) break;
+      const int64_t r0 = r_begin + (int64_t)c * kKC;
+      const int rows = (int)min((int64_t)kKC, r_end - r0);  // even: n is
+      double* raw_st = raw + (size_t)st * stage;
+      if (lane == 0) {
         const uint32_t bytes = (uint32_t)((rows - 1) * B.ld[0] + pb + 1) / 2 * 16u;
         mbar_expect_tx(&raw_full[st], bytes);
-        bulk_g2s(raw + (size_t)st * stage, B.p[0] + r0 * B.ld[0], bytes, &raw_full[st]);
-        issued = c + 1;
-        if (++st == rs) st = 0, ph ^= 1u;
+        bulk_g2s(raw_st + kCB * kColStride, B.p[0] + r0 * B.ld[0], bytes, &raw_full[st]);
       }
+      const int v = 2 * (lane & 15);
+      if (row_a) {  // columns 2 lane, + 1 of every row
+        if (2 * lane < pa) {
+          const double* src = A.p[0] + r0 * ld + a0 + 2 * lane;
+          for (int r = 0; r < rows; ++r, src += ld) cp_async16(raw_st + r * kCB + 2 * lane, src);
+        }
+      } else if (v < rows) {  // rows v, v + 1 of columns lane / 16, + 2, ..
+        const double* src = A.p[0] + (int64_t)(a0 + (lane >> 4)) * ld + r0 + v;
+        for (int m = lane >> 4; m < pa; m += 2, src += 2 * (int64_t)ld) cp_async16(raw_st + m * kColStride + v, src);
+      }
+      cp_async_arrive(&raw_full[st]);  // one arrival per lane, once its copies have landed
+      issued = c + 1;
+      if (++st == rs) st = 0, ph ^= 1u;
     }
   } else if (warp == 0) {
     if (lane == 0) {
@@ -414,13 +468,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int sw = warp - kSplit0, g = sw / wpg, sg = sw % wpg;
     const int gA = (pa + 31) / 32, gB = same ? 0 : (pb + 31) / 32;
     const int units = (gA + gB) * K8;
-    bool fromA[kMaxUW];  // PANEL: a unit of A
     int src[kMaxUW], ecol[kMaxUW], exp_[kMaxUW], rstep[kMaxUW];  // rstep: doubles between rows
     uint32_t dst[kMaxUW], step[kMaxUW], k0[kMaxUW];
 #pragma unroll
     for (int j = 0; j < kMaxUW; ++j) {
       const int u = sg + j * wpg;
-      fromA[j] = false;
       src[j] = -1, dst[j] = 0, step[j] = 0, ecol[j] = 0, rstep[j] = ld, exp_[j] = kExpOne, k0[j] = 0;
       if (u < units) {
         const bool isA = u < gA * K8;
@@ -428,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int k8 = v % K8, m = v / K8 * 32 + lane;
         const int off = colofs[isA ? 0 : 1][m];
         if (off >= 0) {
-          if constexpr (PANEL) rstep[j] = B.ld[0], fromA[j] = isA;
+          if constexpr (PANEL) rstep[j] = isA ? (row_a ? kCB : 1) : B.ld[0];
           src[j] = off + 8 * k8 * rstep[j];
           k0[j] = 8 * k8;
           ecol[j] = isA ? a0 + m : eb0 + b0 + m;
@@ -437,24 +489,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-    // PANEL: the first two units of a warp (the A units are among them) a chunk ahead in registers
-    constexpr int kAhead = PANEL ? 2 : 1;
-    double2 ahead[kAhead][4];
-    auto load_ahead = [&](int c) {
-      if constexpr (PANEL) {
-        const int64_t r0 = r_begin + (int64_t)c * kKC;
-#pragma unroll
-        for (int j = 0; j < kAhead; ++j) {
-          if (!fromA[j]) continue;
-          const double* p = A.p[0] + (int64_t)ecol[j] * ld + r0 + k0[j];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            ahead[j][i] = c < nchunks && r0 + k0[j] + 2 * i < r_end ? __ldg(reinterpret_cast<const double2*>(p) + i)
-                                                                    : make_double2(0.0, 0.0);
-        }
-      }
-    };
-    load_ahead(g);
     int st = g % rs, buf = g % kTS, cur = -1;
     uint32_t ph = 0, tph = 0;
     for (int c = g; c < nchunks; c += kSplitGroups) {
@@ -473,10 +507,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kMaxUW; ++j) {
         if (src[j] < 0) continue;
         double x[8];
-        if (PANEL && j < kAhead && fromA[j]) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) x[2 * i] = ahead[j < kAhead ? j : 0][i].x, x[2 * i + 1] = ahead[j < kAhead ? j : 0][i].y;
-        } else if (rows == kKC) {
+        if (rows == kKC) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) x[i] = rsb[src[j] + i * rstep[j]];
         } else {
@@ -489,7 +520,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         unsigned char* o = tb_ + dst[j];
         put_digits(w, o, step[j]);
       }
-      load_ahead(c + kSplitGroups);
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) {
@@ -503,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   if (abort_flag) {
     // bounded waits for the copies and MMAs in flight before the memory they use goes
-    if (warp == 0 && lane == 0)
+    if (warp == 0 && (PANEL || lane == 0))
       for (int c = max(0, issued - rs); c < issued; ++c) mbar_wait(&raw_full[c % rs], (uint32_t)(c / rs) & 1u, kWaitCycles);
     if (warp == 1 && lane == 0 && committed > 0)
       mbar_wait(&acc_full[(committed - 1) % kAS], (uint32_t)((committed - 1) / kAS) & 1u, kWaitCycles);
@@ -556,7 +586,7 @@ void gram64_launch(int64_t n, const Cols<double>& a, const Cols<double>& b, int 
   }();
   (void)attr;
   gram64_kernel<CA, NB, false><<<(unsigned)ctas, kThreads, smem, st>>>(n, a, b, ld, a0, pa, b0, pb, upper ? 1 : 0, same ? 1 : 0,
-                                                           rs, exps, estride, eb0, flag, part, gpc, 0);
+                                                           rs, exps, estride, eb0, flag, part, gpc, 0, 0);
   LB_LAUNCH_CHECK();
 }
 
@@ -656,16 +686,16 @@ size_t dense64_scratch_bytes(int64_t n, int p) {
   return 256 + exps + (size_t)kMaxSplits * n * p * sizeof(double);
 }
 
-// Y = A X (column i of the dense column-major A against X) through digit products; false without
+// Y = A X (column i of the dense A against X; A column-major, or row-major with row_a) through digit products; false without
 // launching where A or X do not fit (odd n or lda, unaligned).  *scratch is the flag left at 1 when a
 // number is outside the digits' range: Y is then to be formed by launch_spmm_dense on that flag.
 bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
-                              int ldy, void* scratch, cudaStream_t st) {
+                              int ldy, void* scratch, bool row_a, cudaStream_t st) {
   if (n < 2 || (n & 1) || (lda & 1) || lda > INT_MAX || p < 1 || p > 32 || (reinterpret_cast<uintptr_t>(A) & 15) ||
       (reinterpret_cast<uintptr_t>(X) & 15))
     return false;
   constexpr int NB = 32;
-  const size_t stage = (size_t)kKC * ldx * 8;
+  const size_t stage = ((size_t)kCB * (kKC + 2) + (size_t)kKC * ldx) * 8;
   const size_t tiles = (size_t)kTS * (8 * (size_t)(kCB / 8) + kSlices * (size_t)(NB / 8)) * kSBO;
   if (tiles + 2 * stage + 128 > kSmemBudget) return false;
   const int rs = (int)std::min<size_t>(kMaxRS, (kSmemBudget - tiles - 128) / stage);
@@ -683,13 +713,16 @@ bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, co
   double* part = reinterpret_cast<double*>(static_cast<char*>(scratch) + 256 +
                                            ((size_t)groups * estride * sizeof(int) + 255) / 256 * 256);
   LB_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
-  exp_dense_kernel<<<dim3((unsigned)ceil_div(n, 8), (unsigned)groups), 256, 0, st>>>(n, A, lda, exps, estride, flag);
+  if (row_a)
+    exp_dense_rows_kernel<<<dim3((unsigned)panels, (unsigned)groups), 256, 0, st>>>(n, A, lda, exps, estride, flag);
+  else
+    exp_dense_kernel<<<dim3((unsigned)ceil_div(n, 8), (unsigned)groups), 256, 0, st>>>(n, A, lda, exps, estride, flag);
   LB_LAUNCH_CHECK();
   exp_rows_kernel<<<(unsigned)groups, 256, 0, st>>>(n, p, X, ldx, exps + n, estride, flag);
   LB_LAUNCH_CHECK();
   gram64_kernel<kCB, NB, true><<<(unsigned)(panels * splits), kThreads, smem, st>>>(
       n, cols1<double>(A, (int)lda, 1), cols1<double>(X, ldx, p), (int)lda, 0, 0, 0, p, 0, 0, rs, exps, (int)estride,
-      (int)n, flag, part, ceil_div(groups, splits), (int)panels);
+      (int)n, flag, part, ceil_div(groups, splits), (int)panels, row_a ? 1 : 0);
   LB_LAUNCH_CHECK();
   panel_reduce_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n * p, 256), 4096), 256, 0, st>>>(n, p, splits, part, Y,
                                                                                                ldy, flag);

@@ -490,9 +490,17 @@ struct Prec<float> {
   static int64_t lda(lobpcg_ctx& c) { return c.A.n; }
 };
 
-// Multiply-adds from which the digit products win over FP64 FMAs and over double-float.
+// Multiply-adds from which the digit products win over FP64 FMAs and over double-float: their fixed
+// cost (exponents, TMEM, the second kernel) against the older kernels' rates.  Microseconds per call just
+// below and above each line (older kernel, digits), entry-point overhead of about 40 included:
+//   Gram, FP64 FMAs:     16 columns 84, 91    32 columns 96, 76    63 columns 115, 90
+//   Gram, double-float:  16 columns 143, 123  32 columns 111, 88   63 columns 132, 89
+//   update, double-float: 63 columns to 21 98, 67   21 to 7 126, 115   96 to 32 101, 78
+//   dense product, FP64 FMAs, at 3e7 multiply-adds: p = 4 217, 110   p = 13 187, 93   p = 32 159, 85;
+//     half of that is where they meet
+// The update's line against FP64 FMAs is the Gram's: the same pipe, the same fixed cost.
 constexpr double kDigitGram = 2e7, kDigitGramDf = 6e7;
-constexpr double kDigitDense = 3e7;
+constexpr double kDigitDense = 1.5e7;
 constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7;
 
 // launch_update with, in profile mode, the FP64 launches timed and their flops counted.
@@ -538,7 +546,7 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
     if constexpr (std::is_same<T, double>::value) {
       if (dense_digits_pay(c.A.n, p)) {
         c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
-        if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, c.st)) {
+        if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false, c.st)) {
           c.used_digits = true;
           launch_spmm_dense<T>(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.st, c.dense_buf.as<int>());
           return;
@@ -1708,7 +1716,7 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
     PoolBuf work(st);
     if (dense_digits_pay(n, p)) {
       work.alloc(dense64_scratch_bytes(n, p));
-      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, st)) {
+      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, false, st)) {
         launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st, work.as<int>());
         gram64_check(st);
         return LOBPCG_OK;
@@ -1716,6 +1724,25 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
     }
     launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st);
     LB_CUDA(cudaStreamSynchronize(st));
+    return LOBPCG_OK;
+  });
+}
+
+extern "C" lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, int64_t lda, int p, const double* X,
+                                                    int ldx, double* Y, int ldy, int* done, lobpcg_stream stream) {
+  return guarded(nullptr, [&]() -> lobpcg_status {
+    require(n >= 0 && A && X && Y && done && lda >= n, "lobpcg_spmm_dense_rows_f64: NULL argument or lda < n");
+    require(p >= 1 && p <= 32 && ldx >= p && ldy >= p, "lobpcg_spmm_dense_rows_f64: need 1 <= p <= 32, ld >= p");
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    *done = 0;
+    if (!dense_digits_pay(n, p)) return LOBPCG_OK;
+    PoolBuf work(st);
+    work.alloc(dense64_scratch_bytes(n, p));
+    if (!launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, true, st)) return LOBPCG_OK;
+    int flag = 0;
+    LB_CUDA(cudaMemcpyAsync(&flag, work.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    gram64_check(st);
+    *done = flag ? 0 : 1;
     return LOBPCG_OK;
   });
 }

@@ -34,6 +34,20 @@ def test_dense(n, p, graded):
     assert (np.abs((Y - ref).astype(np.float64)) <= tol).all()
 
 
+@pytest.mark.parametrize("n,p", [(1226, 31), (2050, 13)])
+def test_both_storage_orders(n, p):
+    """Column i of A against X, whichever way A is stored (A is not symmetric here)."""
+    import torch
+
+    import paper_2305_06668_gb300 as lb
+    rng = np.random.default_rng(n + 1)
+    A, X = torch.from_numpy(rng.standard_normal((n, n))).cuda(), torch.from_numpy(rng.standard_normal((n, p))).cuda()
+    Y = lb.spmm_dense(A, X)
+    assert torch.equal(Y, lb.spmm_dense(A.t().contiguous().t(), X))
+    ref = A.t() @ X
+    assert (Y - ref).norm() <= 1e-14 * ref.norm()
+
+
 @pytest.mark.parametrize("bad", [np.inf, np.nan, 1e200])
 @pytest.mark.parametrize("where", ["A", "X"])
 def test_outside_the_digits(bad, where):
