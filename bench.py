@@ -36,6 +36,8 @@ WORKLOAD = "CI-like sparse symmetric n=2,000,000, ~65 nnz/row, k=16 (+5 extra), 
 # calls only the oracle.  Both CPU legs scale it to the machine's cores.
 ORACLE_RECORD = os.path.join(ROOT, "oracle", "records", "ci2m_seed0.json")
 FP64_PEAK_SOURCE = "FP64 FMA rate measured in this run (lobpcg_probe_fma_rate)"
+DIGIT_PRODUCTS = 34  # FP16 products of one FP64 multiply-add (csrc/slices.cuh)
+TENSOR_PEAK = 1872.3  # TFLOP/s, cuBLAS bf16 on this part
 DF_OPS_PER_TERM = 15  # FP32 operations of one double-float multiply-add (dfloat.cuh df_fma)
 
 
@@ -339,26 +341,24 @@ def run_ours(args):
                                       "frac": f64 / t64 / 1e12 / fp64_peak, "traffic": None,
                                       "flops_per_launch": f64, "avg_launch_s": t64,
                                       "peak_source": FP64_PEAK_SOURCE}
-    # the FP64 block updates of the refinement, timed per launch with CUDA events.  With
-    # double-float products (the default in the mixed form's refinement) they run on the FP32
-    # pipes: each FP64-equivalent multiply-add is 15 FP32 operations (TwoProduct, TwoSum,
-    # Fast2Sum renormalisation), so the roofline counts FP32 pipe operations (one per issue
-    # slot) against the FP32 FMA instruction rate of this GPU (the probe's FP32 TFLOP/s / 2).
+    # the FP64 block updates of the refinement, timed per launch with CUDA events.  Above the size
+    # rule they are exact digit products on the tensor cores: 34 FP16 products per FP64 multiply-add
+    # (of the padded 32 columns only the used ones are counted), so the roofline counts FP16 tensor
+    # flops; the plain FP64 form below counts FP64 ones.
     ut = sum(i["update_fp64_seconds"] for _, i, _, _ in infos)
     uf = sum(i["update_fp64_flops"] for _, i, _, _ in infos)
     ul = sum(i["update_fp64_launches"] for _, i, _, _ in infos)
     if ul and ut > 0:
         if df:
-            ops = uf / 2.0 * DF_OPS_PER_TERM
-            rooflines["update_fp64"] = {"kernel": "update_df_async_kernel (FP64 block updates in double-float on "
-                                                  "the FP32 pipes: X = V u_x, P = V u_p, W -= Y C, W <- W + W (T - I))",
-                                        "bound": "alu", "achieved": ops / ut / 1e12, "peak": fp32_peak / 2,
-                                        "unit": "TFLOP/s", "frac": ops / ut / 1e12 / (fp32_peak / 2),
-                                        "ops": "FP32 pipe operations, 15 per FP64-equivalent multiply-add",
+            ops = uf * DIGIT_PRODUCTS
+            rooflines["update_fp64"] = {"kernel": "update64_kernel (FP64 block updates through exact FP16 digit "
+                                                  "products, tcgen05: X = V u_x, P = V u_p, W -= Y C, W <- W T)",
+                                        "bound": "tensor", "achieved": ops / ut / 1e12, "peak": TENSOR_PEAK,
+                                        "unit": "TFLOP/s", "frac": ops / ut / 1e12 / TENSOR_PEAK,
+                                        "ops": "FP16 tensor flops, 34 digit products per FP64 multiply-add",
                                         "fp64_equivalent_tflops": uf / ut / 1e12, "traffic": None,
                                         "flops_per_launch": ops / ul, "avg_launch_s": ut / ul,
-                                        "peak_source": "FP32 FMA instruction rate measured in this run "
-                                                       "(lobpcg_probe_fma_rate / 2)"}
+                                        "peak_source": "cuBLAS bf16 throughput, burst"}
         else:
             rooflines["update_fp64"] = {"kernel": "update_kernel<double> (FP64 block updates)", "bound": "alu",
                                         "achieved": uf / ut / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",

@@ -124,7 +124,11 @@ typedef struct {
                                  the FP32 pipes (about 2^-48 per product, chunk sums in FP64).
                                  0 (default): double-float in the FP64 refinement of the MIXED
                                  form, FP64 fused multiply-adds in the FP64 form; 1: double-float
-                                 in every FP64 phase; -1: FP64 fused multiply-adds everywhere */
+                                 in every FP64 phase; -1: FP64 fused multiply-adds everywhere.
+                                 Grams and updates of some size (2e7 to 6e7 multiply-adds) take
+                                 exact digit products on the tensor cores in either form, with
+                                 errors no larger than the fused multiply-adds'; the double-float
+                                 phases keep their tau and CSR products */
   int tc_gram;                /* FP32 Gram matrices of the MIXED form: non-zero (default) on the
                                  tcgen05 tensor cores (lobpcg_gram_f32_tcgen05), 0 with warp-level
                                  mma.sync (lobpcg_gram_f32); both 3xTF32 */
@@ -316,13 +320,13 @@ LOBPCG_API lobpcg_status lobpcg_gram_f64(int64_t n, int p, const double* X, int 
 /* C = X^T Y like lobpcg_gram_f64, formed in double-float arithmetic on the FP32 pipes (the
  * arithmetic of the FP64 refinement, see lobpcg_options.df_products): each FP64 element is
  * split into two floats, products and sums are error-compensated, sums of ~128 rows are
- * added in FP64.  X, Y: 16-byte aligned, one even row stride (ldx == ldy).  Not in the
+ * added in FP64; from n p q = 6e7 on through exact digit products on the tensor cores.  X, Y: 16-byte aligned, one even row stride (ldx == ldy).  Not in the
  * paper; the operation is Algorithm 1's Gram. */
 LOBPCG_API lobpcg_status lobpcg_gram_f64_df(int64_t n, int p, const double* X, int ldx, int q, const double* Y,
                                             int ldy, double* C, lobpcg_stream stream);
 
 /* The FP64 block update X = base + alpha [V_g] U (and AX, residual norms) in double-float
- * arithmetic; arguments as lobpcg_update_f32 with FP64 blocks (V_g, AV_g, base, X, AX:
+ * arithmetic, from 6e7 multiply-adds on through exact digit products on the tensor cores; arguments as lobpcg_update_f32 with FP64 blocks (V_g, AV_g, base, X, AX:
  * double, row stride ld / ld_base / ld_out in doubles). */
 LOBPCG_API lobpcg_status lobpcg_update_f64_df(int64_t n, int nseg, const double* const* V, const double* const* AV,
                                               const int* w, int ld, const double* U, int q, double alpha,
@@ -369,12 +373,14 @@ LOBPCG_API lobpcg_status lobpcg_gram_f32_tcgen05(int64_t n, int p, const float* 
                                                  int ldy, double* C, lobpcg_stream stream);
 
 /* Symmetric eigen-decomposition of s x s column-major a (s <= 96) by parallel-order
- * Jacobi rotations in FP64 (the Rayleigh-Ritz solve of Algorithm 1).  lam: device, s
+ * Jacobi rotations in FP32 and refinement of the vectors in FP64, or by FP64 Jacobi rotations
+ * where that does not converge (the Rayleigh-Ritz solve of Algorithm 1); eigenvalues and
+ * residuals to ~eps ||a||, U orthonormal to FP64 rounding.  lam: device, s
  * values ascending; U: device, column-major s x s eigenvectors. */
 LOBPCG_API lobpcg_status lobpcg_syev_f64(int s, const double* a, double* lam, double* U, lobpcg_stream stream);
 
 /* Same contract, two-stage method (the Rayleigh-Ritz solve of the FP32 phase of the mixed
- * form): FP32 Jacobi, one FP64 Cholesky-QR of its rotation matrix Q, then Jacobi on
+ * form): the refinement of lobpcg_syev_f64 stopped at tol or, where that does not converge, FP32 Jacobi, one FP64 Cholesky-QR of its rotation matrix Q, then Jacobi on
  * Q^T a Q accumulated into Q until its off-diagonal mass is <= tol ||a||_F (tol = 0 means
  * 1e-15).  tol < 1e-12: FP64 rotations; eigenvalues and residuals to FP64 absolute accuracy
  * (~eps ||a||), U orthonormal to FP64 rounding.  1e-12 <= tol < 1e-6 (the solver uses

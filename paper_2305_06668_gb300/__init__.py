@@ -406,7 +406,7 @@ def gram_f32_tcgen05(X, Y, stream=None):
 
 def gram_df(X, Y, stream=None):
     """C = X^T Y of FP64 row-major CUDA blocks (one aligned row stride) in double-float
-    arithmetic (the FP64 refinement's Gram)."""
+    arithmetic or, for large blocks, exact digit products (the FP64 refinement's Gram)."""
     torch = _torch()
     n, p = X.shape
     q = Y.shape[1]
@@ -463,7 +463,7 @@ def gram_noalloc(X, Y, out=None, stream=None):
 
 def syev(a, two_stage=False, tol=0.0, stream=None):
     """Eigenvalues (ascending) and eigenvectors of symmetric a; two_stage selects the
-    FP32-then-FP64 Jacobi used by the FP32 phase of the mixed form, stopped at tol (0: 1e-15)."""
+    FP32-then-FP64 solve used by the FP32 phase of the mixed form, stopped at tol (0: 1e-15)."""
     torch = _torch()
     s = a.shape[0]
     ac = a.t().contiguous()  # column-major storage of a

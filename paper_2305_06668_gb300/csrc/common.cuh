@@ -252,9 +252,9 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
 // ---- small FP64 kernels (one CTA) ----
 // Symmetric eigensolve: a (s x s, column-major; only the upper triangle is read when
 // upper_only) -> lam ascending, U column-major.  sweeps_out: device int (may be null),
-// FP64 sweeps.  two_stage: FP32 Jacobi, Cholesky-QR of its rotations, FP64 Jacobi on
-// Q^T a Q (faster; absolute accuracy eps ||a||); else FP64 Jacobi from a.  The FP64
-// Jacobi stops when its off-diagonal mass is <= tol64 ||a||_F.
+// refinement steps or FP64 sweeps.  From s = 2 on the cluster solver (syev.cu); where it gives up, two_stage:
+// FP32 Jacobi, Cholesky-QR of its rotations, FP64 Jacobi on Q^T a Q (faster; absolute accuracy
+// eps ||a||), else FP64 Jacobi from a, stopped when the off-diagonal mass is <= tol64 ||a||_F.
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,
                  cudaStream_t st, bool two_stage = false, double tol64 = 1e-15);
 
