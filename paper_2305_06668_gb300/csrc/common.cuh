@@ -256,7 +256,7 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
 // FP32 Jacobi, Cholesky-QR of its rotations, FP64 Jacobi on Q^T a Q (faster; absolute accuracy
 // eps ||a||), else FP64 Jacobi from a, stopped when the off-diagonal mass is <= tol64 ||a||_F.
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,
-                 cudaStream_t st, bool two_stage = false, double tol64 = 1e-15);
+                 cudaStream_t st, bool two_stage = false, double tol64 = 1e-15, bool refine = true);
 
 // The cluster eigensolver behind launch_syev (syev.cu): lam[0] = NaN where it gave up.
 void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, double* U, int* steps_out, float stop,

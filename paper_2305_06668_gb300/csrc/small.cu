@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(kSmallThreads) lock_p_kernel(int s, int m, int
 }  // namespace
 
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,
-                 cudaStream_t st, bool two_stage, double tol64) {
+                 cudaStream_t st, bool two_stage, double tol64, bool refine) {
   if (s <= 0) return;
   if (s > kMaxS) throw std::invalid_argument("syev: s > 96");
   const size_t smem = (size_t)(two_stage ? 3 : 2) * s * (s + 1) * sizeof(double);
@@ -979,7 +979,7 @@ void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U
   (void)attr;
   // The cluster solver from 2 columns on (syev.cu; measured per call at s = 63, see there); this
   // kernel then runs only where that one gave up.
-  const bool behind = s > 1;
+  const bool behind = s > 1 && refine;
   if (behind) launch_syev_cluster(s, a, upper_only, lam, U, sweeps_out, tol64 >= 1e-12 ? 1e-5f : 1e-9f, st);
   const double tol32 = 1e-4;  // measured: the stopping point of this stage hardly changes the total
   if (two_stage)

@@ -855,7 +855,7 @@ PhaseOut run_lobpcg(lobpcg_ctx& c, int k, int m, double tol, double tau, int max
   apply_A<T>(c, b.X[0], ld, m, b.AX[0], ld);                            // AX = A X
   gram<T>(c, cols1<T>(b.X[0], ld, m), cols1<T>(b.AX[0], ld, m), true, c.G);  // a = X^T AX
   launch_syev(m, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, sizeof(T) == 4,
-              sizeof(T) == 4 ? 1e-10 : 1e-15);  // a u = u lambda
+              sizeof(T) == 4 ? 1e-10 : 1e-15, sizeof(T) == 4);  // a u = u lambda
   LB_CUDA(cudaMemcpyAsync(c.lam, c.lam_all, m * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
   {
     UpdateJob<T> job{};
@@ -922,7 +922,8 @@ PhaseOut run_lobpcg(lobpcg_ctx& c, int k, int m, double tol, double tau, int max
     c.prof.mark(PH_RR_EIG);
     // Rayleigh-Ritz; the FP32 phase, whose Ritz vectors go to FP32 blocks (rounding 6e-8),
     // takes the two-stage solver stopped at 1e-10 relative, the FP64 phase the full one
-    launch_syev(s, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, sizeof(T) == 4, sizeof(T) == 4 ? 1e-10 : 1e-15);
+    launch_syev(s, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, sizeof(T) == 4, sizeof(T) == 4 ? 1e-10 : 1e-15,
+                sizeof(T) == 4);
     c.prof.mark(PH_UPDATE);
     LB_CUDA(cudaMemcpyAsync(c.lam, c.lam_all, m * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
     const int nxt = cur ^ 1;
@@ -1113,7 +1114,7 @@ PhaseOut run_lobpcg_gen(lobpcg_ctx& c, int k, int m, double tol, double tau, int
   b_ortho(c, b.X[0], c.BX[0], ld, m, tau, cap);
   apply_A<double>(c, b.X[0], ld, m, b.AX[0], ld);
   gram<double>(c, cols1<double>(b.X[0], ld, m), cols1<double>(b.AX[0], ld, m), true, c.G);
-  launch_syev(m, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, false, 1e-15);
+  launch_syev(m, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, false, 1e-15, false);
   LB_CUDA(cudaMemcpyAsync(c.lam, c.lam_all, m * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
   auto rotate = [&](const Cols<double>& V, const Cols<double>& AV, const Cols<double>& BV, int s, int nxt,
                     bool with_p) {
@@ -1148,7 +1149,7 @@ PhaseOut run_lobpcg_gen(lobpcg_ctx& c, int k, int m, double tol, double tau, int
     Cols<double> BV =
         cols_add<double>(cols_add<double>(cols1<double>(c.BX[cur], ld, m), c.BP[cur], ld, pw), c.BW, ld, aw);
     gram<double>(c, V, AV, true, c.G);                                      // a = V^T A V
-    launch_syev(s, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, false, 1e-15);
+    launch_syev(s, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, false, 1e-15, false);
     LB_CUDA(cudaMemcpyAsync(c.lam, c.lam_all, m * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
     const int nxt = cur ^ 1;
     rotate(V, AV, BV, s, nxt, true);

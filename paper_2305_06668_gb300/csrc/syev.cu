@@ -19,7 +19,8 @@
 // K antisymmetric, K_ij = N_ij / (lambda_j - lambda_i), N = (S + S^T) / 2 + R (lambda_i + lambda_j) / 2.  The
 // halves of S come together through U, so K is antisymmetric to the last bit and rounding of S over a
 // small gap only turns vectors, it never takes them off orthonormality (S_ij alone did, by 4e-9 at a
-// gap of 1e-7).  Where N_ij is rounding noise (repeated eigenvalues) K_ij = 0.  Where it is not small
+// gap of 1e-7).  Where N_ij is rounding noise of ||A|| and the gap within 1e-10 ||A|| (repeated
+// eigenvalues) K_ij = 0; over any wider gap a coupling counts whatever its size.  Where it is not small
 // against the gap (close eigenvalues that FP32 did not separate) the Jacobi angle of the pair, halved,
 // takes the quotient's place: the pair turns by a bounded angle, and the quotient applies once it is
 // small.  Without convergence in kMaxSteps, or with a non-finite entry, lambda_0 is set to NaN, on which
@@ -270,13 +271,15 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
       if (i != j) {
         const double gap = lsh[j] - lsh[i];
         const double num = 0.5 * (S[k] + __ldcg(U + j + i * s)) + (0.5 * (lsh[i] + lsh[j])) * R[k];
-        if (fabs(num) > noise) {
-          if (fabs(num) <= 0.2 * fabs(gap)) {
-            E += num / gap;
-          } else {
+        // a small coupling over a normal gap counts whatever its size against ||a||: the Ritz vectors of
+        // a graded matrix (P directions) live on it
+        if (fabs(num) > 0.2 * fabs(gap)) {
+          if (fabs(num) > noise) {
             const double tau = gap / (2.0 * num);
             E += 0.5 * (tau > 0.0 || (tau == 0.0 && i < j) ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
           }
+        } else if (fabs(num) > noise || fabs(gap) > 1e5 * noise) {
+          E += num / gap;
         }
       }
       Eb[i + (j - j0) * ld] = E;
