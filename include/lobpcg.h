@@ -374,7 +374,7 @@ LOBPCG_API lobpcg_status lobpcg_gram_f32_tcgen05(int64_t n, int p, const float* 
 
 /* Symmetric eigen-decomposition of s x s column-major a (s <= 96) by parallel-order
  * Jacobi rotations in FP32 and refinement of the vectors in FP64, or by FP64 Jacobi rotations
- * where that does not converge (the Rayleigh-Ritz solve of Algorithm 1); eigenvalues and
+ * where that does not converge (the Rayleigh-Ritz problem of Algorithm 1); eigenvalues and
  * residuals to ~eps ||a||, U orthonormal to FP64 rounding.  lam: device, s
  * values ascending; U: device, column-major s x s eigenvectors. */
 LOBPCG_API lobpcg_status lobpcg_syev_f64(int s, const double* a, double* lam, double* U, lobpcg_stream stream);

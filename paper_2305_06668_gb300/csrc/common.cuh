@@ -252,7 +252,7 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
 // ---- small FP64 kernels (one CTA) ----
 // Symmetric eigensolve: a (s x s, column-major; only the upper triangle is read when
 // upper_only) -> lam ascending, U column-major.  sweeps_out: device int (may be null),
-// refinement steps or FP64 sweeps.  From s = 2 on the cluster solver (syev.cu); where it gives up, two_stage:
+// refinement steps or FP64 sweeps.  refine: from s = 2 on the cluster solver (syev.cu); else, or where it gives up, two_stage:
 // FP32 Jacobi, Cholesky-QR of its rotations, FP64 Jacobi on Q^T a Q (faster; absolute accuracy
 // eps ||a||), else FP64 Jacobi from a, stopped when the off-diagonal mass is <= tol64 ||a||_F.
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,

@@ -921,7 +921,7 @@ PhaseOut run_lobpcg(lobpcg_ctx& c, int k, int m, double tol, double tau, int max
     if (sizeof(T) == 4) c.stats.rr_gram32_bytes += 2.0 * (double)n * s * sizeof(T), c.stats.rr_gram32_count++;
     c.prof.mark(PH_RR_EIG);
     // Rayleigh-Ritz; the FP32 phase, whose Ritz vectors go to FP32 blocks (rounding 6e-8),
-    // takes the two-stage solver stopped at 1e-10 relative, the FP64 phase the full one
+    // takes the two-stage solver stopped at 1e-10 relative, the FP64 phase plain FP64 Jacobi
     launch_syev(s, c.G, true, c.lam_all, c.U, c.ictl + 4, c.st, sizeof(T) == 4, sizeof(T) == 4 ? 1e-10 : 1e-15,
                 sizeof(T) == 4);
     c.prof.mark(PH_UPDATE);

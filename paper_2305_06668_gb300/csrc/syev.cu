@@ -7,8 +7,10 @@
 // and square roots before them, over 8 or 9 sweeps.  FP32 rounds have no such pipe to wait for, and one
 // refinement step is four s x s x s products (1 M multiply-adds at s = 63) that eight SMs share; it
 // squares the error, so two or three steps take FP32's 1e-6 to FP64's rounding.  Kernel at s = 63:
-// 2,110 us (mean) -> 500 (largest) in the FP64 phase, two-stage 1,700 -> 370; at s = 12: 161 -> 44.  The
-// FP32 rounds, latency-bound, are about two thirds of it.
+// two-stage 1,700 -> 370 us, plain 2,110 (mean) -> 500 (largest); at s = 12 plain 161 -> 44.  The FP32
+// rounds, latency-bound, are about two thirds of it.  The solver's FP64 phases keep plain Jacobi: with this
+// kernel in them a mixed + diagonal solve of n = 10^5 did not converge in 4,000 iterations and a random
+// start of n = 2,000 broke down, for a reason that was not found.
 //
 // Layout.  Every CTA holds all of A and X in shared memory.  In the FP32 stage every CTA rotates its own
 // copy of the matrix (the same operations, so the same rotations) but only its own rows of the
