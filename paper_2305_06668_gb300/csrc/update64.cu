@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr uint32_t kSliceU = u_slice(KP), kSBOU = KP / 8 * 128;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t raw_full[kSplitWarps], tile_full[kMaxTS], tile_empty[kMaxTS], acc_full[2], acc_empty[2], exp_full[kRing];
+  __shared__ uint64_t rows_read[4];  // both epilogue warps of a lane quadrant have read their rows
   __shared__ int16_t row_exp[kRing][kTile];
   __shared__ int col_exp[kQ];
   __shared__ __align__(16) int16_t up[KP];  // exponent of row l of U: V's column l is scaled by 2^up
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int i = 0; i < kMaxTS; ++i) mbar_init(&tile_full[i], kSplitWarps), mbar_init(&tile_empty[i], 1);
     for (int i = 0; i < 2; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], kEpiWarps);
     for (int i = 0; i < kRing; ++i) mbar_init(&exp_full[i], kSplitWarps);
+    for (int i = 0; i < 4; ++i) mbar_init(&rows_read[i], 2);
     fence_barrier_init();
   }
   for (uint32_t e = tid; e < kSlices * kSliceU / 16; e += kThreads) reinterpret_cast<uint4*>(udig)[e] = make_uint4(0, 0, 0, 0);
@@ -306,6 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
     for (int g = 0; g < kQ / 8; ++g) nsum[g] = 0.0, nmax[g] = 0.0;
     bool ok = true;
+    uint32_t rph = 0;  // parity of the next rows_read phase
     for (int it = 0; it < ntiles && ok; ++it) {
       const int64_t grow = r_begin + (int64_t)it * kTile + row;
       const bool live = grow < r_end;
@@ -339,9 +342,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       // rows of this warp
       const int64_t row0 = r_begin + (int64_t)it * kTile + 32 * quad;
       const int nrows = (int)max((int64_t)0, min((int64_t)32, r_end - row0));
-      // both threads of a row have read it before either stores
+      // both threads of a row have read it before either stores (the two warps see the same rows, so both
+      // or neither come here); bounded like every wait, for the partner may have given up
       const bool any_bad = __any_sync(0xffffffffu, er[0] == kBad || er[1] == kBad);
-      if (any_bad) asm volatile("bar.sync %0, 64;\n" ::"r"(5 + quad) : "memory");
+      if (any_bad) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&rows_read[quad]);
+        ok = __all_sync(0xffffffffu, wait_bar(&rows_read[quad], rph, &abort_flag, 4));
+        rph ^= 1u;
+        if (!ok) break;
+      }
 #pragma unroll
       for (int gh = 0; gh < kQ / 8; ++gh) {
         const int g = 2 * gh + half;
