@@ -137,7 +137,7 @@ void launch_spmm_dense(int64_t n, const T* A, int64_t lda, int p, const T* X, in
 // row_a: A is row-major (Y is still column i of A against X).
 size_t dense64_scratch_bytes(int64_t n, int p);
 bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
-                              int ldy, void* scratch, bool row_a, cudaStream_t st);
+                              int ldy, void* scratch, bool row_a, int* err, cudaStream_t st);
 
 // Gram partials: part[g][i + j*pa] = sum over CTA g's rows of a_ri * b_rj.
 // upper: only i <= j entries are produced.  Returns the number of CTAs used.
@@ -158,19 +158,18 @@ int launch_update_pipe(int64_t n, const UpdateJob<T>& job, const double* U, int 
                        const double* lam, double* norm_part, int max_ctas, cudaStream_t st);
 // FP32 Gram partials on the 5th-generation tensor cores (tcgen05, TMA bulk copies, TMEM
 // accumulator; 3xTF32 products); returns 0 without launching when the operands do not
-// share one 16-byte aligned row stride or are wider than 96 columns.  umma_check reads and
-// clears its give-up flag (synchronising the stream) and throws if a CTA gave up waiting.
+// share one 16-byte aligned row stride or are wider than 96 columns.  *err (device, cleared by the
+// caller, here and below): not zero once a CTA gave up waiting (1: a bulk copy, 2: an MMA, 3: a pipeline
+// stage, 4: a partner).
 int gram_partials_umma(int64_t n, const Cols<float>& a, const Cols<float>& b, bool upper, double* part,
-                       int max_ctas, cudaStream_t st);
-void umma_check(cudaStream_t st);
+                       int max_ctas, int* err, cudaStream_t st);
 // FP64 Gram partials through exact digit products on the tensor cores (gram64.cu).  Returns the
 // number of CTAs, or 0 without launching where the blocks do not fit.  scratch:
 // gram64_scratch_ints(n) ints.  *scratch is the flag left at 1 when some column is outside the
 // digits' range: the partials are then to be formed by gram_partials with run_flag = scratch.
 size_t gram64_scratch_ints(int64_t n);
 int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
-                         int max_ctas, int* scratch, cudaStream_t st);
-void gram64_check(cudaStream_t st);
+                         int max_ctas, int* scratch, int* err, cudaStream_t st);
 // out[e] = sum_g part[g][e] for e < count (FP64, fixed order).
 void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st);
 
@@ -206,8 +205,7 @@ int launch_update_df(int64_t n, const UpdateJob<double>& job, const double* U, i
 // The FP64 update through exact digit products on the tensor cores (update64.cu); unit_base is
 // not needed there and ignored.  Returns 0 without launching where the blocks do not fit.
 int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                         const double* lam, double* norm_part, int max_ctas, cudaStream_t st);
-void update64_check(cudaStream_t st);
+                         const double* lam, double* norm_part, int max_ctas, int* err, cudaStream_t st);
 // dst[i] = (hi, lo) split of src[i] (the double-float operands: matrix values, blocks).
 void launch_split_df(int64_t count, const double* src, float2* dst, cudaStream_t st);
 // Y = A X (FP64 result) from the split values vs (nnz) and the split block Xs (n x ldx

@@ -62,24 +62,7 @@ constexpr int kEpi0 = 2, kEpiWarps = 8;
 constexpr int kSplit0 = kEpi0 + kEpiWarps, kSplitWarps = 8, kSplitGroups = 2;
 constexpr int kThreads = 32 * (kSplit0 + kSplitWarps);
 constexpr uint32_t kLBO = 128, kSBO = kKC / 8 * 128;  // bytes between core matrices along K and M / N
-constexpr long long kWaitCycles = 1ll << 31;
 constexpr size_t kSmemBudget = 220 * 1024;
-
-__device__ int g_gram64_err = 0;
-
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int code) {
-  const long long t0 = clock64();
-  for (uint32_t i = 0;; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if ((i & 15u) == 15u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > kWaitCycles) break;
-    }
-  }
-  *abort_flag = 1;
-  atomicExch(&g_gram64_err, code);
-  return false;
-}
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
@@ -220,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     gram64_kernel(int64_t n, Cols<double> A, Cols<double> B, int ld, int a0, int pa, int b0, int pb, int upper,
                   int same, int rs, const int* __restrict__ exps, int estride, int eb0,
                   const int* __restrict__ flag, double* __restrict__ part, int64_t groups_per_cta, int npanels,
-                  int row_a) {
+                  int row_a, int* __restrict__ err) {
   constexpr int kAS = NB <= 32 ? 2 : 1;  // accumulators (of kDiags * NB TMEM columns)
   constexpr int kAcc = kDiags * NB;
   constexpr uint32_t kSliceA = CA / 8 * kSBO, kSliceB = NB / 8 * kSBO;  // bytes of a slice
@@ -309,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int st = 0;
     uint32_t ph = 0;
     for (int c = 0; c < nchunks; ++c) {
-      if (c >= rs && !__all_sync(0xffffffffu, wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, 3))) break;
+      if (c >= rs && !__all_sync(0xffffffffu, wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, err, 3))) break;
       const int64_t r0 = r_begin + (int64_t)c * kKC;
       const int rows = (int)min((int64_t)kKC, r_end - r0);  // even: n is
       double* raw_st = raw + (size_t)st * stage;
@@ -337,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int st = 0;
       uint32_t ph = 0;
       for (int c = 0; c < nchunks; ++c) {
-        if (c >= rs && !wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, 3)) break;
+        if (c >= rs && !wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, err, 3)) break;
         const int64_t r0 = r_begin + (int64_t)c * kKC;
         const int rows = (int)min((int64_t)kKC, r_end - r0);
         uint32_t total = 0;  // the last row's copy stops at the used columns
@@ -358,8 +341,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t tph = 0, aph = 0;
       for (int c = 0; c < nchunks; ++c) {
         const int in_group = c % kChunks;
-        if (!wait_bar(&tile_full[buf], tph, &abort_flag, 3)) break;
-        if (in_group == 0 && c / kChunks >= kAS && !wait_bar(&acc_empty[r], aph ^ 1u, &abort_flag, 3)) break;
+        if (!wait_bar(&tile_full[buf], tph, &abort_flag, err, 3)) break;
+        if (in_group == 0 && c / kChunks >= kAS && !wait_bar(&acc_empty[r], aph ^ 1u, &abort_flag, err, 3)) break;
         tc_fence_after();
         const uint64_t bo = (uint64_t)((uint32_t)buf * tbuf >> 4);
         const uint32_t d = tmem + (uint32_t)(r * kAcc);
@@ -413,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // exponents of this lane's row and of column `lane` of this warp, before the wait
       const int ea = row < pa ? __ldg(ge + a0 + row) : kExpOne;
       const int ebl = lane < kEW && kEW * half + lane < pb ? __ldg(ge + eb0 + b0 + kEW * half + lane) : kExpOne;
-      if (!__all_sync(0xffffffffu, wait_bar(&acc_full[r], aph, &abort_flag, 2))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&acc_full[r], aph, &abort_flag, err, 2))) break;
       tc_fence_after();
       const uint32_t t0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(r * kAcc + kEW * half);
       // element: (sum_t v_t 256^(7-t)) 2^(40 - 110) 2^(ea - 1022) 2^(eb - 1022) / 256^part_
@@ -501,8 +484,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < kMaxUW; ++j)
           if (src[j] >= 0) exp_[j] = __ldg(exps + (g_begin + cur) * (int64_t)estride + ecol[j]);
       }
-      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[st], ph, &abort_flag, 1))) break;
-      if (c >= kTS && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph ^ 1u, &abort_flag, 2))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[st], ph, &abort_flag, err, 1))) break;
+      if (c >= kTS && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph ^ 1u, &abort_flag, err, 2))) break;
       const int rows = (int)min((int64_t)kKC, r_end - (r_begin + (int64_t)c * kKC));
       const double* rsb = raw + (size_t)st * stage;
       unsigned char* tb_ = tiles + (uint32_t)buf * tbuf;
@@ -550,8 +533,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-__global__ void gram64_err_reset_kernel() { g_gram64_err = 0; }
-
 bool same_cols(const Cols<double>& a, const Cols<double>& b) {
   bool same = a.nseg == b.nseg;
   for (int g = 0; same && g < a.nseg; ++g) same = a.p[g] == b.p[g] && a.w[g] == b.w[g];
@@ -582,14 +563,14 @@ int sm_count() {
 template <int CA, int NB>
 void gram64_launch(int64_t n, const Cols<double>& a, const Cols<double>& b, int ld, int a0, int pa, int b0, int pb,
                    bool upper, bool same, int rs, size_t smem, const int* exps, int estride, int eb0,
-                   const int* flag, double* part, int ctas, int64_t gpc, cudaStream_t st) {
+                   const int* flag, double* part, int ctas, int64_t gpc, int* err, cudaStream_t st) {
   static const bool attr = [&] {
     LB_CUDA(cudaFuncSetAttribute(gram64_kernel<CA, NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget));
     return true;
   }();
   (void)attr;
   gram64_kernel<CA, NB, false><<<(unsigned)ctas, kThreads, smem, st>>>(n, a, b, ld, a0, pa, b0, pb, upper ? 1 : 0, same ? 1 : 0,
-                                                           rs, exps, estride, eb0, flag, part, gpc, 0, 0);
+                                                           rs, exps, estride, eb0, flag, part, gpc, 0, 0, err);
   LB_LAUNCH_CHECK();
 }
 
@@ -603,7 +584,7 @@ size_t gram64_scratch_ints(int64_t n) { return (size_t)ceil_div(n, kGroupRows) *
 // the partials are not written, and the caller's general kernel (launched on the same flag) forms
 // them over the same number of CTAs.
 int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
-                         int max_ctas, int* scratch, cudaStream_t st) {
+                         int max_ctas, int* scratch, int* err, cudaStream_t st) {
   if (a.nseg == 0 || b.nseg == 0 || n <= 0) return 0;
   const int ld = a.ld[0];
   if (ld & 1) return 0;
@@ -644,13 +625,13 @@ int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b
       const bool diag = same && ia == ib && nbw == caw;
       if (caw == 32)
         gram64_launch<32, 32>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
-                              (int)ctas, gpc, st);
+                              (int)ctas, gpc, err, st);
       else if (nbw == 32)
         gram64_launch<64, 32>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
-                          (int)ctas, gpc, st);
+                          (int)ctas, gpc, err, st);
       else
         gram64_launch<64, 64>(n, a, b, ld, a0, ca, b0, cb, upper, diag, rs, smem, exps, estride, eb0, flag, part,
-                          (int)ctas, gpc, st);
+                          (int)ctas, gpc, err, st);
     }
   return (int)ctas;
 }
@@ -693,7 +674,7 @@ size_t dense64_scratch_bytes(int64_t n, int p) {
 // launching where A or X do not fit (odd n or lda, unaligned).  *scratch is the flag left at 1 when a
 // number is outside the digits' range: Y is then to be formed by launch_spmm_dense on that flag.
 bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
-                              int ldy, void* scratch, bool row_a, cudaStream_t st) {
+                              int ldy, void* scratch, bool row_a, int* err, cudaStream_t st) {
   if (n < 2 || (n & 1) || (lda & 1) || lda > INT_MAX || p < 1 || p > 32 || (reinterpret_cast<uintptr_t>(A) & 15) ||
       (reinterpret_cast<uintptr_t>(X) & 15))
     return false;
@@ -725,25 +706,12 @@ bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, co
   LB_LAUNCH_CHECK();
   gram64_kernel<kCB, NB, true><<<(unsigned)(panels * splits), kThreads, smem, st>>>(
       n, cols1<double>(A, (int)lda, 1), cols1<double>(X, ldx, p), (int)lda, 0, 0, 0, p, 0, 0, rs, exps, (int)estride,
-      (int)n, flag, part, ceil_div(groups, splits), (int)panels, row_a ? 1 : 0);
+      (int)n, flag, part, ceil_div(groups, splits), (int)panels, row_a ? 1 : 0, err);
   LB_LAUNCH_CHECK();
   panel_reduce_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n * p, 256), 4096), 256, 0, st>>>(n, p, splits, part, Y,
                                                                                                ldy, flag);
   LB_LAUNCH_CHECK();
   return true;
-}
-
-// Reads and clears the give-up flag (synchronises the stream); throws when a CTA gave up waiting.
-void gram64_check(cudaStream_t st) {
-  int err = 0;
-  LB_CUDA(cudaMemcpyFromSymbolAsync(&err, g_gram64_err, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
-  LB_CUDA(cudaStreamSynchronize(st));
-  if (err) {
-    gram64_err_reset_kernel<<<1, 1, 0, st>>>();
-    LB_LAUNCH_CHECK();
-    LB_CUDA(cudaStreamSynchronize(st));
-    throw CudaError("tensor-core FP64 Gram: a pipeline stage did not complete in time");
-  }
 }
 
 }  // namespace lobpcg

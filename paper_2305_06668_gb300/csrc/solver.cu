@@ -176,6 +176,18 @@ void pinned_give(double* h) {
 struct InvalidArg : std::runtime_error {
   using std::runtime_error::runtime_error;
 };
+
+// Error words of the kernels with bounded waits (common.cuh), at ictl + kErr0 of a context.
+enum { kErrGram = 0, kErrUpdate, kErrGram32, kErrWords };
+constexpr int kErr0 = 8;
+void throw_if_gave_up(int kind, int code) {
+  static const char* const what[kErrWords] = {"FP64 Gram", "FP64 update", "Gram"};
+  if (code)
+    throw CudaError(std::string("tensor-core ") + what[kind] +
+                    (code == 1   ? ": a bulk copy did not complete in time"
+                     : code == 2 ? ": an MMA did not complete in time"
+                                 : ": a pipeline stage was not released in time"));
+}
 struct NoMem : std::runtime_error {
   using std::runtime_error::runtime_error;
 };
@@ -385,7 +397,7 @@ struct lobpcg_ctx {
   double *Gpart = nullptr, *G = nullptr, *U = nullptr, *lam_all = nullptr, *up = nullptr;
   double *Tm = nullptr, *C = nullptr, *npart = nullptr, *resnorm = nullptr, *scal = nullptr;
   double *lam = nullptr, *sgn = nullptr, *S = nullptr, *colmax = nullptr;
-  int* ictl = nullptr;  // [0..3] cholqr ctl, [4] sweeps, [5] finite flag
+  int* ictl = nullptr;  // [0..3] cholqr ctl, [4] sweeps, [5] finite flag, [kErr0 ..] error words
   LockState* lock = nullptr;
   DevBuf x0buf;        // column-major FP64 initial block when X0 == NULL
   DevBuf xbest;        // the FP32 phase's X with the smallest largest-sought residual (reading R22)
@@ -393,7 +405,6 @@ struct lobpcg_ctx {
   DevBuf tri_scratch;  // its FP32 scratch (tridiag_scratch_floats(n, a))
   DevBuf gram_buf;         // exponents of the digit Grams (allocated when first used)
   int* gram_ints = nullptr;
-  bool used_digits = false, used_update64 = false;  // launched: the give-up flags are checked at the end
   int* gram_scratch() {
     if (!gram_ints) {
       gram_buf.ensure(gram64_scratch_ints(A.n) * sizeof(int));
@@ -428,12 +439,25 @@ struct lobpcg_ctx {
   bool trace_orth = false;  // LOBPCG_TRACE_ORTH=1: also trace max |V^T V - I|
 
   void sync() { LB_CUDA(cudaStreamSynchronize(st)); }
+  // Error words of the tensor-core kernels, one per kind, this context's own.  Cleared by the first
+  // launch of a call that may raise them.
+  bool err_used[kErrWords] = {};
+  int* err_word(int kind) {
+    if (!err_used[kind]) LB_CUDA(cudaMemsetAsync(ictl + kErr0 + kind, 0, sizeof(int), st));
+    err_used[kind] = true;
+    return ictl + kErr0 + kind;
+  }
+  void begin() { std::fill(err_used, err_used + kErrWords, false); }
   // the end of a call: waits for its work and reports a tensor-core kernel that gave up waiting
   void finish() {
-    if (used_digits) gram64_check(st);
-    if (used_update64) update64_check(st);
-    if (!used_digits && !used_update64) sync();
-    used_digits = used_update64 = false;
+    int* h = reinterpret_cast<int*>(host + kPinnedBytes / sizeof(double)) - kErrWords;
+    bool any = false;
+    for (bool u : err_used) any |= u;
+    if (any) LB_CUDA(cudaMemcpyAsync(h, ictl + kErr0, kErrWords * sizeof(int), cudaMemcpyDeviceToHost, st));
+    sync();
+    for (int k = 0; k < kErrWords; ++k)
+      if (err_used[k]) throw_if_gave_up(k, h[k]);
+    begin();
   }
 
   size_t small_bytes() const {
@@ -514,8 +538,8 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
     // digit products on the tensor cores from the size where they are the faster form
     parts = 0;
     if ((double)c.A.n * s * q * job.nprod >= (c.df_on ? kDigitUpdateDf : kDigitUpdate)) {
-      parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
-      c.used_update64 |= parts > 0;
+      parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.err_word(kErrUpdate),
+                                   c.st);
     }
     if (!parts)
     parts = c.df_on ? launch_update_df(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st)
@@ -546,8 +570,8 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
     if constexpr (std::is_same<T, double>::value) {
       if (dense_digits_pay(c.A.n, p)) {
         c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
-        if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false, c.st)) {
-          c.used_digits = true;
+        if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false,
+                                     c.err_word(kErrGram), c.st)) {
           launch_spmm_dense<T>(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.st, c.dense_buf.as<int>());
           return;
         }
@@ -628,17 +652,15 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
     const double mults = (double)c.A.n * pa * pb * (upper ? 0.5 : 1.0);
     if (mults >= (c.df_on ? kDigitGramDf : kDigitGram)) {
       int* flag = c.gram_scratch();
-      parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.st);
-      if (parts) {
-        c.used_digits = true;
-        gram_partials<T>(c.A.n, a, b, upper, c.Gpart, parts, c.st, flag);
-      }
+      parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.err_word(kErrGram), c.st);
+      if (parts) gram_partials<T>(c.A.n, a, b, upper, c.Gpart, parts, c.st, flag);
     }
     if (!parts && c.df_on) parts = gram_partials_df(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
   } else {
     // FP32: the tcgen05 kernel when the blocks fit it (every block the solver allocates);
-    // its give-up flag is checked once per solve (umma_check)
-    if (c.opt.tc_gram != 0) parts = gram_partials_umma(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
+    // its error word is checked once per solve (finish)
+    if (c.opt.tc_gram != 0)
+      parts = gram_partials_umma(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.err_word(kErrGram32), c.st);
   }
   if (!parts) parts = gram_partials<T>(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
   reduce_partials(c.Gpart, parts, pa * pb, out, c.st);
@@ -1404,6 +1426,7 @@ extern "C" lobpcg_status lobpcg_solve(lobpcg_ctx* c, int k, double tol, const do
     LB_CUDA(cudaEventCreate(&e1));
     LB_CUDA(cudaEventRecord(e0, c->st));
     c->b64.ensure(n, m);
+    c->begin();  // a solve that failed may have left its words in use
     const double* x0 = X0;
     if (!x0) {
       c->x0buf.ensure((size_t)n * m * sizeof(double));
@@ -1499,7 +1522,6 @@ extern "C" lobpcg_status lobpcg_solve(lobpcg_ctx* c, int k, double tol, const do
     LB_CUDA(cudaMemcpyAsync(resnorms, c->resnorm, k * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     LB_CUDA(cudaEventRecord(e1, c->st));
     c->finish();
-    if (c->opt.precision == LOBPCG_MIXED) umma_check(c->st);
     float ms = 0.f;
     LB_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     cudaEventDestroy(e0);
@@ -1717,9 +1739,14 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
     PoolBuf work(st);
     if (dense_digits_pay(n, p)) {
       work.alloc(dense64_scratch_bytes(n, p));
-      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, false, st)) {
-        launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st, work.as<int>());
-        gram64_check(st);
+      int* word = work.as<int>();  // the digits' flag, then the error word
+      LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
+      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, false, word + 1, st)) {
+        launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st, word);
+        int err = 0;
+        LB_CUDA(cudaMemcpyAsync(&err, word + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+        LB_CUDA(cudaStreamSynchronize(st));
+        throw_if_gave_up(kErrGram, err);
         return LOBPCG_OK;
       }
     }
@@ -1739,11 +1766,14 @@ extern "C" lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, 
     if (!dense_digits_pay(n, p)) return LOBPCG_OK;
     PoolBuf work(st);
     work.alloc(dense64_scratch_bytes(n, p));
-    if (!launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, true, st)) return LOBPCG_OK;
-    int flag = 0;
-    LB_CUDA(cudaMemcpyAsync(&flag, work.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-    gram64_check(st);
-    *done = flag ? 0 : 1;
+    int* word = work.as<int>();  // the digits' flag, then the error word
+    LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
+    if (!launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, true, word + 1, st)) return LOBPCG_OK;
+    int h[2] = {0, 0};
+    LB_CUDA(cudaMemcpyAsync(h, word, sizeof h, cudaMemcpyDeviceToHost, st));
+    LB_CUDA(cudaStreamSynchronize(st));
+    throw_if_gave_up(kErrGram, h[1]);
+    *done = h[0] ? 0 : 1;
     return LOBPCG_OK;
   });
 }
@@ -1844,10 +1874,10 @@ extern "C" lobpcg_status lobpcg_gram_f32_tcgen05(int64_t n, int p, const float* 
             "lobpcg_gram_f32_tcgen05: X and Y must be 16-byte aligned with one row stride, a multiple of 4");
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
     const int parts = gram_partials_umma(n, cols1<float>(X, ldx, p), cols1<float>(Y, ldy, q), false, s.c.Gpart,
-                                         s.c.max_ctas, s.c.st);
+                                         s.c.max_ctas, s.c.err_word(kErrGram32), s.c.st);
     if (!parts) throw InvalidArg("lobpcg_gram_f32_tcgen05: operands do not fit the kernel");
     reduce_partials(s.c.Gpart, parts, p * q, C, s.c.st);
-    umma_check(s.c.st);
+    s.c.finish();
     return LOBPCG_OK;
   });
 }

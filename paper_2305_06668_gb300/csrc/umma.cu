@@ -53,45 +53,23 @@ constexpr int kSplit0 = 6;      // first splitter warp
 constexpr int kSplitWarps = 8;  // warps 6..13
 constexpr int kThreads = 32 * (kSplit0 + kSplitWarps);
 constexpr uint32_t kLBO = 128;  // bytes between core matrices along K
-constexpr long long kWaitCycles = 1ll << 31;  // ~1 s at the SM clock: a wait that long has failed
 constexpr size_t kSmemBudget = 220 * 1024;
 
 __host__ __device__ constexpr uint32_t tmem_cols(int cols) {
   return cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
 }
 
-// Set by a CTA that gave up waiting (1: a bulk copy, 2: an MMA, 3: a pipeline stage).
-// Device code names it directly; the host reads it with cudaMemcpyFromSymbol (its
-// host-side name is not a device address and is never passed to a kernel).
-__device__ int g_umma_err = 0;
-
 // x rounded to TF32 (10 stored mantissa bits), to nearest with ties away from zero: half a
 // unit of the 13 dropped bits is added to the magnitude bits, then they are cleared (a
 // carry into the exponent is the correct rounding up).  Finite x only.
 __device__ __forceinline__ uint32_t to_tf32(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
-
-// Wait bounded in time (kWaitCycles) that also returns (false) once another thread of the
-// CTA gave up.
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int code) {
-  const long long t0 = clock64();
-  for (uint32_t i = 0;; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if ((i & 15u) == 15u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > kWaitCycles) break;
-    }
-  }
-  *abort_flag = 1;
-  atomicExch(&g_umma_err, code);
-  return false;
-}
 
 // STACK: both operands at most 64 columns, one stacked MMA per K step; otherwise three.
 template <int NP, int KC, bool STACK>
 __global__ void __launch_bounds__(kThreads, 1) gram_umma_kernel(int64_t n, Cols<float> A, Cols<float> B, int ld,
                                                                 int upper, int rs, int ts, int groups,
                                                                 double* __restrict__ part,
-                                                                int64_t rows_per_cta) {
+                                                                int64_t rows_per_cta, int* __restrict__ err) {
   constexpr int N = 16 * NP;             // columns of C per running sum (>= pb)
   constexpr int MN = STACK ? 128 : N;    // MMA N, and TMEM columns of one accumulator
   constexpr uint32_t kSBO = 32 * KC;     // bytes between core matrices along M / N
@@ -184,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1) gram_umma_kernel(int64_t n, Cols<
       int st = 0;
       uint32_t ph = 0;  // ring slot of chunk c and the parity of its round (c / rs)
       for (int c = 0; c < nchunks; ++c) {
-        if (c >= rs && !wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, 3)) break;
+        if (c >= rs && !wait_bar(&raw_empty[st], ph ^ 1u, &abort_flag, err, 3)) break;
         const int64_t r0 = r_begin + (int64_t)c * KC;
         const int rows = (int)min((int64_t)KC, r_end - r0);
         // every row in full (ld floats) but the last, of which only the used columns
@@ -212,8 +190,8 @@ __global__ void __launch_bounds__(kThreads, 1) gram_umma_kernel(int64_t n, Cols<
       int buf = 0, r = 0;
       uint32_t tph = 0, aph = 0;  // tile / accumulator slots and round parities
       for (int c = 0; c < nchunks; ++c) {
-        if (!wait_bar(&tile_full[buf], tph, &abort_flag, 3)) break;
-        if (c >= kAS && !wait_bar(&acc_empty[r], aph ^ 1u, &abort_flag, 3)) break;
+        if (!wait_bar(&tile_full[buf], tph, &abort_flag, err, 3)) break;
+        if (c >= kAS && !wait_bar(&acc_empty[r], aph ^ 1u, &abort_flag, err, 3)) break;
         tc_fence_after();
         const uint64_t bo = (uint64_t)((uint32_t)(buf * tbuf * 4) >> 4);
         const uint32_t d = tmem + (uint32_t)(r * MN);
@@ -245,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1) gram_umma_kernel(int64_t n, Cols<
     int r = 0, c = 0;
     uint32_t aph = 0;
     for (; c < nchunks; ++c) {
-      if (!__all_sync(0xffffffffu, wait_bar(&acc_full[r], aph, &abort_flag, 2))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&acc_full[r], aph, &abort_flag, err, 2))) break;
       tc_fence_after();
       const uint32_t a0 = tmem + lane_base + (uint32_t)(r * MN);
 #pragma unroll
@@ -339,8 +317,8 @@ __global__ void __launch_bounds__(kThreads, 1) gram_umma_kernel(int64_t n, Cols<
     int st = g % rs, buf = g % ts;
     uint32_t ph = 0, tph = 0;
     for (int c = g; c < nchunks; c += groups) {
-      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[st], ph, &abort_flag, 1))) break;
-      if (c >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph ^ 1u, &abort_flag, 2))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[st], ph, &abort_flag, err, 1))) break;
+      if (c >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph ^ 1u, &abort_flag, err, 2))) break;
       const int rows = (int)min((int64_t)KC, r_end - (r_begin + (int64_t)c * KC));
       const float* rsb = raw + (size_t)st * nu * seg_floats;
       uint32_t* tb = tiles + buf * tbuf;
@@ -405,8 +383,6 @@ __global__ void __launch_bounds__(kThreads, 1) gram_umma_kernel(int64_t n, Cols<
   }
 }
 
-__global__ void umma_err_reset_kernel() { g_umma_err = 0; }
-
 // Launch plan: rows per chunk, raw stages, dynamic shared memory.
 struct UmmaPlan {
   int kc = 0, rs = 0, ts = 0, groups = 1, nu = 0;
@@ -455,7 +431,7 @@ bool umma_plan(const Cols<float>& a, const Cols<float>& b, int ld, UmmaPlan& pl)
 
 template <int NP, int KC, bool STACK>
 int umma_launch(int64_t n, const Cols<float>& a, const Cols<float>& b, int ld, bool upper, double* part, int max_ctas,
-                const UmmaPlan& pl, cudaStream_t st) {
+                const UmmaPlan& pl, int* err, cudaStream_t st) {
   static const bool attr = [&] {
     LB_CUDA(cudaFuncSetAttribute(gram_umma_kernel<NP, KC, STACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kSmemBudget));
@@ -471,21 +447,22 @@ int umma_launch(int64_t n, const Cols<float>& a, const Cols<float>& b, int ld, b
   const int64_t rpc = (ceil_div(n, ctas) + KC - 1) / KC * KC;
   ctas = std::max<int64_t>(1, ceil_div(n, rpc));
   gram_umma_kernel<NP, KC, STACK>
-      <<<(unsigned)ctas, kThreads, pl.smem, st>>>(n, a, b, ld, upper ? 1 : 0, pl.rs, pl.ts, pl.groups, part, rpc);
+      <<<(unsigned)ctas, kThreads, pl.smem, st>>>(n, a, b, ld, upper ? 1 : 0, pl.rs, pl.ts, pl.groups, part, rpc,
+                                          err);
   LB_LAUNCH_CHECK();
   return (int)ctas;
 }
 
 template <int NP>
 int umma_launch_kc(int64_t n, const Cols<float>& a, const Cols<float>& b, int ld, bool upper, double* part,
-                   int max_ctas, const UmmaPlan& pl, cudaStream_t st) {
+                   int max_ctas, const UmmaPlan& pl, int* err, cudaStream_t st) {
   if constexpr (NP <= 4) {
     if (pl.stack)
-      return pl.kc == 64 ? umma_launch<NP, 64, true>(n, a, b, ld, upper, part, max_ctas, pl, st)
-                         : umma_launch<NP, 32, true>(n, a, b, ld, upper, part, max_ctas, pl, st);
+      return pl.kc == 64 ? umma_launch<NP, 64, true>(n, a, b, ld, upper, part, max_ctas, pl, err, st)
+                         : umma_launch<NP, 32, true>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
   }
-  return pl.kc == 64 ? umma_launch<NP, 64, false>(n, a, b, ld, upper, part, max_ctas, pl, st)
-                     : umma_launch<NP, 32, false>(n, a, b, ld, upper, part, max_ctas, pl, st);
+  return pl.kc == 64 ? umma_launch<NP, 64, false>(n, a, b, ld, upper, part, max_ctas, pl, err, st)
+                     : umma_launch<NP, 32, false>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
 }
 
 bool umma_aligned(const Cols<float>& c, int ld) {
@@ -500,7 +477,7 @@ bool umma_aligned(const Cols<float>& c, int ld) {
 // launching when the operands do not share one 16-byte aligned row stride (a multiple of
 // 4 floats), are wider than 96 columns, or need more shared memory than a CTA has.
 int gram_partials_umma(int64_t n, const Cols<float>& a, const Cols<float>& b, bool upper, double* part,
-                       int max_ctas, cudaStream_t st) {
+                       int max_ctas, int* err, cudaStream_t st) {
   if (a.nseg == 0 || b.nseg == 0 || n <= 0) return 0;
   const int ld = a.ld[0];
   if (ld % 4 != 0 || !umma_aligned(a, ld) || !umma_aligned(b, ld)) return 0;
@@ -509,28 +486,12 @@ int gram_partials_umma(int64_t n, const Cols<float>& a, const Cols<float>& b, bo
   UmmaPlan pl;
   if (!umma_plan(a, b, ld, pl)) return 0;
   switch ((pb + 15) / 16) {
-    case 1: return umma_launch_kc<1>(n, a, b, ld, upper, part, max_ctas, pl, st);
-    case 2: return umma_launch_kc<2>(n, a, b, ld, upper, part, max_ctas, pl, st);
-    case 3: return umma_launch_kc<3>(n, a, b, ld, upper, part, max_ctas, pl, st);
-    case 4: return umma_launch_kc<4>(n, a, b, ld, upper, part, max_ctas, pl, st);
-    case 5: return umma_launch_kc<5>(n, a, b, ld, upper, part, max_ctas, pl, st);
-    default: return umma_launch_kc<6>(n, a, b, ld, upper, part, max_ctas, pl, st);
-  }
-}
-
-// Reads and clears the give-up flag of the tcgen05 Gram (synchronises the stream); throws
-// when a CTA gave up waiting, so the failure surfaces as ECUDA.
-void umma_check(cudaStream_t st) {
-  int flag = 0;
-  LB_CUDA(cudaMemcpyFromSymbolAsync(&flag, g_umma_err, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
-  LB_CUDA(cudaStreamSynchronize(st));
-  if (flag) {
-    umma_err_reset_kernel<<<1, 1, 0, st>>>();
-    LB_LAUNCH_CHECK();
-    LB_CUDA(cudaStreamSynchronize(st));
-    throw CudaError(flag == 1   ? "tensor-core Gram: a bulk copy did not complete in time"
-                    : flag == 2 ? "tensor-core Gram: an MMA did not complete in time"
-                                : "tensor-core Gram: a pipeline stage was not released in time");
+    case 1: return umma_launch_kc<1>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
+    case 2: return umma_launch_kc<2>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
+    case 3: return umma_launch_kc<3>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
+    case 4: return umma_launch_kc<4>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
+    case 5: return umma_launch_kc<5>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
+    default: return umma_launch_kc<6>(n, a, b, ld, upper, part, max_ctas, pl, err, st);
   }
 }
 

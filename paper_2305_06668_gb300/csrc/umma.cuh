@@ -71,6 +71,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
   }
 }
 
+constexpr long long kWaitCycles = 1ll << 31;  // ~1 s at the SM clock: a wait that long has failed
+
+// Wait bounded in time (kWaitCycles) that also returns (false) once another thread of the CTA gave
+// up.  The thread that gives up leaves `code` in the call's own error word: calls on other streams
+// and threads have theirs, and the host reads it at the end of the call.
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
+  const long long t0 = clock64();
+  for (uint32_t i = 0;; ++i) {
+    if (mbar_try(bar, parity)) return true;
+    if ((i & 15u) == 15u) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > kWaitCycles) break;
+    }
+  }
+  *abort_flag = 1;
+  atomicExch(err, code);
+  return false;
+}
+
 // TMEM allocation of `ncols` columns (power of two >= 32) by one full warp; the address
 // is written to *slot (shared memory).
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {

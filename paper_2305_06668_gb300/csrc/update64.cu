@@ -54,25 +54,8 @@ constexpr uint32_t kSlice = kTile / 8 * kSBO;  // bytes of one digit of a chunk 
 constexpr uint32_t kBuf = kSlices * kSlice;
 constexpr int kAcc = kDiags * kQ;              // TMEM columns of one accumulator
 constexpr int kBad = -1;
-constexpr long long kWaitCycles = 1ll << 31;
 constexpr size_t kStatic = 14 * 1024;  // static shared memory, at most
 constexpr size_t kSmemBudget = 227 * 1024;
-
-__device__ int g_update64_err = 0;
-
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int code) {
-  const long long t0 = clock64();
-  for (uint32_t i = 0;; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if ((i & 15u) == 15u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > kWaitCycles) break;
-    }
-  }
-  *abort_flag = 1;
-  atomicExch(&g_update64_err, code);
-  return false;
-}
 
 // bytes of U's digits: kSlices slices of kQ columns x KP rows
 __host__ __device__ constexpr uint32_t u_slice(int kp) { return (uint32_t)(kQ * kp * 2); }
@@ -82,7 +65,7 @@ template <int NC, bool NORM>
 __global__ void __launch_bounds__(kThreads, 1)
     update64_kernel(int64_t n, UpdateJob<double> job, const double* __restrict__ U, int s, int q, double alpha,
                     const double* __restrict__ lam, double* __restrict__ norm_part, int64_t tiles_per_cta,
-                    int ts) {
+                    int ts, int* __restrict__ err) {
   constexpr int KP = NC * kKC;
   constexpr uint32_t kSliceU = u_slice(KP), kSBOU = KP / 8 * 128;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -199,7 +182,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t tph = 1;  // parity of the tile_empty phase to wait for (the first ts chunks do not wait)
     int chunk = 0;
     for (int T = 0; T < nT; ++T) {
-      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[warp], (uint32_t)T & 1u, &abort_flag, 1))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&raw_full[warp], (uint32_t)T & 1u, &abort_flag, err, 1))) break;
       const bool live = r_begin + (int64_t)(T / nprod) * kTile + 8 * warp + r < r_end;
       double x[NC][8];
       int E = 0;
@@ -236,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (E <= 0 || bad) E = kExpOne;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        if (chunk >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph, &abort_flag, 2))) break;
+        if (chunk >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph, &abort_flag, err, 2))) break;
         if (c == 0) {
           if (lane < 8) row_exp[T & (kRing - 1)][8 * warp + lane] = (int16_t)(bad ? kBad : E);
           __syncwarp();
@@ -270,10 +253,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       for (int T = 0; T < nT && ok; ++T) {
         const int a = T & 1;
-        if (T >= 2 && !wait_bar(&acc_empty[a], aph ^ 1u, &abort_flag, 3)) break;
+        if (T >= 2 && !wait_bar(&acc_empty[a], aph ^ 1u, &abort_flag, err, 3)) break;
         const uint32_t d = tmem + (uint32_t)(a * kAcc);
         for (int c = 0; c < NC; ++c) {
-          if (!wait_bar(&tile_full[buf], tph, &abort_flag, 3)) {
+          if (!wait_bar(&tile_full[buf], tph, &abort_flag, err, 3)) {
             ok = false;
             break;
           }
@@ -317,8 +300,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = 0; t < 2; ++t) {
         if (t >= nprod) break;
         const int T = it * nprod + t;
-        ok = ok && __all_sync(0xffffffffu, wait_bar(&exp_full[T & (kRing - 1)], (uint32_t)(T / kRing) & 1u, &abort_flag, 2));
-        ok = ok && __all_sync(0xffffffffu, wait_bar(&acc_full[T & 1], (uint32_t)(T / 2) & 1u, &abort_flag, 2));
+        ok = ok && __all_sync(0xffffffffu, wait_bar(&exp_full[T & (kRing - 1)], (uint32_t)(T / kRing) & 1u, &abort_flag, err, 2));
+        ok = ok && __all_sync(0xffffffffu, wait_bar(&acc_full[T & 1], (uint32_t)(T / 2) & 1u, &abort_flag, err, 2));
         if (ok) er[t] = all_bad ? kBad : row_exp[T & (kRing - 1)][row];
       }
       if (!ok) break;
@@ -348,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (any_bad) {
         __syncwarp();
         if (lane == 0) mbar_arrive(&rows_read[quad]);
-        ok = __all_sync(0xffffffffu, wait_bar(&rows_read[quad], rph, &abort_flag, 4));
+        ok = __all_sync(0xffffffffu, wait_bar(&rows_read[quad], rph, &abort_flag, err, 4));
         rph ^= 1u;
         if (!ok) break;
       }
@@ -454,11 +437,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-__global__ void update64_err_reset_kernel() { g_update64_err = 0; }
-
 template <int NC, bool NORM>
 int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, cudaStream_t st) {
+                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, int* err, cudaStream_t st) {
   static const bool attr = [&] {
     LB_CUDA(cudaFuncSetAttribute(update64_kernel<NC, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBudget - kStatic)));
     return true;
@@ -471,7 +452,7 @@ int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, in
   const int64_t per = ceil_div(tiles, std::min<int64_t>(std::min<int64_t>(max_ctas, sms), tiles));
   const int64_t ctas = ceil_div(tiles, per);
   update64_kernel<NC, NORM><<<(unsigned)ctas, kThreads, smem, st>>>(n, job, U, s, q, alpha, lam, norm_part, per,
-                                                                     ts);
+                                                                    ts, err);
   LB_LAUNCH_CHECK();
   return (int)ctas;
 }
@@ -481,7 +462,7 @@ int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, in
 // The block update through digit products; returns 0 without launching where the blocks do not fit
 // (unaligned or odd row strides, products of different layout, more shared memory than a CTA has).
 int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                         const double* lam, double* norm_part, int max_ctas, cudaStream_t st) {
+                         const double* lam, double* norm_part, int max_ctas, int* err, cudaStream_t st) {
   if (n <= 0 || q < 1 || q > kQ || s < 1 || s > kMaxS || job.in[0].nseg < 1) return 0;
   if (norm_part && (job.nprod != 2 || job.base[0] || job.base[1])) return 0;
   size_t raw = 0;
@@ -500,24 +481,12 @@ int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* 
   const size_t smem = fixed + (size_t)ts * kBuf;
   if (smem > kSmemBudget - kStatic) return 0;
 #define LB_UPDATE64(NC)                                                                                          \
-  return norm_part ? update64_launch<NC, true>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, st)        \
-                   : update64_launch<NC, false>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, st)
+  return norm_part ? update64_launch<NC, true>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, err, st)        \
+                   : update64_launch<NC, false>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, err, st)
   if (nc == 1) LB_UPDATE64(1);
   if (nc == 2) LB_UPDATE64(2);
   LB_UPDATE64(3);
 #undef LB_UPDATE64
-}
-
-void update64_check(cudaStream_t st) {
-  int err = 0;
-  LB_CUDA(cudaMemcpyFromSymbolAsync(&err, g_update64_err, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
-  LB_CUDA(cudaStreamSynchronize(st));
-  if (err) {
-    update64_err_reset_kernel<<<1, 1, 0, st>>>();
-    LB_LAUNCH_CHECK();
-    LB_CUDA(cudaStreamSynchronize(st));
-    throw CudaError("tensor-core FP64 update: a pipeline stage did not complete in time");
-  }
 }
 
 }  // namespace lobpcg

@@ -17,10 +17,23 @@ def test_named_barriers_join_the_whole_epilogue(name):
     assert found and all((i.strip(), c.strip()) == ("3", str(EPILOGUE[name])) for i, c in found), found
 
 
-@pytest.mark.parametrize("name", [*EPILOGUE, "umma.cuh"])
-def test_polls_stand_in_bounded_loops(name):
-    text = (gpu_build.CSRC / name).read_text()
-    polls = [m.start() for m in re.finditer(r"if \(mbar_try\(", text)]
+SOURCES = sorted(p.name for p in gpu_build.CSRC.glob("*.cu*"))
+
+
+def test_polls_stand_in_bounded_loops():
+    polls = 0
+    for name in SOURCES:
+        text = (gpu_build.CSRC / name).read_text()
+        for m in re.finditer(r"if \(mbar_try\(", text):
+            polls += 1
+            assert re.search(r"clock64\(\) - t0 > (kWaitCycles|max_cycles)", text[m.start():m.start() + 400]), name
     assert polls
-    for at in polls:
-        assert re.search(r"clock64\(\) - t0 > (kWaitCycles|max_cycles)", text[at:at + 400]), text[at:at + 400]
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_error_words_belong_to_the_call(name):
+    """No kernel writes, and no host code reads or clears, a word that calls on other streams and threads
+    share: a process-wide error flag is cleared by whichever call looks first."""
+    text = (gpu_build.CSRC / name).read_text()
+    word = r"^(?:static\s+)?__device__\s+(?:volatile\s+)?(?:int|unsigned|uint32_t)\s+\w+\s*(?:=[^;(]*)?;"
+    assert not re.findall(word, text, re.M) and "cudaMemcpyFromSymbol" not in text
