@@ -124,11 +124,11 @@ typedef struct {
                                  the FP32 pipes (about 2^-48 per product, chunk sums in FP64).
                                  0 (default): double-float in the FP64 refinement of the MIXED
                                  form, FP64 fused multiply-adds in the FP64 form; 1: double-float
-                                 in every FP64 phase; -1: FP64 fused multiply-adds everywhere.
-                                 Grams and updates of some size (2e7 to 6e7 multiply-adds) take
-                                 exact digit products on the tensor cores in either form, with
-                                 errors no larger than the fused multiply-adds'; the double-float
-                                 phases keep their tau and CSR products */
+                                 in every FP64 phase.  With 0 and 1, Grams, updates and dense
+                                 products of some size (1.5e7 to 6e7 multiply-adds) take digit
+                                 products on the tensor cores instead (accuracy: see
+                                 lobpcg_gram_f64); the double-float phases keep their tau and CSR
+                                 products.  -1: FP64 fused multiply-adds everywhere */
   int tc_gram;                /* FP32 Gram matrices of the MIXED form: non-zero (default) on the
                                  tcgen05 tensor cores (lobpcg_gram_f32_tcgen05), 0 with warp-level
                                  mma.sync (lobpcg_gram_f32); both 3xTF32 */

@@ -438,6 +438,8 @@ struct lobpcg_ctx {
   FILE* trace = nullptr;  // per-iteration JSON lines (LOBPCG_TRACE=path)
   bool trace_orth = false;  // LOBPCG_TRACE_ORTH=1: also trace max |V^T V - I|
 
+  // opt.df_products = -1 asks for FP64 fused multiply-adds in every FP64 product
+  bool digits_on() const { return opt.df_products >= 0; }
   void sync() { LB_CUDA(cudaStreamSynchronize(st)); }
   // Error words of the tensor-core kernels, one per kind, this context's own.  Cleared by the first
   // launch of a call that may raise them.
@@ -537,13 +539,12 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   if constexpr (std::is_same<T, double>::value) {
     // digit products on the tensor cores from the size where they are the faster form
     parts = 0;
-    if ((double)c.A.n * s * q * job.nprod >= (c.df_on ? kDigitUpdateDf : kDigitUpdate)) {
+    if (c.digits_on() && (double)c.A.n * s * q * job.nprod >= (c.df_on ? kDigitUpdateDf : kDigitUpdate))
       parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.err_word(kErrUpdate),
                                    c.st);
-    }
     if (!parts)
-    parts = c.df_on ? launch_update_df(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st)
-                    : launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
+      parts = c.df_on ? launch_update_df(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st)
+                      : launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
   } else {
     parts = launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
   }
@@ -568,7 +569,7 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
                           false, var);
   else {
     if constexpr (std::is_same<T, double>::value) {
-      if (dense_digits_pay(c.A.n, p)) {
+      if (c.digits_on() && dense_digits_pay(c.A.n, p)) {
         c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
         if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false,
                                      c.err_word(kErrGram), c.st)) {
@@ -650,7 +651,7 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
     // outside the digits' range raises their flag, and the FMA kernel behind them (else an empty
     // launch) forms the partials
     const double mults = (double)c.A.n * pa * pb * (upper ? 0.5 : 1.0);
-    if (mults >= (c.df_on ? kDigitGramDf : kDigitGram)) {
+    if (c.digits_on() && mults >= (c.df_on ? kDigitGramDf : kDigitGram)) {
       int* flag = c.gram_scratch();
       parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.err_word(kErrGram), c.st);
       if (parts) gram_partials<T>(c.A.n, a, b, upper, c.Gpart, parts, c.st, flag);
