@@ -165,11 +165,13 @@ int gram_partials_umma(int64_t n, const Cols<float>& a, const Cols<float>& b, bo
                        int max_ctas, int* err, cudaStream_t st);
 // FP64 Gram partials through exact digit products on the tensor cores (gram64.cu).  Returns the
 // number of CTAs, or 0 without launching where the blocks do not fit.  scratch:
-// gram64_scratch_ints(n) ints.  *scratch is the flag left at 1 when some column is outside the
-// digits' range: the partials are then to be formed by gram_partials with run_flag = scratch.
+// gram64_scratch_ints(n) ints.  *scratch is a flag of two bits: 1 when some column is outside the
+// digits' range and, with `spread`, 2 when two columns are so far apart inside 256 rows that an FMA
+// chain would be more exact (gram64.cu).  Where it is not zero the partials are to be formed by
+// gram_partials with run_flag = scratch.
 size_t gram64_scratch_ints(int64_t n);
 int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
-                         int max_ctas, int* scratch, int* err, cudaStream_t st);
+                         int max_ctas, int* scratch, bool spread, int* err, cudaStream_t st);
 // out[e] = sum_g part[g][e] for e < count (FP64, fixed order).
 void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st);
 

@@ -72,15 +72,32 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
 }
 
+// Two columns are close enough in a group where at least kSpreadRows of its rows hold entries of both
+// within kSpreadBits binades of the column's largest there.  With 2^a <= mx < 2^(a+1) and my likewise,
+// those rows alone give sum |x||y| >= 32 2^-6 2^(a+b), and the digits' error is at most
+// 256 mx my 2^-53 <= 2^11 2^-53 of that sum: below the bound of a chain of FMAs over 2^11 rows, and in
+// the mean below their error.  Gaussian columns share 97 rows or more of 256 in the mean.
+constexpr int kSpreadBits = 3, kSpreadRows = 32;
+constexpr int kMaskWords = kGroupRows / 32;
+constexpr int kOutOfRange = 1, kSpread = 2;  // bits of the flag
+
 // exps[g * stride + j]: biased exponent of column j (A's columns, then B's) over the rows of group
 // g, one CTA per group.  A thread keeps one 16-byte pair of columns and strides over the rows with
 // eight loads in flight.
+// CHECK (one segment an operand): also raises kSpread where two columns are too far apart.  The
+// exponents of the group stay in shared memory (two bytes an entry), each column becomes 256 bits, and a
+// pair of columns is the population count of two of those.  The rows of a last, incomplete group are
+// judged with those before them, by a CTA of its own over the last 256.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) exp_kernel(int64_t n, Cols<double> A, Cols<double> B, int ld, int same,
                                                   int* __restrict__ exps, int stride, int* __restrict__ flag) {
+  extern __shared__ uint32_t ex2[];  // CHECK: [kGroupRows][pairs] exponents of two columns
   __shared__ uint32_t key[2 * kMaxS];
-  const int64_t r0 = (int64_t)blockIdx.x * kGroupRows;
+  const bool window = CHECK && (int64_t)blockIdx.x * kGroupRows >= n;
+  const int64_t r0 = window ? n - kGroupRows : (int64_t)blockIdx.x * kGroupRows;
   const int rows = (int)min((int64_t)kGroupRows, n - r0);
   const int pa = A.width(), total = pa + (same ? 0 : B.width());
+  const int va = (pa + 1) / 2, pairs = va + (same ? 0 : (B.width() + 1) / 2);
   for (int j = threadIdx.x; j < 2 * kMaxS; j += blockDim.x) key[j] = 0u;
   __syncthreads();
   int base = 0;
@@ -93,18 +110,21 @@ __global__ void __launch_bounds__(256) exp_kernel(int64_t n, Cols<double> A, Col
         const double2* p = reinterpret_cast<const double2*>(c.p[s] + r0 * ld) + v;
         const int64_t step = ld / 2;
         uint32_t k0 = 0u, k1 = 0u;
+        auto take = [&](const double2& x, int r) {
+          k0 = max(k0, exp_key(x.x)), k1 = max(k1, exp_key(x.y));
+          if (CHECK)
+            ex2[r * pairs + (o ? va : 0) + v] = (((uint32_t)__double2hiint(x.x) >> 20) & 0x7ffu) |
+                                                ((((uint32_t)__double2hiint(x.y) >> 20) & 0x7ffu) << 16);
+        };
         int r = grp;
         for (; r + 7 * groups < rows; r += 8 * groups) {
           double2 x[8];
 #pragma unroll
           for (int u = 0; u < 8; ++u) x[u] = __ldg(p + (r + u * groups) * step);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) k0 = max(k0, exp_key(x[u].x)), k1 = max(k1, exp_key(x[u].y));
+          for (int u = 0; u < 8; ++u) take(x[u], r + u * groups);
         }
-        for (; r < rows; r += groups) {
-          const double2 x = __ldg(p + r * step);
-          k0 = max(k0, exp_key(x.x)), k1 = max(k1, exp_key(x.y));
-        }
+        for (; r < rows; r += groups) take(__ldg(p + r * step), r);
         atomicMax(&key[base + 2 * v], k0);
         if (2 * v + 1 < w) atomicMax(&key[base + 2 * v + 1], k1);
       }
@@ -114,8 +134,44 @@ __global__ void __launch_bounds__(256) exp_kernel(int64_t n, Cols<double> A, Col
   __syncthreads();
   for (int j = threadIdx.x; j < total; j += blockDim.x) {
     const int e = group_exp(key[j]);
-    if (e < 0) *flag = 1;
-    exps[(int64_t)blockIdx.x * stride + j] = e;
+    if (e < 0) atomicOr(flag, kOutOfRange);
+    if (!window) exps[(int64_t)blockIdx.x * stride + j] = e;
+  }
+  if constexpr (CHECK) {
+    if (rows < kGroupRows) return;
+    __shared__ __align__(16) uint32_t mask[2 * kMaxS][kMaskWords];
+    for (int u = threadIdx.x; u < pairs * kMaskWords; u += blockDim.x) {
+      const int v = u % pairs, k = u / pairs;
+      const bool ofB = v >= va;
+      const int c = ofB ? pa + 2 * (v - va) : 2 * v, end = ofB ? total : pa;  // the pair's columns c, c + 1
+      const uint32_t t0 = (key[c] >> 20) - min(key[c] >> 20, (uint32_t)kSpreadBits);
+      const uint32_t k1 = c + 1 < end ? key[c + 1] >> 20 : 0u;
+      const uint32_t t1 = k1 - min(k1, (uint32_t)kSpreadBits);
+      uint32_t m0 = 0u, m1 = 0u;
+#pragma unroll 8
+      for (int r = 0; r < 32; ++r) {
+        const uint32_t e = ex2[(32 * k + r) * pairs + v];
+        m0 |= ((e & 0xffffu) >= t0 ? 1u : 0u) << r;
+        m1 |= ((e >> 16) >= t1 ? 1u : 0u) << r;
+      }
+      mask[c][k] = m0;
+      if (c + 1 < end) mask[c + 1][k] = m1;
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, pb = same ? pa : B.width(), b0 = same ? 0 : pa;
+    bool apart = false;
+    for (int i = lane; i < pa; i += 32) {
+      uint32_t m[kMaskWords];
+#pragma unroll
+      for (int k = 0; k < kMaskWords; ++k) m[k] = mask[i][k];
+      for (int j = threadIdx.x >> 5; j < pb; j += blockDim.x / 32) {
+        int shared_rows = 0;
+#pragma unroll
+        for (int k = 0; k < kMaskWords; ++k) shared_rows += __popc(m[k] & mask[b0 + j][k]);
+        apart |= shared_rows < kSpreadRows && key[i] != 0u && key[b0 + j] != 0u;
+      }
+    }
+    if (apart) atomicOr(flag, kSpread);
   }
 }
 
@@ -139,7 +195,7 @@ __global__ void __launch_bounds__(256) exp_dense_kernel(int64_t n, const double*
   k = __reduce_max_sync(0xffffffffu, k);
   if (lane) return;
   const int e = group_exp(k);
-  if (e < 0) *flag = 1;
+  if (e < 0) atomicOr(flag, kOutOfRange);
   exps[blockIdx.y * stride + col] = e;
 }
 
@@ -168,7 +224,7 @@ __global__ void __launch_bounds__(256) exp_dense_rows_kernel(int64_t n, const do
   const int64_t col = (int64_t)blockIdx.x * 64 + threadIdx.x;
   if (threadIdx.x < 64 && col < n) {
     const int e = group_exp(key[threadIdx.x]);
-    if (e < 0) *flag = 1;
+    if (e < 0) atomicOr(flag, kOutOfRange);
     exps[blockIdx.y * stride + col] = e;
   }
 }
@@ -189,7 +245,7 @@ __global__ void __launch_bounds__(256) exp_rows_kernel(int64_t n, int p, const d
   __syncthreads();
   if (threadIdx.x < p) {
     const int e = group_exp(key[threadIdx.x]);
-    if (e < 0) *flag = 1;
+    if (e < 0) atomicOr(flag, kOutOfRange);
     exps[blockIdx.x * stride + threadIdx.x] = e;
   }
 }
@@ -580,11 +636,11 @@ size_t gram64_scratch_ints(int64_t n) { return (size_t)ceil_div(n, kGroupRows) *
 
 // Gram partials through digit products; returns 0 without launching where the operands do not share
 // one 16-byte aligned row stride or need more shared memory than a CTA has.  scratch:
-// gram64_scratch_ints(n) ints; its first word is the flag: when the launched kernels leave it at 1
-// the partials are not written, and the caller's general kernel (launched on the same flag) forms
-// them over the same number of CTAs.
+// gram64_scratch_ints(n) ints; its first word is the flag: where it is not zero the partials are not
+// written, and the caller's general kernel (launched on the same flag) forms them over the same
+// number of CTAs.  spread: the flag is also raised where two columns of a group are too far apart.
 int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
-                         int max_ctas, int* scratch, int* err, cudaStream_t st) {
+                         int max_ctas, int* scratch, bool spread, int* err, cudaStream_t st) {
   if (a.nseg == 0 || b.nseg == 0 || n <= 0) return 0;
   const int ld = a.ld[0];
   if (ld & 1) return 0;
@@ -614,7 +670,20 @@ int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b
   int* exps = scratch + 4;
   const int estride = pa + (same ? 0 : pb), eb0 = same ? 0 : pa;
   LB_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
-  exp_kernel<<<(unsigned)ngroups, 256, 0, st>>>(n, a, b, ld, same ? 1 : 0, exps, estride, flag);
+  if (spread) {
+    if (a.nseg != 1 || b.nseg != 1 || n < kGroupRows) return 0;
+    static const bool attr = [&] {
+      LB_CUDA(cudaFuncSetAttribute(exp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   kGroupRows * kMaxS * (int)sizeof(uint32_t)));
+      return true;
+    }();
+    (void)attr;
+    const size_t bytes = (size_t)kGroupRows * ((pa + 1) / 2 + (same ? 0 : (pb + 1) / 2)) * sizeof(uint32_t);
+    exp_kernel<true><<<(unsigned)(ngroups + (n % kGroupRows ? 1 : 0)), 256, bytes, st>>>(n, a, b, ld, same ? 1 : 0, exps,
+                                                                                         estride, flag);
+  } else {
+    exp_kernel<false><<<(unsigned)ngroups, 256, 0, st>>>(n, a, b, ld, same ? 1 : 0, exps, estride, flag);
+  }
   LB_LAUNCH_CHECK();
   for (int ia = 0; ia < na; ++ia)
     for (int ib = 0; ib < nb; ++ib) {

@@ -420,6 +420,10 @@ struct lobpcg_ctx {
   DevBuf mlp_params, rho;
   float cscale = 0.f;
   bool use_learned = false;  // cleared for the rest of a solve when the residuals stall
+  // The digit products only where every entry of the result is as exact as the older kernels' (the
+  // building-block entry points, whose callers scale as they like); inside a solve, whose blocks have
+  // normalised columns, errors against the columns' norms are what counts.
+  bool entrywise = false;
   bool df_on = false;        // FP64 Grams and updates in double-float arithmetic (this phase)
   // generalised problem A x = lambda B x (Sec. 3.3): B (borrowed), B X, B P (double-
   // buffered like X and P), B W, and Q = orth(B X, B P) for the projection of W~
@@ -653,7 +657,14 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
     const double mults = (double)c.A.n * pa * pb * (upper ? 0.5 : 1.0);
     if (c.digits_on() && mults >= (c.df_on ? kDigitGramDf : kDigitGram)) {
       int* flag = c.gram_scratch();
-      parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.err_word(kErrGram), c.st);
+      parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.entrywise, c.err_word(kErrGram),
+                                   c.st);
+      if (parts && c.entrywise && c.df_on) {  // columns far apart, all in range: double-float, not the FMAs
+        int* h = reinterpret_cast<int*>(c.host);
+        LB_CUDA(cudaMemcpyAsync(h, flag, sizeof(int), cudaMemcpyDeviceToHost, c.st));
+        c.sync();
+        if (*h == 2) parts = 0;
+      }
       if (parts) gram_partials<T>(c.A.n, a, b, upper, c.Gpart, parts, c.st, flag);
     }
     if (!parts && c.df_on) parts = gram_partials_df(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
@@ -1786,6 +1797,7 @@ extern "C" lobpcg_status lobpcg_gram_f64(int64_t n, int p, const double* X, int 
     require(p >= 1 && q >= 1 && p <= kMaxS && q <= kMaxS && ldx >= p && ldy >= q,
             "lobpcg_gram_f64: need 1 <= p, q <= 96, ld >= width");
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
+    s.c.entrywise = true;
     gram<double>(s.c, cols1<double>(X, ldx, p), cols1<double>(Y, ldy, q), false, C);
     s.c.finish();
     return LOBPCG_OK;
@@ -1803,6 +1815,7 @@ extern "C" lobpcg_status lobpcg_gram_f64_df(int64_t n, int p, const double* X, i
             "lobpcg_gram_f64_df: X and Y must be 16-byte aligned with one even row stride");
     ScratchCtx s(n, reinterpret_cast<cudaStream_t>(stream));
     s.c.df_on = true;
+    s.c.entrywise = true;
     gram<double>(s.c, cols1<double>(X, ldx, p), cols1<double>(Y, ldy, q), false, C);
     s.c.finish();
     return LOBPCG_OK;
