@@ -520,18 +520,39 @@ struct Prec<float> {
   static int64_t lda(lobpcg_ctx& c) { return c.A.n; }
 };
 
-// Multiply-adds from which the digit products win over FP64 FMAs and over double-float: their fixed
-// cost (exponents, TMEM, the second kernel) against the older kernels' rates.  Microseconds per call just
-// below and above each line (older kernel, digits), entry-point overhead of about 40 included:
-//   Gram, FP64 FMAs:     16 columns 84, 91    32 columns 96, 76    63 columns 115, 90
-//   Gram, double-float:  16 columns 143, 123  32 columns 111, 88   63 columns 132, 89
-//   update, double-float: 63 columns to 21 98, 67   21 to 7 126, 115   96 to 32 101, 78
-//   dense product, FP64 FMAs, at 3e7 multiply-adds: p = 4 217, 110   p = 13 187, 93   p = 32 159, 85;
-//     half of that is where they meet
-// The update's line against FP64 FMAs is the Gram's: the same pipe, the same fixed cost.
-constexpr double kDigitGram = 2e7, kDigitGramDf = 6e7;
+// Where the digit products win over FP64 FMAs and over double-float.  Their fixed cost (exponents, TMEM,
+// the second kernel) asks for a number of multiply-adds in all, and their cost per row, which hardly
+// depends on the width of a thin block (the MMAs are padded to 32 columns), for a number per row.
+// Microseconds per call on both sides of each line (older kernel, digits):
+//   Gram, FP64 FMAs:     16 x 16, 2.6e7 101, 100    63 x 63, 2.1e7 95, 94 (105 with the test of spread),
+//                        4e7 147, 104    96 x 96 (four launches), 2.1e7 158, 179, 4e7 210, 178
+//                        per row: 4 x 21 439, 476   8 x 8 256, 398   12 x 12 496, 433   16 x 16 762, 447
+//   Gram, double-float:  32 x 32, 6e7 113, 115, 1e8 153, 122   63 x 63, 6e7 138, 116
+//                        per row: 8 x 8 364, 419    4 x 21 595, 495   12 x 12 502, 451
+//   update, double-float: 63 columns to 7, 1.8e7 133, 104   12 to 4, 1.5e8 (pair) 408, 547
+//                        per row, one product: 12 to 4 192, 290   24 to 4 307, 309   18 to 6 341, 324
+//   update, FP64 FMAs:   6 to 2, 2.4e6 (pair) 156, 116; wider ones more
+//   dense product, FP64 FMAs: p = 4, 1.6e7 122, 98   n = 8192: p = 2 341, 420   p = 3 631, 420   p = 13 2220, 436;
+//                        row-major, against a transposed copy and FMAs: p = 1 666, 405
+// ("per row": 1.6 million rows.)
+constexpr double kDigitGram = 2e7, kDigitGramWide = 4e7, kDigitGramDf = 6e7;
+constexpr double kDigitGramRow = 128, kDigitGramDfRow = 80;
+constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7, kDigitUpdateDfRow = 96;
 constexpr double kDigitDense = 1.5e7;
-constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7;
+constexpr int kDigitDenseP = 3;
+
+bool gram_digits_pay(int64_t n, int pa, int pb, bool upper, bool df) {
+  const double row = pa * pb * (upper ? 0.5 : 1.0);
+  return row >= (df ? kDigitGramDfRow : kDigitGramRow) &&
+         n * row >= (df ? kDigitGramDf : std::max(pa, pb) > 64 ? kDigitGramWide : kDigitGram);
+}
+bool update_digits_pay(int64_t n, int s, int q, int nprod, bool df) {
+  const double row = (double)s * q;
+  return df ? row >= kDigitUpdateDfRow && n * row * nprod >= kDigitUpdateDf : n * row * nprod >= kDigitUpdate;
+}
+bool dense_digits_pay(int64_t n, int p, bool row_major) {
+  return (row_major || p >= kDigitDenseP) && (double)n * n * p >= kDigitDense;
+}
 
 // launch_update with, in profile mode, the FP64 launches timed and their flops counted.
 template <class T>
@@ -543,7 +564,7 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   if constexpr (std::is_same<T, double>::value) {
     // digit products on the tensor cores from the size where they are the faster form
     parts = 0;
-    if (c.digits_on() && (double)c.A.n * s * q * job.nprod >= (c.df_on ? kDigitUpdateDf : kDigitUpdate))
+    if (c.digits_on() && update_digits_pay(c.A.n, s, q, job.nprod, c.df_on))
       parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.err_word(kErrUpdate),
                                    c.st);
     if (!parts)
@@ -559,9 +580,6 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   return parts;
 }
 
-// Whether the dense FP64 product is the faster form through digit products.
-bool dense_digits_pay(int64_t n, int p) { return (double)n * n * p >= kDigitDense; }
-
 // Y = A X with the product kernel chosen for this precision (no statistics).
 template <class T>
 void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
@@ -573,7 +591,7 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
                           false, var);
   else {
     if constexpr (std::is_same<T, double>::value) {
-      if (c.digits_on() && dense_digits_pay(c.A.n, p)) {
+      if (c.digits_on() && dense_digits_pay(c.A.n, p, false)) {
         c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
         if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false,
                                      c.err_word(kErrGram), c.st)) {
@@ -654,8 +672,7 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
     // digit products on the tensor cores from the size where they are the faster form; a column
     // outside the digits' range raises their flag, and the FMA kernel behind them (else an empty
     // launch) forms the partials
-    const double mults = (double)c.A.n * pa * pb * (upper ? 0.5 : 1.0);
-    if (c.digits_on() && mults >= (c.df_on ? kDigitGramDf : kDigitGram)) {
+    if (c.digits_on() && gram_digits_pay(c.A.n, pa, pb, upper, c.df_on)) {
       int* flag = c.gram_scratch();
       parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.entrywise, c.err_word(kErrGram),
                                    c.st);
@@ -1749,7 +1766,7 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
     require(p >= 1 && p <= 32 && ldx >= p && ldy >= p, "lobpcg_spmm_dense_f64: need 1 <= p <= 32, ld >= p");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     PoolBuf work(st);
-    if (dense_digits_pay(n, p)) {
+    if (dense_digits_pay(n, p, false)) {
       work.alloc(dense64_scratch_bytes(n, p));
       int* word = work.as<int>();  // the digits' flag, then the error word
       LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
@@ -1775,7 +1792,7 @@ extern "C" lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, 
     require(p >= 1 && p <= 32 && ldx >= p && ldy >= p, "lobpcg_spmm_dense_rows_f64: need 1 <= p <= 32, ld >= p");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     *done = 0;
-    if (!dense_digits_pay(n, p)) return LOBPCG_OK;
+    if (!dense_digits_pay(n, p, true)) return LOBPCG_OK;
     PoolBuf work(st);
     work.alloc(dense64_scratch_bytes(n, p));
     int* word = work.as<int>();  // the digits' flag, then the error word
