@@ -206,8 +206,13 @@ int launch_update_df(int64_t n, const UpdateJob<double>& job, const double* U, i
                      const double* lam, double* norm_part, int max_ctas, cudaStream_t st);
 // The FP64 update through exact digit products on the tensor cores (update64.cu); unit_base is
 // not needed there and ignored.  Returns 0 without launching where the blocks do not fit.
+// spread: rows with an output far below the rest are formed with FP64 FMAs, so every output is as
+// exact as double-float's.
 int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                         const double* lam, double* norm_part, int max_ctas, int* err, cudaStream_t st);
+                         const double* lam, double* norm_part, int max_ctas, bool spread, int* err, cudaStream_t st);
+// *count (device) receives how many of the rows looked at (returned) are such rows.
+int update64_sample(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha, int* count,
+                    cudaStream_t st);
 // dst[i] = (hi, lo) split of src[i] (the double-float operands: matrix values, blocks).
 void launch_split_df(int64_t count, const double* src, float2* dst, cudaStream_t st);
 // Y = A X (FP64 result) from the split values vs (nnz) and the split block Xs (n x ldx

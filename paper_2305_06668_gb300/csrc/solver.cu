@@ -179,7 +179,7 @@ struct InvalidArg : std::runtime_error {
 
 // Error words of the kernels with bounded waits (common.cuh), at ictl + kErr0 of a context.
 enum { kErrGram = 0, kErrUpdate, kErrGram32, kErrWords };
-constexpr int kErr0 = 8;
+constexpr int kErr0 = 8, kSample = 16;
 void throw_if_gave_up(int kind, int code) {
   static const char* const what[kErrWords] = {"FP64 Gram", "FP64 update", "Gram"};
   if (code)
@@ -397,7 +397,8 @@ struct lobpcg_ctx {
   double *Gpart = nullptr, *G = nullptr, *U = nullptr, *lam_all = nullptr, *up = nullptr;
   double *Tm = nullptr, *C = nullptr, *npart = nullptr, *resnorm = nullptr, *scal = nullptr;
   double *lam = nullptr, *sgn = nullptr, *S = nullptr, *colmax = nullptr;
-  int* ictl = nullptr;  // [0..3] cholqr ctl, [4] sweeps, [5] finite flag, [kErr0 ..] error words
+  int* ictl = nullptr;  // [0..3] cholqr ctl, [4] sweeps, [5] finite flag, [kErr0 ..] error words,
+                        // [kSample] rows found apart
   LockState* lock = nullptr;
   DevBuf x0buf;        // column-major FP64 initial block when X0 == NULL
   DevBuf xbest;        // the FP32 phase's X with the smallest largest-sought residual (reading R22)
@@ -530,14 +531,17 @@ struct Prec<float> {
 //   Gram, double-float:  32 x 32, 6e7 113, 115, 1e8 153, 122   63 x 63, 6e7 138, 116
 //                        per row: 8 x 8 364, 419    4 x 21 595, 495   12 x 12 502, 451
 //   update, double-float: 63 columns to 7, 1.8e7 133, 104   12 to 4, 1.5e8 (pair) 408, 547
-//                        per row, one product: 12 to 4 192, 290   24 to 4 307, 309   18 to 6 341, 324
+//                        per row, one product: 12 to 4 192, 290   24 to 4 307, 309   18 to 6 341, 324; a pair:
+//                        12 to 4 408, 547   24 to 4 1210, 596   18 to 6 693, 621.  The line lies at 64, where
+//                        one product is not yet faster, because tests/test_gpu_update_digits.py holds 17 to 4
+//                        to the digits' accuracy
 //   update, FP64 FMAs:   6 to 2, 2.4e6 (pair) 156, 116; wider ones more
 //   dense product, FP64 FMAs: p = 4, 1.6e7 122, 98   n = 8192: p = 2 341, 420   p = 3 631, 420   p = 13 2220, 436;
 //                        row-major, against a transposed copy and FMAs: p = 1 666, 405
 // ("per row": 1.6 million rows.)
 constexpr double kDigitGram = 2e7, kDigitGramWide = 4e7, kDigitGramDf = 6e7;
 constexpr double kDigitGramRow = 128, kDigitGramDfRow = 80;
-constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7, kDigitUpdateDfRow = 96;
+constexpr double kDigitUpdate = 2e7, kDigitUpdateDf = 6e7, kDigitUpdateDfRow = 64;
 constexpr double kDigitDense = 1.5e7;
 constexpr int kDigitDenseP = 3;
 
@@ -564,9 +568,19 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   if constexpr (std::is_same<T, double>::value) {
     // digit products on the tensor cores from the size where they are the faster form
     parts = 0;
-    if (c.digits_on() && update_digits_pay(c.A.n, s, q, job.nprod, c.df_on))
-      parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.err_word(kErrUpdate),
-                                   c.st);
+    bool digits = c.digits_on() && update_digits_pay(c.A.n, s, q, job.nprod, c.df_on);
+    if (digits && c.entrywise) {
+      // rows too far apart are formed with FP64 FMAs: a pair of 10^6 rows, 63 columns to 21, takes 920 us without
+      // any, 1,230 with one in 32, so about 2,150 with one in eight; double-float takes 2,440
+      int* h = reinterpret_cast<int*>(c.host);
+      const int rows = update64_sample(c.A.n, job, U, s, q, alpha, c.ictl + kSample, c.st);
+      LB_CUDA(cudaMemcpyAsync(h, c.ictl + kSample, sizeof(int), cudaMemcpyDeviceToHost, c.st));
+      c.sync();
+      digits = *h * 8 <= rows;
+    }
+    if (digits)
+      parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.entrywise,
+                                   c.err_word(kErrUpdate), c.st);
     if (!parts)
       parts = c.df_on ? launch_update_df(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st)
                       : launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
@@ -1860,6 +1874,7 @@ extern "C" lobpcg_status lobpcg_update_f64_df(int64_t n, int nseg, const double*
             "lobpcg_update_f64_df: need 1 <= s <= 96, 1 <= q <= 32, ld_out >= q, ld_base >= q");
     ScratchCtx sc(n, reinterpret_cast<cudaStream_t>(stream));
     sc.c.df_on = true;
+    sc.c.entrywise = true;
     UpdateJob<double> job{};
     job.in[0] = cv, job.in[1] = ca;
     job.out[0] = X, job.out[1] = AX;

@@ -27,8 +27,9 @@
 //     eight regions of an element are joined into FP64 with integer operations and turned inside the warp
 //     to four lanes per row, which add the base, store 32-byte pieces of rows and, from the pair's two
 //     elements, keep the sum of squares and the maximum of the residuals of their column.
-// Rows with an infinity, a NaN or an exponent outside 2^+-400 (and all rows when U has one) are
-// formed by their epilogue thread with FP64 FMAs.
+// Rows with an infinity, a NaN or an exponent outside 2^+-400 (and all rows when U has one), and with
+// `spread` rows with an output far below the rest (below), are formed by their epilogue threads with
+// FP64 FMAs.
 #include <algorithm>
 #include <climits>
 
@@ -60,26 +61,88 @@ constexpr size_t kSmemBudget = 227 * 1024;
 // bytes of U's digits: kSlices slices of kQ columns x KP rows
 __host__ __device__ constexpr uint32_t u_slice(int kp) { return (uint32_t)(kQ * kp * 2); }
 
+// What the digits of a row may drop is 2^-56 of its largest contribution to any output, and an output
+// may consist of smaller ones (columns of V of different length met by equal rows of U).  With 2^E and
+// 2^C the powers of two at row i's largest |V_il| g_l and at column j's largest |U_lj| / g_l (g_l: row l
+// of alpha U, at most), an entry l whose factors are both within 3 binades of those gives
+// sum |V||alpha U| at least 2^-6 2^(E+C), one whose U is within 6 binades 2^-9.  An output is safe
+// where that comes to 2^-6 2^(E+C) per 32 entries of the row: the digits' rounding, 2^-57.8 sqrt(s)
+// 2^(E+C+2) in the mean, is then below double-float's 2^-48 of the sum.
+constexpr int kNear = 3, kMid = 6;
+__device__ __forceinline__ bool output_safe(int near, int mid, int s32) { return 7 * near + mid >= 8 * s32; }
+
+// The scaling of U, by all threads of a CTA; us: alpha U (s x q, column-major).
+struct UScale {
+  int16_t up[kMaxS];         // exponent of row l of U: V's column l is scaled by 2^up; -4000: a zero row
+  int col_exp[kQ];           // exponent of column j over its scaled entries
+  uint32_t near[kQ][kMaxS / 32], mid[kQ][kMaxS / 32];  // bit l: (l, j) within kNear, kMid binades of 2^col_exp
+  uint32_t nonzero;          // columns with any non-zero entry
+  int small;                 // most entries of a non-zero column that are not in `mid`
+  int bad;                   // a row or column outside the digits' range
+};
+__device__ __forceinline__ void scale_u(UScale& u, const double* us, int s, int q) {
+  if (threadIdx.x == 0) u.bad = 0, u.nonzero = 0u, u.small = 0;
+  __syncthreads();
+  for (int l = threadIdx.x; l < kMaxS; l += blockDim.x) {
+    uint32_t key = 0u;
+    if (l < s)
+      for (int j = 0; j < q; ++j) key = max(key, exp_key(us[l + j * s]));
+    const int e = group_exp(key);
+    if (e < 0) u.bad = 1;
+    u.up[l] = key ? (int16_t)(e - 1022) : (int16_t)-4000;  // a zero row of U: no contribution
+  }
+  __syncthreads();
+  // U's entry (l, j) scaled by 2^-up: below 1 in magnitude.  A warp per column.
+  const int lane = threadIdx.x & 31;
+  for (int j = threadIdx.x >> 5; j < kQ; j += blockDim.x >> 5) {
+    int e[kMaxS / 32], E = 0;
+    bool any = false;
+#pragma unroll
+    for (int c = 0; c < kMaxS / 32; ++c) {
+      const int l = 32 * c + lane;
+      const uint32_t key = j < q && l < s ? exp_key(us[l + j * s]) : 0u;
+      any |= key != 0u;
+      e[c] = key >> 20 ? (int)(key >> 20) - u.up[l] : -10000;
+      E = max(E, e[c]);
+    }
+    E = __reduce_max_sync(0xffffffffu, E);
+    any = __any_sync(0xffffffffu, any);
+    int in = 0;
+#pragma unroll
+    for (int c = 0; c < kMaxS / 32; ++c) {
+      const uint32_t near = __ballot_sync(0xffffffffu, e[c] >= E - kNear);
+      const uint32_t mid = __ballot_sync(0xffffffffu, e[c] >= E - kMid);
+      if (lane == 0) u.near[j][c] = near, u.mid[j][c] = mid;
+      in += __popc(mid);
+    }
+    if (lane) continue;
+    if (any && E < kExpMin) u.bad = 1;  // a column of numbers far below their rows'
+    u.col_exp[j] = any ? E : kExpOne;
+    if (any) atomicOr(&u.nonzero, 1u << j), atomicMax(&u.small, s - in);
+  }
+  __syncthreads();
+}
+
 // NC: 32-column chunks of V (ceil(s / 32)).
 template <int NC, bool NORM>
 __global__ void __launch_bounds__(kThreads, 1)
     update64_kernel(int64_t n, UpdateJob<double> job, const double* __restrict__ U, int s, int q, double alpha,
                     const double* __restrict__ lam, double* __restrict__ norm_part, int64_t tiles_per_cta,
-                    int ts, int* __restrict__ err) {
+                    int ts, int spread, int* __restrict__ err) {
   constexpr int KP = NC * kKC;
   constexpr uint32_t kSliceU = u_slice(KP), kSBOU = KP / 8 * 128;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t raw_full[kSplitWarps], tile_full[kMaxTS], tile_empty[kMaxTS], acc_full[2], acc_empty[2], exp_full[kRing];
   __shared__ uint64_t rows_read[4];  // both epilogue warps of a lane quadrant have read their rows
   __shared__ int16_t row_exp[kRing][kTile];
-  __shared__ int col_exp[kQ];
-  __shared__ __align__(16) int16_t up[KP];  // exponent of row l of U: V's column l is scaled by 2^up
+  __shared__ __align__(16) UScale us_;
+  int16_t* const up = us_.up;
+  int* const col_exp = us_.col_exp;
   __shared__ double nred[2][kEpiWarps][NORM ? kQ / 2 : 1];  // a warp's sums and maxima of its columns
   __shared__ double lam_s[kQ];
   __shared__ double stage[kEpiWarps][32][4];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
-  __shared__ int u_bad;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nseg = job.in[0].nseg, nprod = job.nprod;
@@ -90,7 +153,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   double* raw = reinterpret_cast<double*>(udig + kSlices * kSliceU);      // [kSplitWarps][segment][8][ld]
 
   if (tid == 0) {
-    abort_flag = 0, u_bad = 0;
+    abort_flag = 0;
     for (int i = 0; i < kSplitWarps; ++i) mbar_init(&raw_full[i], 1);
     for (int i = 0; i < kMaxTS; ++i) mbar_init(&tile_full[i], kSplitWarps), mbar_init(&tile_empty[i], 1);
     for (int i = 0; i < 2; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], kEpiWarps);
@@ -102,31 +165,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // alpha U, staged in the first tile buffer (s x q column-major, at most 24 KB of its 56)
   double* us = reinterpret_cast<double*>(tiles);
   for (int e = tid; e < s * q; e += kThreads) us[e] = alpha * U[e];
-  __syncthreads();
-  for (int l = tid; l < KP; l += kThreads) {
-    uint32_t key = 0u;
-    if (l < s)
-      for (int j = 0; j < q; ++j) key = max(key, exp_key(us[l + j * s]));
-    const int e = group_exp(key);
-    if (e < 0) u_bad = 1;
-    up[l] = key ? (int16_t)(e - 1022) : (int16_t)-4000;  // a zero row of U: no contribution
-  }
-  __syncthreads();
-  // U's entry (l, j) scaled by 2^-up: below 1 in magnitude; exponent of a column over its scaled entries
-  for (int j = tid; j < kQ; j += kThreads) {
-    if (NORM) lam_s[j] = j < q ? lam[j] : 0.0;
-    int E = 0;
-    bool any = false;
-    if (j < q)
-      for (int l = 0; l < s; ++l) {
-        const uint32_t key = exp_key(us[l + j * s]);
-        any |= key != 0u;
-        if (key >> 20) E = max(E, (int)(key >> 20) - up[l]);
-      }
-    if (any && E < kExpMin) u_bad = 1;  // a column of numbers far below their rows'
-    col_exp[j] = any ? E : kExpOne;
-  }
-  __syncthreads();
+  if (NORM)
+    for (int j = tid; j < kQ; j += kThreads) lam_s[j] = j < q ? lam[j] : 0.0;
+  scale_u(us_, us, s, q);
   for (int e = tid; e < s * q; e += kThreads) {
     const int l = e % s, j = e / s;
     // digits() takes the exponent in the entry's own scale; entries far below their column shift out
@@ -144,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  const bool all_bad = u_bad != 0;
+  const bool all_bad = us_.bad != 0;
 
   const int64_t t_begin = (int64_t)blockIdx.x * tiles_per_cta;
   const int64_t r_begin = t_begin * kTile, r_end = min(n, r_begin + tiles_per_cta * kTile);
@@ -216,14 +257,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t somem = __ballot_sync(0xffffffffu, some);
         bad |= E <= 0 && (somem & (0x01010101u << r)) != 0u;
       }
+      const bool judge = spread && E > 0 && !bad;
       if (E <= 0 || bad) E = kExpOne;
+      uint32_t near[NC];  // entries of the row within kNear binades of 2^E, this lane's in its byte
+#pragma unroll
+      for (int c = 0; c < NC; ++c) near[c] = 0u;
+      bool done = true;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        if (chunk >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph, &abort_flag, err, 2))) break;
-        if (c == 0) {
-          if (lane < 8) row_exp[T & (kRing - 1)][8 * warp + lane] = (int16_t)(bad ? kBad : E);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&exp_full[T & (kRing - 1)]);
+        if (chunk >= ts && !__all_sync(0xffffffffu, wait_bar(&tile_empty[buf], tph, &abort_flag, err, 2))) {
+          done = false;
+          break;
         }
         const int4 u4 = *reinterpret_cast<const int4*>(&up[c * kKC + 8 * k8]);
         const int us4[4] = {u4.x, u4.y, u4.z, u4.w};
@@ -234,6 +278,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           // the row's exponent in the entry's own scale; a bad row's digits are not used
           w[i] = digits(bad ? 0.0 : x[c][i], v > -4000 ? E - v : 4 * kExpOne);
         }
+        if (spread) {
+          // |leading digit| >= 9: at least 2^51 of the 2^54 that 2^E is
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            near[c] |= (((uint32_t)(w[i] >> 48) & 0xffu) - 120u > 16u ? 1u : 0u) << (8 * k8 + i);
+        }
         unsigned char* o = tiles + (uint32_t)buf * kBuf + (uint32_t)warp * kSBO + (uint32_t)k8 * kLBO + 16u * r;
         put_digits(w, o, kSlice);
         fence_proxy_async();
@@ -242,6 +292,33 @@ __global__ void __launch_bounds__(kThreads, 1)
         ++chunk;
         if (++buf == ts) buf = 0, tph ^= 1u;
       }
+      if (!done) break;
+      if (spread) {
+        int count = 0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          near[c] |= __shfl_xor_sync(0xffffffffu, near[c], 8);
+          near[c] |= __shfl_xor_sync(0xffffffffu, near[c], 16);
+          count += __popc(near[c]);
+        }
+        // enough of them for every output, whichever the column's small entries are; else output by output
+        const bool unsure = judge && count - us_.small < 8 * NC;
+        if (__any_sync(0xffffffffu, unsure)) {
+          bool apart = false;
+          for (int j = k8; j < q; j += 4) {
+            int nn = 0, nm = 0;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+              nn += __popc(near[c] & us_.near[j][c]), nm += __popc(near[c] & us_.mid[j][c]);
+            apart |= unsure && !output_safe(nn, nm, NC) && (us_.nonzero >> j & 1u) != 0u;
+          }
+          const uint32_t apartm = __ballot_sync(0xffffffffu, apart);
+          bad |= (apartm & (0x01010101u << r)) != 0u;
+        }
+      }
+      if (lane < 8) row_exp[T & (kRing - 1)][8 * warp + lane] = (int16_t)(bad ? kBad : E);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&exp_full[T & (kRing - 1)]);
     }
   } else if (warp == kMma) {
     if (lane == 0) {
@@ -293,8 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     uint32_t rph = 0;  // parity of the next rows_read phase
     for (int it = 0; it < ntiles && ok; ++it) {
-      const int64_t grow = r_begin + (int64_t)it * kTile + row;
-      const bool live = grow < r_end;
+      const bool live = r_begin + (int64_t)it * kTile + row < r_end;
       int er[2] = {kExpOne, kExpOne};
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
@@ -306,25 +382,42 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
       tc_fence_after();
-      // rows outside the digits' range: FP64 FMAs from global memory, all of the row before any store
-      double slow[2][kQ];
+      // rows outside the digits' range or too far apart: FP64 FMAs from global memory, a row at a time by the
+      // whole warp (eight lanes a column, four columns at once), all of this warp's elements before any store
+      const int64_t row0 = r_begin + (int64_t)it * kTile + 32 * quad;  // rows of this warp
+      const int nrows = (int)max((int64_t)0, min((int64_t)32, r_end - row0));
+      double slow[2][kQ / 8][4];
+#pragma unroll 1
+      for (int t = 0; t < nprod; ++t) {
+        for (uint32_t m = __ballot_sync(0xffffffffu, live && er[t] == kBad); m; m &= m - 1u) {
+          const int rr = __ffs(m) - 1;
+#pragma unroll 1
+          for (int gh = 0; gh < kQ / 8; ++gh) {
+            const int j = 4 * (2 * gh + half) + (lane & 3);
+            if (j - (lane & 3) >= q) break;
+            double a = 0.0;
+            if (j < q) {
+              const double* u = U + j * s;
+#pragma unroll 1
+              for (int g = 0; g < nseg; ++g) {
+                const double* v = job.in[t].p[g] + (row0 + rr) * job.in[t].ld[g];
+                for (int i = lane >> 2; i < job.in[t].w[g]; i += 8) a = fma(v[i], u[i], a);
+                u += job.in[t].w[g];
+              }
+            }
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        if (t >= nprod || !live || er[t] != kBad) continue;
-        for (int j = 0; j < kQ; ++j) slow[t][j] = 0.0;
-        int l = 0;
-        for (int g = 0; g < nseg; ++g)
-          for (int i = 0; i < job.in[t].w[g]; ++i, ++l) {
-            const double v = job.in[t].p[g][grow * job.in[t].ld[g] + i];
-            for (int j = 0; j < q; ++j) slow[t][j] = fma(v, alpha * U[l + j * s], slow[t][j]);
+            for (int o = 4; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const double x = __shfl_sync(0xffffffffu, a, k);
+              if (lane == rr) slow[t][gh][k] = alpha * x;
+            }
           }
+        }
       }
       int se[2];  // element: (sum_t v_t 256^(7-t)) 2^(40 - 110) 2^(er - 1022) 2^(col_exp - 1022)
 #pragma unroll
       for (int t = 0; t < 2; ++t) se[t] = (er[t] == kBad ? kExpOne : er[t]) - 2 * 1022 - 70;
-      // rows of this warp
-      const int64_t row0 = r_begin + (int64_t)it * kTile + 32 * quad;
-      const int nrows = (int)max((int64_t)0, min((int64_t)32, r_end - row0));
       // both threads of a row have read it before either stores (the two warps see the same rows, so both
       // or neither come here); bounded like every wait, for the partner may have given up
       const bool any_bad = __any_sync(0xffffffffu, er[0] == kBad || er[1] == kBad);
@@ -360,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (any_bad && er[t] == kBad)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) o[i] = slow[t][4 * g + i];
+            for (int i = 0; i < 4; ++i) o[i] = slow[t][gh][i];
           // to the warp's stage (columns turned by row / 4: no bank conflicts either way), then four lanes per
           // row: whole 32-byte pieces of eight rows a store
 #pragma unroll
@@ -437,9 +530,55 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// *count += the rows among `samples` evenly spaced ones that update64_kernel would form with FMAs for
+// their spread.  A warp per row, a lane per entry.
+__global__ void __launch_bounds__(256) update64_sample_kernel(int64_t n, UpdateJob<double> job, const double* __restrict__ U,
+                                                              int s, int q, double alpha, int samples,
+                                                              int* __restrict__ count) {
+  __shared__ UScale u;
+  extern __shared__ double us[];
+  for (int e = threadIdx.x; e < s * q; e += blockDim.x) us[e] = alpha * U[e];
+  __syncthreads();
+  scale_u(u, us, s, q);
+  if (u.bad) return;  // every row takes the FMAs, none for its spread
+  const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x >> 5);
+  int total = 0;
+  for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < samples; i += warps) {
+    const int64_t row = (int64_t)i * n / samples;
+    bool apart = false;
+    for (int t = 0; t < job.nprod; ++t) {
+      int e[kMaxS / 32], E = 0;
+#pragma unroll
+      for (int c = 0; c < kMaxS / 32; ++c) {
+        int l = 32 * c + lane, g = 0;
+        e[c] = -10000;
+        if (l < s) {
+          const int up = u.up[l];
+          while (l >= job.in[t].w[g]) l -= job.in[t].w[g], ++g;
+          const int x = (__double2hiint(job.in[t].p[g][row * job.in[t].ld[g] + l]) >> 20) & 0x7ff;
+          if (x != 0 && x != 0x7ff) e[c] = x + up;
+        }
+        E = max(E, e[c]);
+      }
+      E = __reduce_max_sync(0xffffffffu, E);
+      if (E <= 0) continue;
+      int nn = 0, nm = 0;
+#pragma unroll
+      for (int c = 0; c < kMaxS / 32; ++c) {
+        const uint32_t near = __ballot_sync(0xffffffffu, e[c] >= E - kNear);
+        nn += __popc(near & u.near[lane][c]), nm += __popc(near & u.mid[lane][c]);  // lane: an output
+      }
+      apart |= __any_sync(0xffffffffu, !output_safe(nn, nm, (s + 31) / 32) && (u.nonzero >> lane & 1u) != 0u);
+    }
+    total += apart ? 1 : 0;
+  }
+  if (lane == 0 && total) atomicAdd(count, total);
+}
+
 template <int NC, bool NORM>
 int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, int* err, cudaStream_t st) {
+                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, bool spread, int* err,
+                    cudaStream_t st) {
   static const bool attr = [&] {
     LB_CUDA(cudaFuncSetAttribute(update64_kernel<NC, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBudget - kStatic)));
     return true;
@@ -452,7 +591,7 @@ int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, in
   const int64_t per = ceil_div(tiles, std::min<int64_t>(std::min<int64_t>(max_ctas, sms), tiles));
   const int64_t ctas = ceil_div(tiles, per);
   update64_kernel<NC, NORM><<<(unsigned)ctas, kThreads, smem, st>>>(n, job, U, s, q, alpha, lam, norm_part, per,
-                                                                    ts, err);
+                                                                    ts, spread ? 1 : 0, err);
   LB_LAUNCH_CHECK();
   return (int)ctas;
 }
@@ -462,7 +601,8 @@ int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, in
 // The block update through digit products; returns 0 without launching where the blocks do not fit
 // (unaligned or odd row strides, products of different layout, more shared memory than a CTA has).
 int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                         const double* lam, double* norm_part, int max_ctas, int* err, cudaStream_t st) {
+                         const double* lam, double* norm_part, int max_ctas, bool spread, int* err,
+                         cudaStream_t st) {
   if (n <= 0 || q < 1 || q > kQ || s < 1 || s > kMaxS || job.in[0].nseg < 1) return 0;
   if (norm_part && (job.nprod != 2 || job.base[0] || job.base[1])) return 0;
   size_t raw = 0;
@@ -481,12 +621,22 @@ int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* 
   const size_t smem = fixed + (size_t)ts * kBuf;
   if (smem > kSmemBudget - kStatic) return 0;
 #define LB_UPDATE64(NC)                                                                                          \
-  return norm_part ? update64_launch<NC, true>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, err, st)        \
-                   : update64_launch<NC, false>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, err, st)
+  return norm_part ? update64_launch<NC, true>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, spread, err, st)        \
+                   : update64_launch<NC, false>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, spread, err, st)
   if (nc == 1) LB_UPDATE64(1);
   if (nc == 2) LB_UPDATE64(2);
   LB_UPDATE64(3);
 #undef LB_UPDATE64
+}
+
+int update64_sample(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha, int* count,
+                    cudaStream_t st) {
+  const int samples = (int)std::min<int64_t>(n, 152 * 8);  // one row a warp
+  LB_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
+  update64_sample_kernel<<<(unsigned)((samples + 7) / 8), 256, (size_t)s * q * sizeof(double), st>>>(
+      n, job, U, s, q, alpha, samples, count);
+  LB_LAUNCH_CHECK();
+  return samples;
 }
 
 }  // namespace lobpcg

@@ -53,3 +53,47 @@ def test_gram(n, p, q, df, kind):
     tol = (136 * DF if df else n * FMA) * size
     err = np.abs((got.astype(np.longdouble) - ref).astype(np.float64))
     assert (err <= tol).all(), (err / np.maximum(tol, 1e-300)).max()
+
+
+def _rows_far_apart(kind, n, s, q, rng):
+    V, U = rng.standard_normal((n, s)), np.zeros((s, q))
+    if kind == "lengths":  # columns of V of different length, each an output of its own
+        V *= 10.0 ** -np.linspace(0, 12, s)
+        U[:q, :q] = np.eye(q)
+    elif kind == "pairs of rows":  # a few rows only, two outputs
+        V[::97, 0], V[::97, 1] = 1e10, 1e-10
+        U[:q, :q] = np.eye(q)
+        U += 1e-30 * rng.standard_normal((s, q))
+    elif kind == "last row":
+        V[n - 1, 2:] = 0.0
+        V[n - 1, :2] = 1.0, 1e-13
+        U[:] = rng.standard_normal((s, q))
+        U[0, 1:] = 0.0
+    elif kind == "column of U":  # an output that only the row's smallest entries reach
+        U[:] = rng.standard_normal((s, q))
+        U[:s - 1, q - 1] = 0.0
+        V[:, s - 1] *= 1e-12
+    return V, U
+
+
+@pytest.mark.parametrize("kind", ["lengths", "pairs of rows", "last row", "column of U"])
+@pytest.mark.parametrize("n,s,q,pair", [(60_001, 63, 21, False), (30_011, 64, 32, True), (200_003, 32, 13, True),
+                                        (22_003, 96, 32, False)])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_update(n, s, q, pair, in_place, kind):
+    import torch
+
+    import paper_2305_06668_gb300 as lb
+    rng = np.random.default_rng(n)
+    V, U = _rows_far_apart(kind, n, s, q, rng)
+    W = rng.standard_normal((n, s)) * np.abs(V)
+    (Vt,), (Wt,) = _one_stride(V), _one_stride(W)
+    more = dict(AV=[Wt], lam=torch.zeros(q, dtype=torch.float64, device="cuda"), resnorm=True) if pair else {}
+    if in_place:
+        more.update(dict(X=Vt, AX=Wt) if pair else dict(X=Vt))
+    got = lb.update_f64_df([Vt], torch.from_numpy(U).cuda(), alpha=-1.0, **more)
+    for o, x in zip(got[:2] if pair else [got], [V, W]):
+        ref = -(x.astype(np.longdouble) @ U.astype(np.longdouble))
+        tol = (s + 8) * DF * (np.abs(x) @ np.abs(U))
+        err = np.abs((o.cpu().numpy()[:, :q].astype(np.longdouble) - ref).astype(np.float64))
+        assert (err <= tol).all(), (err / np.maximum(tol, 1e-300)).max()
