@@ -132,12 +132,13 @@ template <class T>
 void launch_spmm_dense(int64_t n, const T* A, int64_t lda, int p, const T* X, int ldx, T* Y,
                        int ldy, cudaStream_t st, const int* run_flag = nullptr);
 // The FP64 product through exact digit products on the tensor cores (gram64.cu); false without
-// launching where the operands do not fit.  *scratch (dense64_scratch_bytes) is the flag left at 1
-// when a number is outside the digits' range: Y is then to be formed by launch_spmm_dense on it.
+// launching where the operands do not fit.  *scratch (dense64_scratch_bytes) is the flag, not zero
+// when a number is outside the digits' range or, with `spread`, two columns are too far apart (as in the
+// Gram, the diagonal of A aside): Y is then to be formed by launch_spmm_dense on it.
 // row_a: A is row-major (Y is still column i of A against X).
 size_t dense64_scratch_bytes(int64_t n, int p);
 bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
-                              int ldy, void* scratch, bool row_a, int* err, cudaStream_t st);
+                              int ldy, void* scratch, bool row_a, bool spread, int* err, cudaStream_t st);
 
 // Gram partials: part[g][i + j*pa] = sum over CTA g's rows of a_ri * b_rj.
 // upper: only i <= j entries are produced.  Returns the number of CTAs used.

@@ -175,78 +175,174 @@ __global__ void __launch_bounds__(256) exp_kernel(int64_t n, Cols<double> A, Col
   }
 }
 
+// The dense product asks the same of every column of A and of X, the diagonal of A left out: it has its
+// own place in the sums, for one large entry per column would take the others' digits.
+// Bit l of word 2 u + h of a mask is row 64 u + 2 l + h of the group, the order in which a warp reads a
+// column of A by 16-byte pairs.  xmask: per group 32 columns of X, kMaskWords each, then a word of the
+// columns that are not zero; the last group's are those of the last 256 rows where it is incomplete.
+constexpr int kXMask = 32 * kMaskWords + 1;
+__device__ __forceinline__ uint32_t near_limit(uint32_t key) {  // smallest exponent that counts as near
+  return (key >> 20) - min(key >> 20, (uint32_t)kSpreadBits);
+}
+__device__ __forceinline__ uint32_t exp_of(double x) { return ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu; }
+// Whether a column with mask m and any of the p <= 32 of X in the group share too few rows (j, j + step, ..).
+__device__ __forceinline__ bool far_from_x(const uint32_t (&m)[kMaskWords], const uint32_t* __restrict__ xm, int p, int j,
+                                           int step) {
+  const uint32_t nonzero = __ldg(xm + 32 * kMaskWords);
+  bool apart = false;
+  for (; j < p; j += step) {
+    int both = 0;
+#pragma unroll
+    for (int k = 0; k < kMaskWords; ++k) both += __popc(m[k] & __ldg(xm + j * kMaskWords + k));
+    apart |= both < kSpreadRows && (nonzero >> j & 1u) != 0u;
+  }
+  return apart;
+}
+// First row of block y of the groups, one more than there are for the last 256 rows.
+__device__ __forceinline__ int64_t group_row(int64_t n, bool& window) {
+  window = (int64_t)blockIdx.y * kGroupRows >= n;
+  return window ? n - kGroupRows : (int64_t)blockIdx.y * kGroupRows;
+}
+
 // Exponents of a dense column-major A (n x n, lda): one warp per column and group of kGroupRows rows.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) exp_dense_kernel(int64_t n, const double* __restrict__ A, int64_t lda,
-                                                        int* __restrict__ exps, int64_t stride,
-                                                        int* __restrict__ flag) {
+                                                        int* __restrict__ exps, int64_t stride, int p,
+                                                        const uint32_t* __restrict__ xmask, int* __restrict__ flag) {
   const int64_t col = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (col >= n) return;
-  const int64_t r0 = (int64_t)blockIdx.y * kGroupRows;
+  bool window;
+  const int64_t r0 = group_row(n, window);
   const int rows = (int)min((int64_t)kGroupRows, n - r0);
-  const double2* p = reinterpret_cast<const double2*>(A + col * lda + r0);
+  const double2* a = reinterpret_cast<const double2*>(A + col * lda + r0);
   double2 x[kGroupRows / 64];
 #pragma unroll
   for (int u = 0; u < kGroupRows / 64; ++u)
-    x[u] = 2 * (lane + 32 * u) < rows ? __ldg(p + lane + 32 * u) : make_double2(0.0, 0.0);  // rows is even
+    x[u] = 2 * (lane + 32 * u) < rows ? __ldg(a + lane + 32 * u) : make_double2(0.0, 0.0);  // rows is even
   uint32_t k = 0u;
 #pragma unroll
-  for (int u = 0; u < kGroupRows / 64; ++u) k = max(k, max(exp_key(x[u].x), exp_key(x[u].y)));
+  for (int u = 0; u < kGroupRows / 64; ++u) {
+    const int64_t r = r0 + 2 * (lane + 32 * u);
+    if (r == col) x[u].x = 0.0;
+    if (r + 1 == col) x[u].y = 0.0;
+    k = max(k, max(exp_key(x[u].x), exp_key(x[u].y)));
+  }
   k = __reduce_max_sync(0xffffffffu, k);
+  if constexpr (CHECK) {
+    if (rows == kGroupRows && k != 0u) {
+      const uint32_t limit = near_limit(k);
+      uint32_t m[kMaskWords];
+#pragma unroll
+      for (int u = 0; u < kGroupRows / 64; ++u) {
+        m[2 * u] = __ballot_sync(0xffffffffu, exp_of(x[u].x) >= limit);
+        m[2 * u + 1] = __ballot_sync(0xffffffffu, exp_of(x[u].y) >= limit);
+      }
+      const uint32_t* xm = xmask + (int64_t)blockIdx.y * kXMask;
+      if (__any_sync(0xffffffffu, far_from_x(m, xm, p, lane, 32)) && lane == 0) atomicOr(flag, kSpread);
+    }
+  }
   if (lane) return;
   const int e = group_exp(k);
   if (e < 0) atomicOr(flag, kOutOfRange);
-  exps[blockIdx.y * stride + col] = e;
+  if (!window) exps[blockIdx.y * stride + col] = e;
 }
 
 // The same of a row-major A: one CTA per group and 64 columns, a lane per 16-byte pair of columns.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) exp_dense_rows_kernel(int64_t n, const double* __restrict__ A, int64_t lda,
-                                                             int* __restrict__ exps, int64_t stride,
-                                                             int* __restrict__ flag) {
+                                                             int* __restrict__ exps, int64_t stride, int p,
+                                                             const uint32_t* __restrict__ xmask, int* __restrict__ flag) {
   __shared__ uint32_t key[64];
+  __shared__ uint32_t ex2[CHECK ? kGroupRows : 1][32];  // exponents of a pair of columns
   if (threadIdx.x < 64) key[threadIdx.x] = 0u;
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t c = (int64_t)blockIdx.x * 64 + 2 * lane, r0 = (int64_t)blockIdx.y * kGroupRows;
+  bool window;
+  const int64_t c = (int64_t)blockIdx.x * 64 + 2 * lane, r0 = group_row(n, window);
   const int rows = (int)min((int64_t)kGroupRows, n - r0);
   uint32_t k0 = 0u, k1 = 0u;
   if (c < n) {  // n is even
-    const double* p = A + r0 * lda + c;
+    const double* a = A + r0 * lda + c;
 #pragma unroll 8
     for (int r = w; r < rows; r += 8) {
-      const double2 x = __ldg(reinterpret_cast<const double2*>(p + r * lda));
+      double2 x = __ldg(reinterpret_cast<const double2*>(a + r * lda));
+      if (r0 + r == c) x.x = 0.0;
+      if (r0 + r == c + 1) x.y = 0.0;
       k0 = max(k0, exp_key(x.x)), k1 = max(k1, exp_key(x.y));
+      if (CHECK) ex2[r][lane] = exp_of(x.x) | exp_of(x.y) << 16;
     }
   }
   atomicMax(&key[2 * lane], k0);
   atomicMax(&key[2 * lane + 1], k1);
   __syncthreads();
-  const int64_t col = (int64_t)blockIdx.x * 64 + threadIdx.x;
+  const int64_t col = (int64_t)blockIdx.x * 64 + (threadIdx.x & 63);
+  if constexpr (CHECK) {
+    if (rows == kGroupRows) {
+      __shared__ uint32_t mask[64][kMaskWords];
+      const int cc = threadIdx.x & 63, q = threadIdx.x >> 6;
+      const uint32_t limit = near_limit(key[cc]);
+      for (int k = q; k < kMaskWords; k += 4) {
+        uint32_t m = 0u;
+#pragma unroll 8
+        for (int l = 0; l < 32; ++l)
+          m |= ((ex2[64 * (k >> 1) + 2 * l + (k & 1)][cc >> 1] >> (16 * (cc & 1)) & 0xffffu) >= limit ? 1u : 0u) << l;
+        mask[cc][k] = m;
+      }
+      __syncthreads();
+      if (col < n && key[cc] != 0u) {
+        uint32_t m[kMaskWords];
+#pragma unroll
+        for (int k = 0; k < kMaskWords; ++k) m[k] = mask[cc][k];
+        if (far_from_x(m, xmask + (int64_t)blockIdx.y * kXMask, p, q, 4)) atomicOr(flag, kSpread);
+      }
+    }
+  }
   if (threadIdx.x < 64 && col < n) {
     const int e = group_exp(key[threadIdx.x]);
     if (e < 0) atomicOr(flag, kOutOfRange);
-    exps[blockIdx.y * stride + col] = e;
+    if (!window) exps[blockIdx.y * stride + col] = e;
   }
 }
 
-// Exponents of a row-major block of p <= 32 columns (any row stride), one CTA per group.
+// Exponents of a row-major block of p <= 32 columns (any row stride), one CTA per group; CHECK: and xmask.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) exp_rows_kernel(int64_t n, int p, const double* __restrict__ X, int ldx,
                                                        int* __restrict__ exps, int64_t stride,
-                                                       int* __restrict__ flag) {
+                                                       uint32_t* __restrict__ xmask, int* __restrict__ flag) {
   __shared__ uint32_t key[32];
+  __shared__ uint16_t ex[CHECK ? kGroupRows : 1][32];
   if (threadIdx.x < 32) key[threadIdx.x] = 0u;
   __syncthreads();
-  const int64_t r0 = (int64_t)blockIdx.x * kGroupRows;
+  bool window;
+  const int64_t r0 = group_row(n, window);
   const int rows = (int)min((int64_t)kGroupRows, n - r0), j = threadIdx.x & 31;
   uint32_t k = 0u;
   if (j < p)
-    for (int r = threadIdx.x >> 5; r < rows; r += 8) k = max(k, exp_key(__ldg(X + (r0 + r) * ldx + j)));
+    for (int r = threadIdx.x >> 5; r < rows; r += 8) {
+      const double x = __ldg(X + (r0 + r) * ldx + j);
+      k = max(k, exp_key(x));
+      if (CHECK) ex[r][j] = (uint16_t)exp_of(x);
+    }
   atomicMax(&key[j], k);
   __syncthreads();
+  if constexpr (CHECK) {
+    if (rows == kGroupRows) {
+      uint32_t* xm = xmask + (int64_t)blockIdx.y * kXMask;
+      const int w = threadIdx.x >> 5;
+      const uint32_t limit = near_limit(key[j]);
+      uint32_t m = 0u;
+      if (j < p)
+        for (int l = 0; l < 32; ++l) m |= (ex[64 * (w >> 1) + 2 * l + (w & 1)][j] >= limit ? 1u : 0u) << l;
+      xm[j * kMaskWords + w] = m;
+      const uint32_t nonzero = __ballot_sync(0xffffffffu, key[j] != 0u);
+      if (threadIdx.x == 0) xm[32 * kMaskWords] = nonzero;
+    }
+  }
   if (threadIdx.x < p) {
     const int e = group_exp(key[threadIdx.x]);
     if (e < 0) atomicOr(flag, kOutOfRange);
-    exps[blockIdx.x * stride + threadIdx.x] = e;
+    if (!window) exps[blockIdx.y * stride + threadIdx.x] = e;
   }
 }
 
@@ -556,6 +652,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int i = 0; i < 8; ++i) x[i] = (int)k0[j] + i < rows ? rsb[src[j] + i * rstep[j]] : 0.0;
         }
+        if constexpr (PANEL) {  // A's diagonal goes to the sums by itself
+          const int64_t d = ecol[j] - (r_begin + (int64_t)c * kKC + k0[j]);
+          if (ecol[j] < eb0 && d >= 0 && d < 8)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = i == (int)d ? 0.0 : x[i];
+        }
         uint64_t w[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = digits(x[i], exp_[j]);
@@ -706,14 +808,16 @@ int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b
 }
 
 namespace {
-// Y[i][j] = sum over the splits, in order
-__global__ void panel_reduce_kernel(int64_t n, int p, int splits, const double* __restrict__ part, double* __restrict__ Y,
-                                    int ldy, const int* __restrict__ flag) {
+// Y[i][j] = sum over the splits, in order, then A's diagonal against X
+__global__ void panel_reduce_kernel(int64_t n, int p, int splits, const double* __restrict__ part,
+                                    const double* __restrict__ A, int64_t lda, const double* __restrict__ X, int ldx,
+                                    double* __restrict__ Y, int ldy, const int* __restrict__ flag) {
   if (*flag) return;  // no sums were written
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * p; e += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int g = 0; g < splits; ++g) s += part[g * n * p + e];
-    Y[e / p * ldy + e % p] = s;
+    const int64_t i = e / p, j = e % p;
+    Y[i * ldy + j] = fma(A[i * lda + i], X[i * ldx + j], s);
   }
 }
 
@@ -733,18 +837,24 @@ int panel_splits(int64_t panels, int64_t groups, int sms) {
 }
 }  // namespace
 
-// Scratch of launch_spmm_dense_digits in bytes: flag, exponents, partial sums.
+// Scratch of launch_spmm_dense_digits in bytes: flag, exponents, masks of X, partial sums.
+static size_t dense64_exps_bytes(int64_t n, int p) {
+  return ((size_t)ceil_div(n, kGroupRows) * (n + p) * sizeof(int) + 255) / 256 * 256;
+}
+static size_t dense64_mask_bytes(int64_t n) {
+  return ((size_t)(ceil_div(n, kGroupRows) + 1) * kXMask * sizeof(uint32_t) + 255) / 256 * 256;
+}
 size_t dense64_scratch_bytes(int64_t n, int p) {
-  const size_t exps = ((size_t)ceil_div(n, kGroupRows) * (n + p) * sizeof(int) + 255) / 256 * 256;
-  return 256 + exps + (size_t)kMaxSplits * n * p * sizeof(double);
+  return 256 + dense64_exps_bytes(n, p) + dense64_mask_bytes(n) + (size_t)kMaxSplits * n * p * sizeof(double);
 }
 
 // Y = A X (column i of the dense A against X; A column-major, or row-major with row_a) through digit products; false without
-// launching where A or X do not fit (odd n or lda, unaligned).  *scratch is the flag left at 1 when a
-// number is outside the digits' range: Y is then to be formed by launch_spmm_dense on that flag.
+// launching where A or X do not fit (odd n or lda, unaligned).  *scratch is the flag, not zero when a
+// number is outside the digits' range or, with `spread`, two columns of a group are too far apart: Y is
+// then to be formed by launch_spmm_dense on that flag.
 bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, const double* X, int ldx, double* Y,
-                              int ldy, void* scratch, bool row_a, int* err, cudaStream_t st) {
-  if (n < 2 || (n & 1) || (lda & 1) || lda > INT_MAX || p < 1 || p > 32 || (reinterpret_cast<uintptr_t>(A) & 15) ||
+                              int ldy, void* scratch, bool row_a, bool spread, int* err, cudaStream_t st) {
+  if (n < kGroupRows || (n & 1) || (lda & 1) || lda > INT_MAX || p < 1 || p > 32 || (reinterpret_cast<uintptr_t>(A) & 15) ||
       (reinterpret_cast<uintptr_t>(X) & 15))
     return false;
   constexpr int NB = 32;
@@ -763,22 +873,32 @@ bool launch_spmm_dense_digits(int64_t n, const double* A, int64_t lda, int p, co
   int* flag = static_cast<int*>(scratch);
   int* exps = flag + 64;
   const int64_t estride = n + p;
-  double* part = reinterpret_cast<double*>(static_cast<char*>(scratch) + 256 +
-                                           ((size_t)groups * estride * sizeof(int) + 255) / 256 * 256);
+  uint32_t* xmask = reinterpret_cast<uint32_t*>(static_cast<char*>(scratch) + 256 + dense64_exps_bytes(n, p));
+  double* part = reinterpret_cast<double*>(reinterpret_cast<char*>(xmask) + dense64_mask_bytes(n));
   LB_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
-  if (row_a)
-    exp_dense_rows_kernel<<<dim3((unsigned)panels, (unsigned)groups), 256, 0, st>>>(n, A, lda, exps, estride, flag);
-  else
-    exp_dense_kernel<<<dim3((unsigned)ceil_div(n, 8), (unsigned)groups), 256, 0, st>>>(n, A, lda, exps, estride, flag);
-  LB_LAUNCH_CHECK();
-  exp_rows_kernel<<<(unsigned)groups, 256, 0, st>>>(n, p, X, ldx, exps + n, estride, flag);
+  const unsigned gy = (unsigned)(groups + (spread && n % kGroupRows ? 1 : 0));
+  if (spread) {
+    exp_rows_kernel<true><<<dim3(1, gy), 256, 0, st>>>(n, p, X, ldx, exps + n, estride, xmask, flag);
+    LB_LAUNCH_CHECK();
+    if (row_a)
+      exp_dense_rows_kernel<true><<<dim3((unsigned)panels, gy), 256, 0, st>>>(n, A, lda, exps, estride, p, xmask, flag);
+    else
+      exp_dense_kernel<true><<<dim3((unsigned)ceil_div(n, 8), gy), 256, 0, st>>>(n, A, lda, exps, estride, p, xmask, flag);
+  } else {
+    exp_rows_kernel<false><<<dim3(1, gy), 256, 0, st>>>(n, p, X, ldx, exps + n, estride, xmask, flag);
+    LB_LAUNCH_CHECK();
+    if (row_a)
+      exp_dense_rows_kernel<false><<<dim3((unsigned)panels, gy), 256, 0, st>>>(n, A, lda, exps, estride, p, xmask, flag);
+    else
+      exp_dense_kernel<false><<<dim3((unsigned)ceil_div(n, 8), gy), 256, 0, st>>>(n, A, lda, exps, estride, p, xmask, flag);
+  }
   LB_LAUNCH_CHECK();
   gram64_kernel<kCB, NB, true><<<(unsigned)(panels * splits), kThreads, smem, st>>>(
       n, cols1<double>(A, (int)lda, 1), cols1<double>(X, ldx, p), (int)lda, 0, 0, 0, p, 0, 0, rs, exps, (int)estride,
       (int)n, flag, part, ceil_div(groups, splits), (int)panels, row_a ? 1 : 0, err);
   LB_LAUNCH_CHECK();
-  panel_reduce_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n * p, 256), 4096), 256, 0, st>>>(n, p, splits, part, Y,
-                                                                                               ldy, flag);
+  panel_reduce_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n * p, 256), 4096), 256, 0, st>>>(n, p, splits, part, A,
+                                                                                               lda, X, ldx, Y, ldy, flag);
   LB_LAUNCH_CHECK();
   return true;
 }

@@ -608,7 +608,7 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
       if (c.digits_on() && dense_digits_pay(c.A.n, p, false)) {
         c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
         if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false,
-                                     c.err_word(kErrGram), c.st)) {
+                                     c.entrywise, c.err_word(kErrGram), c.st)) {
           launch_spmm_dense<T>(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.st, c.dense_buf.as<int>());
           return;
         }
@@ -1784,7 +1784,7 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
       work.alloc(dense64_scratch_bytes(n, p));
       int* word = work.as<int>();  // the digits' flag, then the error word
       LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
-      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, false, word + 1, st)) {
+      if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, false, true, word + 1, st)) {
         launch_spmm_dense<double>(n, A, lda, p, X, ldx, Y, ldy, st, word);
         int err = 0;
         LB_CUDA(cudaMemcpyAsync(&err, word + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1811,7 +1811,7 @@ extern "C" lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, 
     work.alloc(dense64_scratch_bytes(n, p));
     int* word = work.as<int>();  // the digits' flag, then the error word
     LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
-    if (!launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, true, word + 1, st)) return LOBPCG_OK;
+    if (!launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, true, true, word + 1, st)) return LOBPCG_OK;
     int h[2] = {0, 0};
     LB_CUDA(cudaMemcpyAsync(h, word, sizeof h, cudaMemcpyDeviceToHost, st));
     LB_CUDA(cudaStreamSynchronize(st));

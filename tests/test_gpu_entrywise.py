@@ -97,3 +97,25 @@ def test_update(n, s, q, pair, in_place, kind):
         tol = (s + 8) * DF * (np.abs(x) @ np.abs(U))
         err = np.abs((o.cpu().numpy()[:, :q].astype(np.longdouble) - ref).astype(np.float64))
         assert (err <= tol).all(), (err / np.maximum(tol, 1e-300)).max()
+
+
+@pytest.mark.parametrize("kind", ["spikes", "alternate", "tail", "diagonal"])
+@pytest.mark.parametrize("n,p", [(2048, 5), (2050, 13), (1226, 32)])
+def test_dense(n, p, kind):
+    """Column i of A against X; the FMA kernel where an entry asks for it, in either storage order."""
+    import torch
+
+    import paper_2305_06668_gb300 as lb
+    rng = np.random.default_rng(n + p)
+    if kind == "diagonal":  # dominant, and X without the rows it would meet
+        A, X = 1e-3 * rng.standard_normal((n, n)), rng.standard_normal((n, p))
+        np.fill_diagonal(A, 1e8)
+        X[::64] = 0.0
+    else:
+        A, X = _far_apart(kind, n, n, p, rng)
+    ref = A.T.astype(np.longdouble) @ X.astype(np.longdouble)
+    tol = n * FMA * (np.abs(A).T @ np.abs(X))
+    At, Xt = torch.from_numpy(A).cuda(), torch.from_numpy(X).cuda()
+    for a in (At, At.t().contiguous().t()):
+        err = np.abs((lb.spmm_dense(a, Xt).cpu().numpy().astype(np.longdouble) - ref).astype(np.float64))
+        assert (err <= tol).all(), (err / np.maximum(tol, 1e-300)).max()
