@@ -21,7 +21,8 @@
 // K antisymmetric, K_ij = N_ij / (lambda_j - lambda_i), N = (S + S^T) / 2 + R (lambda_i + lambda_j) / 2.  The
 // halves of S come together through U, so K is antisymmetric to the last bit and rounding of S over a
 // small gap only turns vectors, it never takes them off orthonormality (S_ij alone did, by 4e-9 at a
-// gap of 1e-7).  Where N_ij is rounding noise of ||A|| and the gap within 1e-10 ||A|| (repeated
+// gap of 1e-7), but for the second order K^T K: steps that no longer converge, over gaps of 1e-10 ||A||,
+// are followed by steps of R / 2 alone.  Where N_ij is rounding noise of ||A|| and the gap within 1e-10 ||A|| (repeated
 // eigenvalues) K_ij = 0; over any wider gap a coupling counts whatever its size.  Where it is not small
 // against the gap (close eigenvalues that FP32 did not separate) the Jacobi angle of the pair, halved,
 // takes the quotient's place: the pair turns by a bounded angle, and the quotient applies once it is
@@ -42,7 +43,7 @@ constexpr int kCl = 8;           // CTAs of the cluster
 constexpr int kThreads = 1024;
 constexpr int kMaxNb = kMaxS / kCl;                                   // columns per CTA
 constexpr int kPer = (kMaxS * kMaxNb + kThreads - 1) / kThreads;      // elements per thread
-constexpr int kMaxSteps = 16;
+constexpr int kMaxSteps = 18;
 constexpr int kMaxSweeps32 = 14;
 
 __device__ __forceinline__ float block_sumf(float v, float* red) {
@@ -168,7 +169,7 @@ __device__ void jacobi32(int s, float* a, int ld, float* v, int nb, float tol, f
   }
 }
 
-// stop: the step that follows corrections below it is the last.
+// stop: a step whose corrections do not exceed it is the last.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
     syev_cluster_kernel(int s, const double* __restrict__ a_in, int upper_only, double* __restrict__ lam,
                         double* __restrict__ U, int* steps_out, float stop) {
@@ -226,7 +227,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
   const double noise = 1e-15 * fro;  // what the plain solver leaves off the diagonal
   float last = 1.f;
   int step = 0;
-  bool good = false;
+  bool good = false, ortho = false;
   for (; step < kMaxSteps; ++step) {
     double R[kPer], S[kPer];
 #pragma unroll
@@ -270,7 +271,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
       if (e >= cnt) break;
       const int i = e % s, j = j0 + e / s;
       double E = 0.5 * R[k];
-      if (i != j) {
+      if (i != j && !ortho) {
         const double gap = lsh[j] - lsh[i];
         const double num = 0.5 * (S[k] + __ldcg(U + j + i * s)) + (0.5 * (lsh[i] + lsh[j])) * R[k];
         // a small coupling over a normal gap counts whatever its size against ||a||: the Ritz vectors of
@@ -314,13 +315,15 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
     }
     cluster.sync();
     if (!(m < 0.75f)) break;  // diverging or NaN (the same in every CTA)
-    // small enough for the next correction, its square, to be below rounding; or no longer falling
-    // as squares do: rounding over a small gap
-    if (m <= stop || (step >= 3 && m <= 1e-5f && m >= 0.1f * last)) {
+    // small enough for the next correction, its square, to be below rounding
+    if (ortho ? m <= 1e-9f : m <= stop) {
       good = true;
       ++step;
       break;
     }
+    // no longer falling as squares do: rounding over small gaps, which turns vectors by up to m and takes
+    // them off orthonormality by the square of it, K^T K.  Steps of R / 2 alone take that back.
+    if (step >= 3 && m <= 1e-5f && m >= 0.1f * last) ortho = true;
     last = m;
   }
   // ascending eigenvalues (ties keep index order); CTA c writes its columns
