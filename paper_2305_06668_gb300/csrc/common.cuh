@@ -264,8 +264,9 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,
                  cudaStream_t st, bool two_stage = false, double tol64 = 1e-15, bool refine = true);
 
-// The cluster eigensolver behind launch_syev (syev.cu): lam[0] = NaN where it gave up.
-void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, double* U, int* steps_out, float stop,
+// The cluster eigensolver before launch_syev's (syev.cu), until the off-diagonal mass is at most tol ||a||_F:
+// lam[0] = NaN where it gave up.
+void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, double* U, int* steps_out, double tol,
                          cudaStream_t st);
 
 // Cholesky-QR step on the reduced Gram matrix M (p x p, column-major):

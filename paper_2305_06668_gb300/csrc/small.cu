@@ -980,7 +980,7 @@ void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U
   // The cluster solver from 2 columns on where the caller lets it refine (syev.cu; measured per call at s = 63, see there); this
   // kernel then runs only where that one gave up.
   const bool behind = s > 1 && refine;
-  if (behind) launch_syev_cluster(s, a, upper_only, lam, U, sweeps_out, tol64 >= 1e-12 ? 1e-5f : 1e-9f, st);
+  if (behind) launch_syev_cluster(s, a, upper_only, lam, U, sweeps_out, tol64, st);
   const double tol32 = 1e-4;  // measured: the stopping point of this stage hardly changes the total
   if (two_stage)
     syev_kernel<true><<<1, kSmallThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, sweeps_out, tol32, tol64,

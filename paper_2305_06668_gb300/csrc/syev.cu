@@ -169,7 +169,7 @@ __device__ void jacobi32(int s, float* a, int ld, float* v, int nb, float tol, f
   }
 }
 
-// stop: a step whose corrections do not exceed it is the last.
+// stop: a step with ||E||_F^2 at most this is the last.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
     syev_cluster_kernel(int s, const double* __restrict__ a_in, int upper_only, double* __restrict__ lam,
                         double* __restrict__ U, int* steps_out, float stop) {
@@ -177,7 +177,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
   __shared__ float red[32];
   __shared__ float2 cs[kMaxS / 2];
   __shared__ double lsh[kMaxS];       // lambda, written by its column's CTA
-  __shared__ float emax_all[kCl];
+  __shared__ float emax_all[kCl], esum_all[kCl];
   __shared__ int rank_of[kMaxS];
   cg::cluster_group cluster = cg::this_cluster();
   const int me = (int)cluster.block_rank(), tid = threadIdx.x;
@@ -264,7 +264,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
       }
     }
     cluster.sync();  // lambda and S complete
-    float em = 0.f;
+    float em = 0.f, es = 0.f;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       const int e = tid + k * kThreads;
@@ -287,9 +287,11 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
       }
       Eb[i + (j - j0) * ld] = E;
       em = __uint_as_float(max(__float_as_uint(em), __float_as_uint((float)E) & 0x7fffffffu));
+      es += (float)E * (float)E;
     }
     em = block_maxf(em, red);  // its barriers also complete Eb
-    if (tid < kCl) cluster.map_shared_rank(emax_all, tid)[me] = em;
+    es = block_sumf(es, red);
+    if (tid < kCl) cluster.map_shared_rank(emax_all, tid)[me] = em, cluster.map_shared_rank(esum_all, tid)[me] = es;
     double xn[kPer];
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
@@ -302,10 +304,12 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
       for (int i = 0; i < s; ++i) g = fma(X[r + i * ld], ej[i], g);
       xn[k] = X[r + (j0 + jl) * ld] + g;
     }
-    cluster.sync();  // every CTA has read X; emax_all complete
-    float m = 0.f;
-    for (int t = 0; t < kCl; ++t)
+    cluster.sync();  // every CTA has read X; emax_all and esum_all complete
+    float m = 0.f, f2 = 0.f;
+    for (int t = 0; t < kCl; ++t) {
       m = __uint_as_float(max(__float_as_uint(m), __float_as_uint(emax_all[t]) & 0x7fffffffu));
+      f2 += esum_all[t];
+    }
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       const int e = tid + k * kThreads;
@@ -315,8 +319,8 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
     }
     cluster.sync();
     if (!(m < 0.75f)) break;  // diverging or NaN (the same in every CTA)
-    // small enough for the next correction, its square, to be below rounding
-    if (ortho ? m <= 1e-9f : m <= stop) {
+    // what a step leaves off the diagonal is of second order, at most 5 ||E||_F^2 ||a||_F
+    if (ortho ? m <= 1e-9f : f2 <= stop) {
       good = true;
       ++step;
       break;
@@ -345,7 +349,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
 }  // namespace
 
 // Leaves lam[0] = NaN where the refinement did not converge (see above).
-void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, double* U, int* steps_out, float stop,
+void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, double* U, int* steps_out, double tol,
                          cudaStream_t st) {
   const int ld = s | 1, nb = (s + kCl - 1) / kCl;
   const size_t smem = ((size_t)2 * s * ld + (size_t)2 * nb * ld) * sizeof(double);
@@ -356,7 +360,7 @@ void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, d
     return true;
   }();
   (void)attr;
-  syev_cluster_kernel<<<kCl, kThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, steps_out, stop);
+  syev_cluster_kernel<<<kCl, kThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, steps_out, (float)(tol / 5.0));
   LB_LAUNCH_CHECK();
 }
 
