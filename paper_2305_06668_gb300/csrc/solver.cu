@@ -1969,12 +1969,21 @@ extern "C" lobpcg_status lobpcg_update_f32(int64_t n, int nseg, const float* con
   });
 }
 
+namespace {
+// The refinement writes U and lam[0] before the kernel behind it reads a, so results over a (which
+// that kernel alone reads first) leave the refinement out.
+bool syev_refines(int s, const double* a, const double* lam, const double* U) {
+  const double* end = a + (size_t)s * s;
+  return !(U < end && a < U + (size_t)s * s) && !(lam < end && a < lam + s);
+}
+}  // namespace
+
 extern "C" lobpcg_status lobpcg_syev_f64(int s, const double* a, double* lam, double* U,
                                          lobpcg_stream stream) {
   return guarded(nullptr, [&]() -> lobpcg_status {
     require(s >= 1 && s <= kMaxS && a && lam && U, "lobpcg_syev_f64: need 1 <= s <= 96 and non-NULL arrays");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    launch_syev(s, a, false, lam, U, nullptr, st);
+    launch_syev(s, a, false, lam, U, nullptr, st, false, 1e-15, syev_refines(s, a, lam, U));
     LB_CUDA(cudaStreamSynchronize(st));
     return LOBPCG_OK;
   });
@@ -1986,7 +1995,7 @@ extern "C" lobpcg_status lobpcg_syev2_f64(int s, const double* a, double tol, do
     require(s >= 1 && s <= kMaxS && a && lam && U, "lobpcg_syev2_f64: need 1 <= s <= 96 and non-NULL arrays");
     require(tol >= 0.0 && tol < 1e-6, "lobpcg_syev2_f64: need 0 <= tol < 1e-6");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    launch_syev(s, a, false, lam, U, nullptr, st, true, tol > 0.0 ? tol : 1e-15);
+    launch_syev(s, a, false, lam, U, nullptr, st, true, tol > 0.0 ? tol : 1e-15, syev_refines(s, a, lam, U));
     LB_CUDA(cudaStreamSynchronize(st));
     return LOBPCG_OK;
   });
