@@ -53,6 +53,17 @@ namespace {
 // ~d ||A||, 1e-12 x 2000 = 2e-9 for tol 1e-8 on the CI-like workload).
 constexpr double kTauDf = 1e-12;
 
+// Whether an allocation failed for want of memory (the error is then cleared); throws on any other failure.
+bool out_of_memory(cudaError_t e) {
+  if (e != cudaErrorMemoryAllocation) {
+    LB_CUDA(e);
+    return false;
+  }
+  cudaGetLastError();
+  return true;
+}
+void trim_pools();
+
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
@@ -61,13 +72,21 @@ struct DevBuf {
   DevBuf& operator=(const DevBuf&) = delete;
   ~DevBuf() { release(); }  // also on an exception between allocation and the explicit release
   void ensure(size_t b) {
-    if (b <= bytes) return;
-    if (p) cudaFree(p);
-    p = nullptr;
-    bytes = 0;
-    if (b == 0) return;
-    LB_CUDA(cudaMalloc(&p, b));
+    if (!try_ensure(b)) LB_CUDA(cudaErrorMemoryAllocation);
+  }
+  // false where the device has no such memory, also after the workspace pools have given theirs back
+  bool try_ensure(size_t b) {
+    if (b <= bytes) return true;
+    release();
+    if (out_of_memory(cudaMalloc(&p, b))) {
+      trim_pools();
+      if (out_of_memory(cudaMalloc(&p, b))) {
+        p = nullptr;
+        return false;
+      }
+    }
     bytes = b;
+    return true;
   }
   void release() {
     if (p) cudaFree(p);
@@ -140,11 +159,23 @@ struct PoolBuf {
     if (p) cudaFreeAsync(p, st);
   }
   void alloc(size_t bytes) { LB_CUDA(cudaMallocFromPoolAsync(&p, bytes, work_pool(), st)); }
+  // false where the device has no such memory: a kernel that needs none runs instead
+  bool try_alloc(size_t bytes) {
+    if (!out_of_memory(cudaMallocFromPoolAsync(&p, bytes, work_pool(), st))) return true;
+    p = nullptr;
+    return false;
+  }
   template <class T>
   T* as() const {
     return static_cast<T*>(p);
   }
 };
+
+void trim_pools() {
+  std::lock_guard<std::mutex> g(work_mutex());
+  for (int d = 0; d < kMaxDevices; ++d)
+    if (work_pools()[d]) LB_CUDA(cudaMemPoolTrimTo(work_pools()[d], 0));
+}
 
 double* pinned_take() {
   {
@@ -406,13 +437,13 @@ struct lobpcg_ctx {
   DevBuf tri_scratch;  // its FP32 scratch (tridiag_scratch_floats(n, a))
   DevBuf gram_buf;         // exponents of the digit Grams (allocated when first used)
   int* gram_ints = nullptr;
+  // null where there is no memory for them: the older kernels need none
   int* gram_scratch() {
-    if (!gram_ints) {
-      gram_buf.ensure(gram64_scratch_ints(A.n) * sizeof(int));
+    if (!gram_ints && !workspace_only && gram_buf.try_ensure(gram64_scratch_ints(A.n) * sizeof(int)))
       gram_ints = gram_buf.as<int>();
-    }
     return gram_ints;
   }
+  bool workspace_only = false;  // a building-block call: its memory is the pool's
   DevBuf dense_buf;  // exponents and partial sums of the dense digit product
   double* host = nullptr;  // pinned readback area
   Stats stats;
@@ -605,8 +636,7 @@ void spmm_product(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
                           false, var);
   else {
     if constexpr (std::is_same<T, double>::value) {
-      if (c.digits_on() && dense_digits_pay(c.A.n, p, false)) {
-        c.dense_buf.ensure(dense64_scratch_bytes(c.A.n, p));
+      if (c.digits_on() && dense_digits_pay(c.A.n, p, false) && c.dense_buf.try_ensure(dense64_scratch_bytes(c.A.n, p))) {
         if (launch_spmm_dense_digits(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.dense_buf.p, false,
                                      c.entrywise, c.err_word(kErrGram), c.st)) {
           launch_spmm_dense<T>(c.A.n, c.A.dense, c.A.ld, p, X, ldx, Y, ldy, c.st, c.dense_buf.as<int>());
@@ -688,8 +718,9 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
     // launch) forms the partials
     if (c.digits_on() && gram_digits_pay(c.A.n, pa, pb, upper, c.df_on)) {
       int* flag = c.gram_scratch();
-      parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.entrywise, c.err_word(kErrGram),
-                                   c.st);
+      if (flag)
+        parts = gram_partials_digits(c.A.n, a, b, upper, c.Gpart, c.max_ctas, flag, c.entrywise,
+                                     c.err_word(kErrGram), c.st);
       if (parts && c.entrywise && c.df_on) {  // columns far apart, all in range: double-float, not the FMAs
         int* h = reinterpret_cast<int*>(c.host);
         LB_CUDA(cudaMemcpyAsync(h, flag, sizeof(int), cudaMemcpyDeviceToHost, c.st));
@@ -1657,9 +1688,11 @@ struct ScratchCtx {
     c.max_ctas = 2 * c.sms;
     lobpcg_options_default(&c.opt);
     const size_t small = (c.small_bytes() + 255) / 256 * 256;
-    mem.alloc(small + gram64_scratch_ints(n) * sizeof(int));
+    c.workspace_only = true;
+    const bool digits = mem.try_alloc(small + gram64_scratch_ints(n) * sizeof(int));
+    if (!digits) mem.alloc(small);
     c.lay_out_small(mem.as<double>());
-    c.gram_ints = reinterpret_cast<int*>(mem.as<char>() + small);
+    if (digits) c.gram_ints = reinterpret_cast<int*>(mem.as<char>() + small);
     c.host = pinned_take();
   }
   ~ScratchCtx() {
@@ -1780,8 +1813,7 @@ extern "C" lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
     require(p >= 1 && p <= 32 && ldx >= p && ldy >= p, "lobpcg_spmm_dense_f64: need 1 <= p <= 32, ld >= p");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     PoolBuf work(st);
-    if (dense_digits_pay(n, p, false)) {
-      work.alloc(dense64_scratch_bytes(n, p));
+    if (dense_digits_pay(n, p, false) && work.try_alloc(dense64_scratch_bytes(n, p))) {
       int* word = work.as<int>();  // the digits' flag, then the error word
       LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
       if (launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, false, true, word + 1, st)) {
@@ -1806,9 +1838,8 @@ extern "C" lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, 
     require(p >= 1 && p <= 32 && ldx >= p && ldy >= p, "lobpcg_spmm_dense_rows_f64: need 1 <= p <= 32, ld >= p");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     *done = 0;
-    if (!dense_digits_pay(n, p, true)) return LOBPCG_OK;
     PoolBuf work(st);
-    work.alloc(dense64_scratch_bytes(n, p));
+    if (!dense_digits_pay(n, p, true) || !work.try_alloc(dense64_scratch_bytes(n, p))) return LOBPCG_OK;
     int* word = work.as<int>();  // the digits' flag, then the error word
     LB_CUDA(cudaMemsetAsync(word + 1, 0, sizeof(int), st));
     if (!launch_spmm_dense_digits(n, A, lda, p, X, ldx, Y, ldy, work.p, true, true, word + 1, st)) return LOBPCG_OK;
@@ -2043,9 +2074,8 @@ extern "C" lobpcg_status lobpcg_ortho_against_f64(int64_t n, int p, double* X, i
 
 extern "C" lobpcg_status lobpcg_trim_workspace(void) {
   return guarded(nullptr, [&]() -> lobpcg_status {
+    trim_pools();
     std::lock_guard<std::mutex> g(work_mutex());
-    for (int d = 0; d < kMaxDevices; ++d)
-      if (work_pools()[d]) LB_CUDA(cudaMemPoolTrimTo(work_pools()[d], 0));
     for (double* h : pinned_list()) cudaFreeHost(h);
     pinned_list().clear();
     return LOBPCG_OK;
