@@ -37,7 +37,6 @@ WORKLOAD = "CI-like sparse symmetric n=2,000,000, ~65 nnz/row, k=16 (+5 extra), 
 ORACLE_RECORD = os.path.join(ROOT, "oracle", "records", "ci2m_seed0.json")
 FP64_PEAK_SOURCE = "FP64 FMA rate measured in this run (lobpcg_probe_fma_rate)"
 DIGIT_PRODUCTS = 34  # FP16 products of one FP64 multiply-add (csrc/slices.cuh)
-TENSOR_PEAK = 1872.3  # TFLOP/s, cuBLAS bf16 on this part
 DF_OPS_PER_TERM = 15  # FP32 operations of one double-float multiply-add (dfloat.cuh df_fma)
 
 
@@ -133,6 +132,15 @@ def measured_peaks():
         return float(p["hbm_gbs"]), "measured"
     except Exception:
         return 6800.0, "fallback"
+
+
+def tensor_peak():
+    """Dense FP16 / BF16 tensor rate in TFLOP/s and its source."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"]), "measured (cuBLAS bf16, burst)"
+    except Exception:
+        return 1900.0, "fallback (cuBLAS bf16, burst)"
 
 
 def mean_offdiag_row_norm(a):
@@ -341,30 +349,38 @@ def run_ours(args):
                                       "frac": f64 / t64 / 1e12 / fp64_peak, "traffic": None,
                                       "flops_per_launch": f64, "avg_launch_s": t64,
                                       "peak_source": FP64_PEAK_SOURCE}
-    # the FP64 block updates of the refinement, timed per launch with CUDA events.  Above the size
-    # rule they are exact digit products on the tensor cores: 34 FP16 products per FP64 multiply-add
-    # (of the padded 32 columns only the used ones are counted), so the roofline counts FP16 tensor
-    # flops; the plain FP64 form below counts FP64 ones.
-    ut = sum(i["update_fp64_seconds"] for _, i, _, _ in infos)
-    uf = sum(i["update_fp64_flops"] for _, i, _, _ in infos)
-    ul = sum(i["update_fp64_launches"] for _, i, _, _ in infos)
-    if ul and ut > 0:
-        if df:
-            ops = uf * DIGIT_PRODUCTS
-            rooflines["update_fp64"] = {"kernel": "update64_kernel (FP64 block updates through exact FP16 digit "
-                                                  "products, tcgen05: X = V u_x, P = V u_p, W -= Y C, W <- W T)",
-                                        "bound": "tensor", "achieved": ops / ut / 1e12, "peak": TENSOR_PEAK,
-                                        "unit": "TFLOP/s", "frac": ops / ut / 1e12 / TENSOR_PEAK,
-                                        "ops": "FP16 tensor flops, 34 digit products per FP64 multiply-add",
-                                        "fp64_equivalent_tflops": uf / ut / 1e12, "traffic": None,
-                                        "flops_per_launch": ops / ul, "avg_launch_s": ut / ul,
-                                        "peak_source": "cuBLAS bf16 throughput, burst"}
-        else:
-            rooflines["update_fp64"] = {"kernel": "update_kernel<double> (FP64 block updates)", "bound": "alu",
-                                        "achieved": uf / ut / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
-                                        "frac": uf / ut / 1e12 / fp64_peak, "traffic": None,
-                                        "flops_per_launch": uf / ul, "avg_launch_s": ut / ul,
-                                        "peak_source": FP64_PEAK_SOURCE}
+    # the FP64 block updates of the refinement, timed per launch with CUDA events: digit products above
+    # their size rules (34 FP16 products per FP64 multiply-add, of the padded 32 columns only the used ones
+    # counted), the double-float or FMA kernels below, each against its own peak
+    def total(key):
+        return sum(i[key] for _, i, _, _ in infos)
+    dt_, df_, dl_ = total("update_digit_seconds"), total("update_digit_flops"), total("update_digit_launches")
+    ot, of, ol = (total("update_fp64_seconds") - dt_, total("update_fp64_flops") - df_,
+                  total("update_fp64_launches") - dl_)
+    if dl_ and dt_ > 0:
+        peak, source = tensor_peak()
+        ops = df_ * DIGIT_PRODUCTS
+        rooflines["update_fp64"] = {"kernel": "update64_kernel (FP64 block updates through FP16 digit products, "
+                                              "tcgen05: X = V u_x, P = V u_p, W -= Y C, W <- W T)",
+                                    "bound": "alu",
+                                    "limited_by": "integer pipe (cutting into digits, joining of the sums)",
+                                    "achieved": ops / dt_ / 1e12, "peak": peak, "unit": "TFLOP/s",
+                                    "frac": ops / dt_ / 1e12 / peak,
+                                    "ops": "FP16 tensor flops, 34 digit products per FP64 multiply-add",
+                                    "fp64_equivalent_tflops": df_ / dt_ / 1e12, "traffic": None,
+                                    "launches": dl_, "flops_per_launch": ops / dl_, "avg_launch_s": dt_ / dl_,
+                                    "peak_source": source}
+    if ol and ot > 0:
+        ops = of / 2.0 * DF_OPS_PER_TERM if df else of
+        rooflines["update_fp64_small"] = {
+            "kernel": ("update_df_async_kernel (FP64 block updates below the size rule, double-float)" if df
+                       else "update_kernel<double> (FP64 block updates below the size rule)"),
+            "bound": "alu", "achieved": ops / ot / 1e12, "peak": fp32_peak / 2 if df else fp64_peak,
+            "unit": "TFLOP/s", "frac": ops / ot / 1e12 / (fp32_peak / 2 if df else fp64_peak),
+            "fp64_equivalent_tflops": of / ot / 1e12, "traffic": None, "launches": ol,
+            "flops_per_launch": ops / ol, "avg_launch_s": ot / ol,
+            "peak_source": ("FP32 FMA instruction rate measured in this run (lobpcg_probe_fma_rate / 2)" if df
+                            else FP64_PEAK_SOURCE)}
     # the FP32 Rayleigh-Ritz Grams (tcgen05 kernel): algorithmic bytes 2 n s 4 per Gram over the
     # FP32 part of the Rayleigh-Ritz Gram phase
     gb = sum(i["rr_gram32_bytes"] for _, i, _, _ in infos)

@@ -231,6 +231,10 @@ LOBPCG_API lobpcg_status lobpcg_solve_batched(lobpcg_ctx* const* ctxs, int nprob
                                               double* const* resnorms, lobpcg_info* infos, lobpcg_status* statuses,
                                               int nthreads);
 
+/* With opt.profile: the part of the last solve's update_fp64_seconds, _flops and _launches that ran as digit
+ * products on the tensor cores (df_products); the rest ran on the FP32 or FP64 pipes. */
+LOBPCG_API lobpcg_status lobpcg_digit_updates(lobpcg_ctx* ctx, double* seconds, double* flops, int64_t* launches);
+
 /* Releases the context and everything it owns.  NULL-safe. */
 LOBPCG_API void lobpcg_destroy(lobpcg_ctx* ctx);
 

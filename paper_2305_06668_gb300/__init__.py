@@ -80,7 +80,7 @@ def lib():
                      "lobpcg_probe_fma_rate", "lobpcg_gram_f64_df", "lobpcg_update_f64_df",
                      "lobpcg_spmm_csr_f64_df", "lobpcg_gram_f32_tcgen05", "lobpcg_precond_tridiag",
                      "lobpcg_mixed_switch_replay", "lobpcg_trim_workspace",
-                     "lobpcg_spmm_dense_rows_f64"):
+                     "lobpcg_spmm_dense_rows_f64", "lobpcg_digit_updates"):
             getattr(L, name).restype = C.c_int
         L.lobpcg_last_error.restype = C.c_char_p
         L.lobpcg_last_error.argtypes = [C.c_void_p]
@@ -227,6 +227,10 @@ class Solver:
         d = {f: getattr(info, f) for f, _ in _Info._fields_}
         d["phase_seconds"] = dict(zip(PHASES, list(info.phase_seconds)))
         d["phase_seconds_fp64"] = dict(zip(PHASES, list(info.phase_seconds_fp64)))
+        sec, fl, num = C.c_double(), C.c_double(), C.c_int64()
+        lib().lobpcg_digit_updates(self._ctx, C.byref(sec), C.byref(fl), C.byref(num))
+        d["update_digit_seconds"], d["update_digit_flops"] = sec.value, fl.value
+        d["update_digit_launches"] = num.value
         return Result(st, evals, evecs, res, d)
 
     @property

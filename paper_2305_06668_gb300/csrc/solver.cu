@@ -252,7 +252,8 @@ struct Profiler {
     used = 0;
     phase.clear();
     kused = 0;
-    kflops = 0.0;
+    kdigits.clear();
+    kflops = kflops_digits = 0.0;
   }
   void mark(int ph) {
     if (!on) return;
@@ -281,8 +282,9 @@ struct Profiler {
   // event pairs around every FP64 block update (the FP64-bound update kernel), with the
   // algorithmic flops of each: 2 n s q per product
   std::vector<cudaEvent_t> kpool;
+  std::vector<char> kdigits;  // of each pair: whether it ran on digit products
   size_t kused = 0;
-  double kflops = 0.0;
+  double kflops = 0.0, kflops_digits = 0.0;
   void kmark() {
     if (kused == kpool.size()) {
       cudaEvent_t e;
@@ -292,10 +294,18 @@ struct Profiler {
     LB_CUDA(cudaEventRecord(kpool[kused], st));
     ++kused;
   }
-  // seconds of the timed updates (after finish's synchronisation)
-  double kseconds() {
+  void kdone(double flops, bool digits) {
+    kmark();
+    kdigits.resize(kused / 2);
+    kdigits.back() = digits;
+    kflops += flops;
+    if (digits) kflops_digits += flops;
+  }
+  // seconds of the timed updates, or of those on digit products (after finish's synchronisation)
+  double kseconds(bool digits_only) {
     double t = 0.0;
     for (size_t i = 0; i + 1 < kused; i += 2) {
+      if (digits_only && !kdigits[i / 2]) continue;
       float ms = 0.f;
       LB_CUDA(cudaEventElapsedTime(&ms, kpool[i], kpool[i + 1]));
       t += ms * 1e-3;
@@ -596,6 +606,7 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
   const bool timed = c.prof.on && sizeof(T) == 8;
   if (timed) c.prof.kmark();
   int parts;
+  bool on_digits = false;
   if constexpr (std::is_same<T, double>::value) {
     // digit products on the tensor cores from the size where they are the faster form
     parts = 0;
@@ -612,16 +623,14 @@ int update(lobpcg_ctx& c, const UpdateJob<T>& job, const double* U, int s, int q
     if (digits)
       parts = launch_update_digits(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.entrywise,
                                    c.err_word(kErrUpdate), c.st);
+    on_digits = parts > 0;
     if (!parts)
       parts = c.df_on ? launch_update_df(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st)
                       : launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
   } else {
     parts = launch_update<T>(c.A.n, job, U, s, q, alpha, lam, norm_part, c.max_ctas, c.st);
   }
-  if (timed) {
-    c.prof.kmark();
-    c.prof.kflops += 2.0 * (double)c.A.n * s * q * job.nprod;
-  }
+  if (timed) c.prof.kdone(2.0 * (double)c.A.n * s * q * job.nprod, on_digits);
   return parts;
 }
 
@@ -1621,7 +1630,7 @@ extern "C" lobpcg_status lobpcg_solve(lobpcg_ctx* c, int k, double tol, const do
       info->kernel_launches = launch_counter() - launches0;
       info->spmm_launches = c->stats.spmm_launches;
       info->precond_fallback = c->stats.precond_fallback;
-      info->update_fp64_seconds = c->prof.on ? c->prof.kseconds() : 0.0;
+      info->update_fp64_seconds = c->prof.on ? c->prof.kseconds(false) : 0.0;
       info->update_fp64_flops = c->prof.on ? c->prof.kflops : 0.0;
       info->update_fp64_launches = c->prof.on ? (int64_t)(c->prof.kused / 2) : 0;
       info->spmm_variant_fp32 = c->var32;
@@ -1639,6 +1648,19 @@ extern "C" lobpcg_status lobpcg_solve(lobpcg_ctx* c, int k, double tol, const do
       if (!std::isfinite(evals[j]) || !std::isfinite(resnorms[j]))
         return fail(c, LOBPCG_EBREAKDOWN, "lobpcg_solve: non-finite result (basis breakdown)");
     if (!ph.converged) return fail(c, LOBPCG_ENOCONV, "lobpcg_solve: maxiter reached before convergence");
+    return LOBPCG_OK;
+  });
+}
+
+extern "C" lobpcg_status lobpcg_digit_updates(lobpcg_ctx* c, double* seconds, double* flops, int64_t* launches) {
+  if (!c || !seconds || !flops || !launches) {
+    fail(c, LOBPCG_EINVAL, "lobpcg_digit_updates: NULL argument");
+    return LOBPCG_EINVAL;
+  }
+  return guarded(c, [&]() -> lobpcg_status {
+    *seconds = c->prof.on ? c->prof.kseconds(true) : 0.0;
+    *flops = c->prof.on ? c->prof.kflops_digits : 0.0;
+    *launches = c->prof.on ? (int64_t)std::count(c->prof.kdigits.begin(), c->prof.kdigits.end(), (char)1) : 0;
     return LOBPCG_OK;
   });
 }

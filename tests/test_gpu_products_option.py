@@ -34,3 +34,19 @@ def test_minus_one_is_another_arithmetic(dense):
         assert out[df].status == lb.OK
     assert np.abs(out[0].evals - out[-1].evals).max() <= 1e-12 * max(1.0, np.abs(out[0].evals).max())
     assert not torch.equal(out[0].evecs, out[-1].evecs)
+
+
+def test_profile_tells_the_digit_updates():
+    torch = cuda()
+    import paper_2305_06668_gb300 as lb
+    n, k = 100_003, 8
+    a = synth.sparse_cfg1(n=n, seed=11)
+    x0 = dev(torch, synth.diag_guess(a.diag, k + 4, seed=11))
+    for df in (0, -1):
+        s = lb.Solver(**lb.upload_csr(a), extra=4, df_products=df, profile=True)
+        i = s.solve(k, 1e-9, X0=x0).info
+        s.close()
+        assert 0 <= i["update_digit_launches"] <= i["update_fp64_launches"]
+        assert (i["update_digit_launches"] > 0) == (df == 0)
+        assert (i["update_digit_flops"] > 0) == (i["update_digit_seconds"] > 0) == (df == 0)
+        assert i["update_digit_seconds"] <= i["update_fp64_seconds"]
