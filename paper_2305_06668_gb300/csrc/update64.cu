@@ -5,14 +5,16 @@
 // What bounds it.  As FP64 FMAs (2 per clock and SM) the pair X, AX of 10^6 rows, 63 columns to 21,
 // takes 5 ms, in double-float on the FP32 pipes 2.4 ms; its bytes take 0.2 ms and its digit products
 // 0.12 ms of tensor time.  What is left to pay is the cutting into digits and the joining of the sums, on
-// the integer pipe: a call of that pair with norms went from 2,870 (double-float) to 805 us.  Four epilogue warps instead of eight took 1,480, stores
-// by row instead of turned ones and residuals exchanged behind barriers 868.
+// the integer pipe (60% busy at 200,000 rows; tensor pipe 13%, DRAM 18%): a call of that pair with norms
+// went from 2,890 (double-float) to 800 us, 910 with the test of spread below.  Four epilogue warps instead
+// of eight took 1,480, stores by row instead of turned ones and residuals exchanged behind barriers 868.
 //
 // Scaling.  Column l of V and row l of U are scaled against each other by the power of two above
 // max_j |alpha U_lj|, so an entry of a row counts by the most it contributes to any output; then every
 // row of V has one exponent and every column of U one.  A row's entries are held to 2^-56 of its
 // largest contribution, digit sums are exact, each product is rounded to FP64 once and the base is
-// added in FP64.
+// added in FP64.  That is a bound against the row's norm; SPREAD finds the rows with an output whose own
+// terms are far below it.
 //
 // One persistent CTA per SM takes a contiguous range of 128-row tiles:
 //   * warps 0..15, splitters: warp w owns rows 8 w .. 8 w + 7 of the tile.  Its lane 0 copies them
@@ -28,8 +30,7 @@
 //     to four lanes per row, which add the base, store 32-byte pieces of rows and, from the pair's two
 //     elements, keep the sum of squares and the maximum of the residuals of their column.
 // Rows with an infinity, a NaN or an exponent outside 2^+-400 (and all rows when U has one), and with
-// `spread` rows with an output far below the rest (below), are formed by their epilogue threads with
-// FP64 FMAs.
+// SPREAD rows with an output far below the rest, are formed by their epilogue warp with FP64 FMAs.
 #include <algorithm>
 #include <climits>
 
@@ -123,12 +124,12 @@ __device__ __forceinline__ void scale_u(UScale& u, const double* us, int s, int 
   __syncthreads();
 }
 
-// NC: 32-column chunks of V (ceil(s / 32)).
-template <int NC, bool NORM>
+// NC: 32-column chunks of V (ceil(s / 32)).  SPREAD: rows too far apart are found and formed with FMAs.
+template <int NC, bool NORM, bool SPREAD>
 __global__ void __launch_bounds__(kThreads, 1)
     update64_kernel(int64_t n, UpdateJob<double> job, const double* __restrict__ U, int s, int q, double alpha,
                     const double* __restrict__ lam, double* __restrict__ norm_part, int64_t tiles_per_cta,
-                    int ts, int spread, int* __restrict__ err) {
+                    int ts, int* __restrict__ err) {
   constexpr int KP = NC * kKC;
   constexpr uint32_t kSliceU = u_slice(KP), kSBOU = KP / 8 * 128;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t somem = __ballot_sync(0xffffffffu, some);
         bad |= E <= 0 && (somem & (0x01010101u << r)) != 0u;
       }
-      const bool judge = spread && E > 0 && !bad;
+      const bool judge = SPREAD && E > 0 && !bad;
       if (E <= 0 || bad) E = kExpOne;
       uint32_t near[NC];  // entries of the row within kNear binades of 2^E, this lane's in its byte
 #pragma unroll
@@ -278,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           // the row's exponent in the entry's own scale; a bad row's digits are not used
           w[i] = digits(bad ? 0.0 : x[c][i], v > -4000 ? E - v : 4 * kExpOne);
         }
-        if (spread) {
+        if constexpr (SPREAD) {
           // |leading digit| >= 9: at least 2^51 of the 2^54 that 2^E is
 #pragma unroll
           for (int i = 0; i < 8; ++i)
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (++buf == ts) buf = 0, tph ^= 1u;
       }
       if (!done) break;
-      if (spread) {
+      if constexpr (SPREAD) {
         int count = 0;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
@@ -575,12 +576,12 @@ __global__ void __launch_bounds__(256) update64_sample_kernel(int64_t n, UpdateJ
   if (lane == 0 && total) atomicAdd(count, total);
 }
 
-template <int NC, bool NORM>
+template <int NC, bool NORM, bool SPREAD>
 int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, int s, int q, double alpha,
-                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, bool spread, int* err,
+                    const double* lam, double* norm_part, int max_ctas, size_t smem, int ts, int* err,
                     cudaStream_t st) {
   static const bool attr = [&] {
-    LB_CUDA(cudaFuncSetAttribute(update64_kernel<NC, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBudget - kStatic)));
+    LB_CUDA(cudaFuncSetAttribute(update64_kernel<NC, NORM, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemBudget - kStatic)));
     return true;
   }();
   (void)attr;
@@ -590,8 +591,8 @@ int update64_launch(int64_t n, const UpdateJob<double>& job, const double* U, in
   const int64_t tiles = ceil_div(n, kTile);
   const int64_t per = ceil_div(tiles, std::min<int64_t>(std::min<int64_t>(max_ctas, sms), tiles));
   const int64_t ctas = ceil_div(tiles, per);
-  update64_kernel<NC, NORM><<<(unsigned)ctas, kThreads, smem, st>>>(n, job, U, s, q, alpha, lam, norm_part, per,
-                                                                    ts, spread ? 1 : 0, err);
+  update64_kernel<NC, NORM, SPREAD><<<(unsigned)ctas, kThreads, smem, st>>>(n, job, U, s, q, alpha, lam, norm_part, per,
+                                                                    ts, err);
   LB_LAUNCH_CHECK();
   return (int)ctas;
 }
@@ -620,12 +621,19 @@ int launch_update_digits(int64_t n, const UpdateJob<double>& job, const double* 
   const int ts = fixed + 2 * (size_t)kBuf <= kSmemBudget - kStatic ? 2 : 1;
   const size_t smem = fixed + (size_t)ts * kBuf;
   if (smem > kSmemBudget - kStatic) return 0;
-#define LB_UPDATE64(NC)                                                                                          \
-  return norm_part ? update64_launch<NC, true>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, spread, err, st)        \
-                   : update64_launch<NC, false>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, spread, err, st)
-  if (nc == 1) LB_UPDATE64(1);
-  if (nc == 2) LB_UPDATE64(2);
-  LB_UPDATE64(3);
+#define LB_UPDATE64_(NC, NORM, SPREAD) \
+  return update64_launch<NC, NORM, SPREAD>(n, job, U, s, q, alpha, lam, norm_part, max_ctas, smem, ts, err, st)
+#define LB_UPDATE64(NC)                                \
+  {                                                    \
+    if (norm_part && spread) LB_UPDATE64_(NC, true, true);   \
+    if (norm_part) LB_UPDATE64_(NC, true, false);      \
+    if (spread) LB_UPDATE64_(NC, false, true);         \
+    LB_UPDATE64_(NC, false, false);                    \
+  }
+  if (nc == 1) LB_UPDATE64(1)
+  if (nc == 2) LB_UPDATE64(2)
+  LB_UPDATE64(3)
+#undef LB_UPDATE64_
 #undef LB_UPDATE64
 }
 
