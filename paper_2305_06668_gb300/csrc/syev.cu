@@ -6,11 +6,17 @@
 // 62 rounds a sweep at s = 63, 8k clocks of one SM's FP64 pipe, and a serial chain of FP64 divisions
 // and square roots before them, over 8 or 9 sweeps.  FP32 rounds have no such pipe to wait for, and one
 // refinement step is four s x s x s products (1 M multiply-adds at s = 63) that eight SMs share; it
-// squares the error, so two or three steps take FP32's 1e-6 to FP64's rounding.  Kernel at s = 63:
-// two-stage 1,700 -> 370 us, plain 2,110 (mean) -> 500 (largest); at s = 12 plain 161 -> 44.  The FP32
-// rounds, latency-bound, are about two thirds of it.  The solver's FP64 phases keep plain Jacobi: with this
-// kernel in them a mixed + diagonal solve of n = 10^5 did not converge in 4,000 iterations and a random
-// start of n = 2,000 broke down, for a reason that was not found.
+// squares the error, so two or three steps take FP32's 1e-6 to FP64's rounding.  Microseconds per call,
+// one-CTA Jacobi (plain) and this: s = 3 122, 93   8 186, 98   12 239, 107   24 520, 148   63 3,680, 468.  The FP32
+// rounds, latency-bound, are about two thirds of it (counters at s = 63: FP64 pipe 17%, integer 21%, the
+// warps wait at barriers).
+//
+// The solver's FP64 phases keep plain Jacobi.  With this kernel in them the mixed + diagonal form on one
+// matrix (n = 10^5) needs more than 4,000 iterations from each of five starts 1e-14 apart, where Jacobi
+// takes 885 to 3,929; on another both take the same.  Eigenvalues and vectors agree in every iteration
+// compared to Jacobi's own rounding (1e-14, entries above 1e-14 to 5e-12 of themselves), so what slows
+// that solve is not known.  Random starts of n = 2,000 fail with either kernel (9 of 24 with Jacobi, 3 of
+// 24 with this one).
 //
 // Layout.  Every CTA holds all of A and X in shared memory.  In the FP32 stage every CTA rotates its own
 // copy of the matrix (the same operations, so the same rotations) but only its own rows of the
@@ -169,10 +175,10 @@ __device__ void jacobi32(int s, float* a, int ld, float* v, int nb, float tol, f
   }
 }
 
-// stop: a step with ||E||_F^2 at most this is the last.
+// stop, mstop: a step with ||E||_F^2 and max |E| at most these is the last.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
     syev_cluster_kernel(int s, const double* __restrict__ a_in, int upper_only, double* __restrict__ lam,
-                        double* __restrict__ U, int* steps_out, float stop) {
+                        double* __restrict__ U, int* steps_out, float stop, float mstop) {
   extern __shared__ double sm[];
   __shared__ float red[32];
   __shared__ float2 cs[kMaxS / 2];
@@ -320,7 +326,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThreads)
     cluster.sync();
     if (!(m < 0.75f)) break;  // diverging or NaN (the same in every CTA)
     // what a step leaves off the diagonal is of second order, at most 5 ||E||_F^2 ||a||_F
-    if (ortho ? m <= 1e-9f : f2 <= stop) {
+    if (ortho ? m <= 1e-9f : f2 <= stop && m <= mstop) {
       good = true;
       ++step;
       break;
@@ -360,7 +366,8 @@ void launch_syev_cluster(int s, const double* a, bool upper_only, double* lam, d
     return true;
   }();
   (void)attr;
-  syev_cluster_kernel<<<kCl, kThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, steps_out, (float)(tol / 5.0));
+  syev_cluster_kernel<<<kCl, kThreads, smem, st>>>(s, a, upper_only ? 1 : 0, lam, U, steps_out, (float)(tol / 5.0),
+                                                  tol < 1e-12 ? 1e-9f : 1.f);
   LB_LAUNCH_CHECK();
 }
 
