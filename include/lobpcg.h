@@ -309,29 +309,46 @@ LOBPCG_API lobpcg_status lobpcg_spmm_dense_f64(int64_t n, const double* A, int64
                                     const double* X, int ldx, double* Y, int ldy,
                                     lobpcg_stream stream);
 
-/* The same product (column i of A against X) of a row-major A, read in place.  *done (host) is 0, and Y not
- * written, where this form does not apply: fewer than 1.5e7 multiply-adds, odd n or lda, A or X not 16-byte
- * aligned, or a number that is infinite, NaN or outside about 2^+-400 (zeros apart); pass the
+/* The same product (column i of A against X) of a row-major A, read in place.  *done (host) is 0, and Y
+ * not written, where this form does not apply: fewer than 1.5e7 multiply-adds, odd n or lda, A or X not
+ * 16-byte aligned, a number that is infinite, NaN or outside about 2^+-400 (zeros and the diagonal apart),
+ * columns that are large at different rows (see lobpcg_gram_f64), or no memory for its workspace; pass the
  * column-major matrix to lobpcg_spmm_dense_f64 then. */
 LOBPCG_API lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, int64_t lda, int p, const double* X,
                                                     int ldx, double* Y, int ldy, int* done, lobpcg_stream stream);
 
 /* C = X^T Y (the Gram / projected matrices of Algorithm 1 and Eq. (CDOrtho)).
- * X: n x p (ldx), Y: n x q (ldy), p, q <= 96.  C: device, column-major p x q. */
+ * X: n x p (ldx), Y: n x q (ldy), p, q <= 96.  C: device, column-major p x q.
+ *
+ * From about 2e7 multiply-adds on (128 of them a row, one 16-byte aligned even row stride) the product goes
+ * through exact digit products on the tensor cores.  A column's entries share one power of two over 256
+ * rows, to which they are held to 2^-56; with mx, my the largest magnitudes of two columns in a block of
+ * r <= 256 rows, C is off by at most r mx my 2^-53 per block beside the rounding of the blocks' sums.  This
+ * entry point takes digits only where each pair of columns (neither all zero in the block) has in every
+ * 256 rows at least 32 where both are within three binades of their largest, so that the error is at
+ * most 2^-41 |X|^T |Y| entry by entry, and in the mean below that of fused multiply-adds; else those
+ * run.  The same holds for lobpcg_gram_f64_df and the dense product (its diagonal is added by
+ * itself).  Inside a solve, whose columns are normalised, only the first bound is kept, unless
+ * lobpcg_options.df_products is -1. */
 LOBPCG_API lobpcg_status lobpcg_gram_f64(int64_t n, int p, const double* X, int ldx, int q, const double* Y,
                               int ldy, double* C, lobpcg_stream stream);
 
 /* C = X^T Y like lobpcg_gram_f64, formed in double-float arithmetic on the FP32 pipes (the
  * arithmetic of the FP64 refinement, see lobpcg_options.df_products): each FP64 element is
  * split into two floats, products and sums are error-compensated, sums of ~128 rows are
- * added in FP64; from n p q = 6e7 on through exact digit products on the tensor cores.  X, Y: 16-byte aligned, one even row stride (ldx == ldy).  Not in the
- * paper; the operation is Algorithm 1's Gram. */
+ * added in FP64; from n p q = 6e7 on through digit products where lobpcg_gram_f64 takes them.  X, Y: 16-byte
+ * aligned, one even row stride (ldx == ldy).  Not in the paper; the operation is Algorithm 1's Gram. */
 LOBPCG_API lobpcg_status lobpcg_gram_f64_df(int64_t n, int p, const double* X, int ldx, int q, const double* Y,
                                             int ldy, double* C, lobpcg_stream stream);
 
 /* The FP64 block update X = base + alpha [V_g] U (and AX, residual norms) in double-float
- * arithmetic, from 6e7 multiply-adds on through exact digit products on the tensor cores; arguments as lobpcg_update_f32 with FP64 blocks (V_g, AV_g, base, X, AX:
- * double, row stride ld / ld_base / ld_out in doubles). */
+ * arithmetic; arguments as lobpcg_update_f32 with FP64 blocks (V_g, AV_g, base, X, AX:
+ * double, row stride ld / ld_base / ld_out in doubles).  From 6e7 multiply-adds on (64 of them a
+ * row) through exact digit products on the tensor cores: with g_l the largest |alpha U_lj| of row l, a row's
+ * entries are held to 2^-56 of its largest |V_l| g_l.  Rows with an output whose own terms are far below
+ * that are formed with FP64 fused multiply-adds, so that every output is good to about 2^-48 of
+ * |V| |alpha U|, as in double-float; where they are more than one in eight the whole call is
+ * double-float's. */
 LOBPCG_API lobpcg_status lobpcg_update_f64_df(int64_t n, int nseg, const double* const* V, const double* const* AV,
                                               const int* w, int ld, const double* U, int q, double alpha,
                                               const double* base, int ld_base, double* X, double* AX, int ld_out,
@@ -384,13 +401,14 @@ LOBPCG_API lobpcg_status lobpcg_gram_f32_tcgen05(int64_t n, int p, const float* 
 LOBPCG_API lobpcg_status lobpcg_syev_f64(int s, const double* a, double* lam, double* U, lobpcg_stream stream);
 
 /* Same contract, two-stage method (the Rayleigh-Ritz solve of the FP32 phase of the mixed
- * form): the refinement of lobpcg_syev_f64 stopped at tol or, where that does not converge, FP32 Jacobi, one FP64 Cholesky-QR of its rotation matrix Q, then Jacobi on
- * Q^T a Q accumulated into Q until its off-diagonal mass is <= tol ||a||_F (tol = 0 means
- * 1e-15).  tol < 1e-12: FP64 rotations; eigenvalues and residuals to FP64 absolute accuracy
- * (~eps ||a||), U orthonormal to FP64 rounding.  1e-12 <= tol < 1e-6 (the solver uses
- * 1e-10): the rotations of that last stage update the small off-diagonal part in FP32
- * (diagonal and rotation product in FP64), good to about tol.  Exact zero couplings of a
- * are not kept.  EINVAL for tol outside [0, 1e-6). */
+ * form): the refinement of lobpcg_syev_f64 until the off-diagonal mass is <= tol ||a||_F (tol = 0 means
+ * 1e-15) or, where that does not converge, FP32 Jacobi, one FP64 Cholesky-QR of its rotation
+ * matrix Q, then Jacobi on Q^T a Q accumulated into Q with the same stop.  tol < 1e-12: FP64
+ * rotations; eigenvalues and residuals to FP64 absolute accuracy (~eps ||a||), U orthonormal to FP64
+ * rounding.  1e-12 <= tol < 1e-6 (the solver uses 1e-10): the rotations of that last stage update
+ * the small off-diagonal part in FP32 (diagonal and rotation product in FP64), good to about
+ * tol.  Exact zero couplings of a are not kept.  U and lam may lie in a's own memory (the Jacobi
+ * kernels run then), here and above.  EINVAL for tol outside [0, 1e-6). */
 LOBPCG_API lobpcg_status lobpcg_syev2_f64(int s, const double* a, double tol, double* lam, double* U,
                                           lobpcg_stream stream);
 

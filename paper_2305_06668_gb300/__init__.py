@@ -410,7 +410,8 @@ def gram_f32_tcgen05(X, Y, stream=None):
 
 def gram_df(X, Y, stream=None):
     """C = X^T Y of FP64 row-major CUDA blocks (one aligned row stride) in double-float
-    arithmetic or, for large blocks, exact digit products (the FP64 refinement's Gram)."""
+    arithmetic or, for large blocks without columns far apart, exact digit products (the FP64
+    refinement's Gram)."""
     torch = _torch()
     n, p = X.shape
     q = Y.shape[1]

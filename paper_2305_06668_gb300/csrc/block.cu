@@ -128,7 +128,9 @@ __global__ void __launch_bounds__(512) gram_kernel(int64_t n, Cols<T> A, Cols<T>
 // turn (g = h, h + 8, ..), then their sums in order.  One thread per element waited on memory once per
 // eight partials, 15 us for the 128 of n = 4096 and 21 us for the 304 of the largest blocks.
 __global__ void __launch_bounds__(256) reduce_kernel(const double* __restrict__ part, int nparts, int count,
-                                                     double* __restrict__ out) {
+                                                     double* __restrict__ out, const int* __restrict__ flag,
+                                                     int nparts_flag) {
+  if (flag && *flag) nparts = nparts_flag;
   __shared__ double sum[8][33];
   const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
   double s = 0.0;
@@ -646,9 +648,10 @@ int gram_partials(int64_t n, const Cols<T>& a, const Cols<T>& b, bool upper, dou
   return gram_launch<T, 8, 8, 32>(n, a, b, upper, part, max_ctas, st, run_flag);
 }
 
-void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st) {
+void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st, const int* flag,
+                     int nparts_flag) {
   if (count <= 0) return;
-  reduce_kernel<<<(count + 31) / 32, 256, 0, st>>>(part, nparts, count, out);
+  reduce_kernel<<<(count + 31) / 32, 256, 0, st>>>(part, nparts, count, out, flag, nparts_flag);
   LB_LAUNCH_CHECK();
 }
 

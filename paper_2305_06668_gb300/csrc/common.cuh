@@ -173,8 +173,10 @@ int gram_partials_umma(int64_t n, const Cols<float>& a, const Cols<float>& b, bo
 size_t gram64_scratch_ints(int64_t n);
 int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
                          int max_ctas, int* scratch, bool spread, int* err, cudaStream_t st);
-// out[e] = sum_g part[g][e] for e < count (FP64, fixed order).
-void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st);
+// out[e] = sum_g part[g][e] for e < count (FP64, fixed order), g < nparts; g < nparts_flag instead where
+// *flag (device, may be null) is not zero.
+void reduce_partials(const double* part, int nparts, int count, double* out, cudaStream_t st,
+                     const int* flag = nullptr, int nparts_flag = 0);
 
 // out_t = base_t + alpha * in_t * U for t = 0..nprod-1 (U: s x q column-major FP64 on device).
 // in_t: Cols of width s; out_t/base_t row-major (ld).  base_t may be null (then 0).
@@ -257,10 +259,11 @@ void launch_all_finite(int64_t count, const double* src, int* flag, cudaStream_t
 
 // ---- small FP64 kernels (one CTA) ----
 // Symmetric eigensolve: a (s x s, column-major; only the upper triangle is read when
-// upper_only) -> lam ascending, U column-major.  sweeps_out: device int (may be null),
-// refinement steps or FP64 sweeps.  refine: from s = 2 on the cluster solver (syev.cu); else, or where it gives up, two_stage:
-// FP32 Jacobi, Cholesky-QR of its rotations, FP64 Jacobi on Q^T a Q (faster; absolute accuracy
-// eps ||a||), else FP64 Jacobi from a, stopped when the off-diagonal mass is <= tol64 ||a||_F.
+// upper_only) -> lam ascending, U column-major.  sweeps_out: device int (may be null), refinement
+// steps or FP64 sweeps.  refine (from s = 2 on): the cluster solver (syev.cu) first.  Without it, or
+// where it gives up: two_stage, FP32 Jacobi, Cholesky-QR of its rotations, FP64 Jacobi on Q^T a Q
+// (faster; absolute accuracy eps ||a||), else FP64 Jacobi from a, stopped when the off-diagonal mass is
+// <= tol64 ||a||_F.
 void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U, int* sweeps_out,
                  cudaStream_t st, bool two_stage = false, double tol64 = 1e-15, bool refine = true);
 

@@ -5,13 +5,17 @@
 // rows takes it 7.2 ms, 50 times the time its bytes take.  34 digit products of the same Gram are
 // 0.28 TFLOP of FP16, which the tensor cores do in 0.15 ms, so what is left to pay is the cutting
 // into digits (about 25 integer instructions per element, at half the rate of FMAs), the joining of the
-// sums, and reading the blocks.  A call of that Gram went from 7,230 to 666 us (exponents 165, products
-// 450); its bytes take 150.  Clocks of the roles at 63 columns: the MMA thread issues about 40% of the
-// time and waits for tiles 35%, for the joins 25%; at 21 columns it issues 85%.
+// sums, and reading the blocks.  A call of that Gram went from 7,230 to 660 us (exponents 165, products
+// 450) and takes 750 with the test of spread below; its bytes take 150.  Counters at 200,000 rows: integer
+// pipe 47%, tensor pipe 27%, DRAM 24%.  Clocks of the roles at 63 columns: the MMA thread issues about 40%
+// of the time and waits for tiles 35%, for the joins 25%; at 21 columns it issues 85%.
 //
 // Accuracy.  Each column has its own exponent in every block of 256 rows (kGroupRows): its
 // entries are held to 2^-56 of the column's largest magnitude there, digit sums are exact, and each
-// block's sum is rounded to FP64 once and added in FP64.
+// block's sum is rounded to FP64 once and added in FP64.  So an entry of the product is off by at most
+// 256 mx my 2^-53 per block, a bound against the columns' norms.  It is not one against the entry's own
+// sum |x||y|, as an FMA chain has, where columns are large at different rows; callers that ask for that
+// one have such columns found (kSpread) and formed by the older kernels.
 //
 // Two kernels.  exp_kernel reads the blocks once and writes the exponents.  gram64_kernel is one
 // persistent CTA per SM with the roles of the FP32 Gram (umma.cu): a producer thread (1-D TMA bulk
@@ -35,9 +39,9 @@
 // each, 4.5k per chunk (1078 us a product of n = 8192), loads by the splitters a chunk ahead left 16 KB in
 // flight (899 us).  A row-major A (row_a) is copied by rows of 64 columns; it needs no transposed copy.
 //
-// A flag set by exp_kernel (a column's block with an infinity, a NaN or an exponent outside
-// 2^+-400) makes gram64_kernel return at once; the caller's general kernel, launched behind it on
-// the same flag, then forms the partials.
+// A flag raised by exp_kernel (a column's block with an infinity, a NaN or an exponent outside 2^+-400,
+// or columns too far apart) makes gram64_kernel return at once; the caller's general kernel, launched
+// behind it on the same flag, then forms the partials.
 #include <algorithm>
 #include <climits>
 
@@ -513,15 +517,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             mma(kk, 4, 0, 3, 1u);
             mma(kk, 4, 3, 1, acc);  // region 7
           } else {
-          // regions 0..6
+            // regions 0..6
 #pragma unroll
-          for (int j = 0; j < kSlices; j += W) mma(kk, 0, j, min(W, kSlices - j), acc);
-          // regions 2..6, then 7, whose first product overwrites what an earlier group left
+            for (int j = 0; j < kSlices; j += W) mma(kk, 0, j, min(W, kSlices - j), acc);
+            // regions 2..6, then 7, whose first product overwrites what an earlier group left
 #pragma unroll
-          for (int j = 0; j < 5; j += W) mma(kk, 2, j, min(W, 5 - j), 1u);
-          mma(kk, 2, 5, 1, acc);
-          mma(kk, 4, 0, 4, 1u);
-          mma(kk, 6, 0, 2, 1u);
+            for (int j = 0; j < 5; j += W) mma(kk, 2, j, min(W, 5 - j), 1u);
+            mma(kk, 2, 5, 1, acc);
+            mma(kk, 4, 0, 4, 1u);
+            mma(kk, 6, 0, 2, 1u);
           }
         }
         mma_commit(&tile_empty[buf]);
@@ -739,8 +743,8 @@ size_t gram64_scratch_ints(int64_t n) { return (size_t)ceil_div(n, kGroupRows) *
 // Gram partials through digit products; returns 0 without launching where the operands do not share
 // one 16-byte aligned row stride or need more shared memory than a CTA has.  scratch:
 // gram64_scratch_ints(n) ints; its first word is the flag: where it is not zero the partials are not
-// written, and the caller's general kernel (launched on the same flag) forms them over the same
-// number of CTAs.  spread: the flag is also raised where two columns of a group are too far apart.
+// written, and the caller's general kernel (launched on the same flag) forms them.  spread: the flag is
+// also raised where two columns of a group are too far apart.
 int gram_partials_digits(int64_t n, const Cols<double>& a, const Cols<double>& b, bool upper, double* part,
                          int max_ctas, int* scratch, bool spread, int* err, cudaStream_t st) {
   if (a.nseg == 0 || b.nseg == 0 || n <= 0) return 0;

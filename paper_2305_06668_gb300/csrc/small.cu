@@ -977,8 +977,8 @@ void launch_syev(int s, const double* a, bool upper_only, double* lam, double* U
     return true;
   }();
   (void)attr;
-  // The cluster solver from 2 columns on where the caller lets it refine (syev.cu; measured per call at s = 63, see there); this
-  // kernel then runs only where that one gave up.
+  // The cluster solver from 2 columns on where the caller lets it refine (syev.cu, with both sides'
+  // times: at 2 columns they meet); this kernel then runs only where that one gave up.
   const bool behind = s > 1 && refine;
   if (behind) launch_syev_cluster(s, a, upper_only, lam, U, sweeps_out, tol64, st);
   const double tol32 = 1e-4;  // measured: the stopping point of this stage hardly changes the total

@@ -720,7 +720,8 @@ void apply_A(lobpcg_ctx& c, const T* X, int ldx, int p, T* Y, int ldy) {
 template <class T>
 void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double* out) {
   const int pa = a.width(), pb = b.width();
-  int parts = 0;
+  int parts = 0, parts_behind = 0;
+  const int* behind = nullptr;  // flag on which the kernel behind the digits formed the partials
   if constexpr (std::is_same<T, double>::value) {
     // digit products on the tensor cores from the size where they are the faster form; a column
     // outside the digits' range raises their flag, and the FMA kernel behind them (else an empty
@@ -736,7 +737,7 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
         c.sync();
         if (*h == 2) parts = 0;
       }
-      if (parts) gram_partials<T>(c.A.n, a, b, upper, c.Gpart, parts, c.st, flag);
+      if (parts) behind = flag, parts_behind = gram_partials<T>(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st, flag);
     }
     if (!parts && c.df_on) parts = gram_partials_df(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
   } else {
@@ -746,7 +747,7 @@ void gram(lobpcg_ctx& c, const Cols<T>& a, const Cols<T>& b, bool upper, double*
       parts = gram_partials_umma(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.err_word(kErrGram32), c.st);
   }
   if (!parts) parts = gram_partials<T>(c.A.n, a, b, upper, c.Gpart, c.max_ctas, c.st);
-  reduce_partials(c.Gpart, parts, pa * pb, out, c.st);
+  reduce_partials(c.Gpart, parts, pa * pb, out, c.st, behind, parts_behind);
 }
 
 // W <- W * T (p x p FP64 matrix on device), in place.
