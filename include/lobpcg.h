@@ -326,10 +326,10 @@ LOBPCG_API lobpcg_status lobpcg_spmm_dense_rows_f64(int64_t n, const double* A, 
  * r <= 256 rows, C is off by at most r mx my 2^-53 per block beside the rounding of the blocks' sums.  This
  * entry point takes digits only where each pair of columns (neither all zero in the block) has in every
  * 256 rows at least 32 where both are within three binades of their largest, so that the error is at
- * most 2^-41 |X|^T |Y| entry by entry, and in the mean below that of fused multiply-adds; else those
- * run.  The same holds for lobpcg_gram_f64_df and the dense product (its diagonal is added by
- * itself).  Inside a solve, whose columns are normalised, only the first bound is kept, unless
- * lobpcg_options.df_products is -1. */
+ * most 2^-41 |X|^T |Y| entry by entry; else fused multiply-adds run.  The same holds for lobpcg_gram_f64_df and the dense product (its diagonal is added by
+ * itself).  Inside a solve (unless lobpcg_options.df_products is -1) and in lobpcg_ortho_f64 and
+ * lobpcg_ortho_against_f64, where errors against the columns' norms count, only the first bound is
+ * kept. */
 LOBPCG_API lobpcg_status lobpcg_gram_f64(int64_t n, int p, const double* X, int ldx, int q, const double* Y,
                               int ldy, double* C, lobpcg_stream stream);
 
